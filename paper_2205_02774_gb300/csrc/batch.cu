@@ -99,6 +99,14 @@ int index_of(const stg_batch *b, const stg_lbm *h)
     return -1;
 }
 
+// what each member's launches share the GPU with (the lengths of their runs)
+void share_gpu(stg_batch *b)
+{
+    int64_t cells = 0;
+    for (const stg_lbm *h : b->m) cells += (int64_t)h->P;
+    for (stg_lbm *h : b->m) h->in_flight = cells;
+}
+
 // the batch stream waits for whatever each member has queued on its own stream
 int order_after_members(stg_batch *b)
 {
@@ -130,8 +138,7 @@ int capture_block(stg_batch *b)
         const cudaStream_t own = h->stream;
         h->stream = b->ms[d];  // the member's steps go to its branch
         e = cudaStreamWaitEvent(h->stream, b->fork, 0);
-        for (int s = 0; s < b->B && e == cudaSuccess; ++s)
-            e = enqueue_step(h, (int)((h->t + s) & 1), is_stats_step(h, h->t + s));
+        if (e == cudaSuccess) e = enqueue_steps(h, h->t, b->B);
         if (e == cudaSuccess) e = cudaEventRecord(b->join[d], h->stream);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, b->join[d], 0);
         h->stream = own;
@@ -168,9 +175,7 @@ int capture_member(stg_batch *b, size_t d)
     h->stream = b->ms[d];
     cudaError_t e = cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        cudaError_t e1 = cudaSuccess;
-        for (int s = 0; s < b->B && e1 == cudaSuccess; ++s)
-            e1 = enqueue_step(h, (int)((h->t + s) & 1), is_stats_step(h, h->t + s));
+        const cudaError_t e1 = enqueue_steps(h, h->t, b->B);
         e = cudaStreamEndCapture(h->stream, &g);
         if (e1 != cudaSuccess) e = e1;
     }
@@ -242,6 +247,8 @@ int remove_at(stg_batch *b, int d)
     cudaEventDestroy(b->join[d]);
     if (b->mg[d]) cudaGraphExecDestroy(b->mg[d]);
     b->m.erase(b->m.begin() + d);
+    h->in_flight = 0;
+    share_gpu(b);
     b->ms.erase(b->ms.begin() + d);
     b->join.erase(b->join.begin() + d);
     b->mg.erase(b->mg.begin() + d);
@@ -318,6 +325,7 @@ int stg_batch_add(stg_batch *b, stg_lbm *h)
         return bfail(b, STG_ERR_CUDA, "cudaEventCreate");
     }
     b->m.push_back(h);
+    share_gpu(b);
     b->ms.push_back(s);
     b->join.push_back(j);
     b->mg.push_back(nullptr);

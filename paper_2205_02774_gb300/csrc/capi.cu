@@ -184,12 +184,6 @@ double vk_spectrum(double k, double le, double leta, double lcut)
     return e;
 }
 
-double wrap2pi(double v)
-{
-    v = std::fmod(v, 2.0 * kPi);
-    return v < 0.0 ? v + 2.0 * kPi : v;
-}
-
 // Inlet tables: Algorithm 1, LBM section steps 1-4.
 int build_inlet(stg_lbm *h, const stg_rans_profile *r, uint64_t seed)
 {
@@ -236,7 +230,9 @@ int build_inlet(stg_lbm *h, const stg_rans_profile *r, uint64_t seed)
     h->info.max_le = max_le;
     int N = 0;
     std::vector<double> kn, dk, phi, omg;
-    std::vector<float> sig, A, B;
+    std::vector<float> sig;
+    std::vector<double> A;
+    std::vector<float2> BS;
     if (max_le > 0.0) {
         const double kmin = kPi / max_le, kmax = 1.5 * max_kcut;
         h->info.k_min = kmin;
@@ -257,7 +253,7 @@ int build_inlet(stg_lbm *h, const stg_rans_profile *r, uint64_t seed)
         phi.resize(N);
         omg.resize(N);
         A.resize((size_t)N * ny);
-        B.resize((size_t)N * nz);
+        BS.resize((size_t)N * nz);
         for (int n = 0; n < N; ++n) {
             // eq. (dn): Phi, Theta = arccos(1 - 2 gamma), eta, phi
             const double Phi = 2.0 * kPi * u[4 * n + 0];
@@ -272,8 +268,11 @@ int build_inlet(stg_lbm *h, const stg_rans_profile *r, uint64_t seed)
             sig[3 * n + 2] = (float)(-st * ce);
             // eq. (psu) at x = 0: phase advance -2 pi d_x U_b / max l_e per step
             omg[n] = -2.0 * kPi * dx * h->info.U_b / max_le;
-            for (int j = 0; j < ny; ++j) A[(size_t)n * ny + j] = (float)wrap2pi(kn[n] * dy * (j + 0.5));
-            for (int k = 0; k < nz; ++k) B[(size_t)n * nz + k] = (float)wrap2pi(kn[n] * dz * k);
+            for (int j = 0; j < ny; ++j) A[(size_t)n * ny + j] = kn[n] * dy * (j + 0.5);
+            for (int k = 0; k < nz; ++k) {
+                const double b = kn[n] * dz * k;
+                BS[(size_t)n * nz + k] = make_float2((float)std::cos(b), (float)std::sin(b));
+            }
         }
     }
     h->N = N;
@@ -281,9 +280,9 @@ int build_inlet(stg_lbm *h, const stg_rans_profile *r, uint64_t seed)
     h->a_filter = h->p.T_filter > 0.0 ? (float)std::exp(-1.0 / h->p.T_filter) : 0.0f;
     h->info.a_filter = h->a_filter;
 
-    // mode amplitudes sqrt(6 q^n(y_j)), eq. (qn), per inlet node, FP64 on the
-    // host (terms added in mode order)
-    std::vector<float> SQ((size_t)std::max(N, 1) * ny, 0.0f);
+    // mode amplitudes sqrt(6 q^n(y_j)), eq. (qn), times (cos, sin) of the y part
+    // of the phase, per inlet node, FP64 on the host (terms added in mode order)
+    std::vector<float2> AS((size_t)std::max(N, 1) * ny, make_float2(0.f, 0.f));
     {
         std::vector<double> e(std::max(N, 1));
         for (int j = 0; j < ny; ++j) {
@@ -292,7 +291,10 @@ int build_inlet(stg_lbm *h, const stg_rans_profile *r, uint64_t seed)
                 e[n] = vk_spectrum(kn[n], le[j], leta[j], lcut[j]) * dk[n];
                 total += e[n];
             }
-            for (int n = 0; n < N; ++n) SQ[(size_t)n * ny + j] = total > 0.0 ? (float)std::sqrt(6.0 * e[n] / total) : 0.0f;
+            for (int n = 0; n < N && total > 0.0; ++n) {
+                const double q = std::sqrt(6.0 * e[n] / total), p = A[(size_t)n * ny + j];
+                AS[(size_t)n * ny + j] = make_float2((float)(q * std::cos(p)), (float)(q * std::sin(p)));
+            }
         }
     }
     // time part of the phase, phi^n + omega^n t, as Q0.64 fractions of a turn:
@@ -306,25 +308,23 @@ int build_inlet(stg_lbm *h, const stg_rans_profile *r, uint64_t seed)
 
     // device tables
     const size_t Nn = (size_t)std::max(N, 1);
-    h->A = (float *)dalloc(h, sizeof(float) * Nn * ny);
-    h->B = (float *)dalloc(h, sizeof(float) * Nn * nz);
-    h->SQ = (float *)dalloc(h, sizeof(float) * Nn * ny);
+    h->AS = (float2 *)dalloc(h, sizeof(float2) * Nn * ny);
+    h->BS = (float2 *)dalloc(h, sizeof(float2) * Nn * nz);
     h->sig = (float *)dalloc(h, sizeof(float) * 3 * Nn);
     h->phq = (unsigned long long *)dalloc(h, sizeof(unsigned long long) * Nn);
     h->omq = (unsigned long long *)dalloc(h, sizeof(unsigned long long) * Nn);
     h->a6 = (float *)dalloc(h, sizeof(float) * 6 * ny);
     h->u_int = (float *)dalloc(h, sizeof(float) * ny);
     double *dR6 = (double *)dalloc(h, sizeof(double) * 6 * ny);
-    if (!h->A || !h->B || !h->SQ || !h->sig || !h->phq || !h->omq || !h->a6 || !h->u_int || !dR6)
+    if (!h->AS || !h->BS || !h->sig || !h->phq || !h->omq || !h->a6 || !h->u_int || !dR6)
         return fail(h, STG_ERR_NOMEM, "device allocation of the inlet tables failed");
     std::vector<float> uf(ny);
     for (int j = 0; j < ny; ++j) uf[j] = (float)u_int[j];
     CK(cudaMemcpy(h->u_int, uf.data(), sizeof(float) * ny, cudaMemcpyHostToDevice));
     CK(cudaMemcpy(dR6, R6.data(), sizeof(double) * 6 * ny, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(h->SQ, SQ.data(), sizeof(float) * SQ.size(), cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(h->AS, AS.data(), sizeof(float2) * AS.size(), cudaMemcpyHostToDevice));
     if (N > 0) {
-        CK(cudaMemcpy(h->A, A.data(), sizeof(float) * A.size(), cudaMemcpyHostToDevice));
-        CK(cudaMemcpy(h->B, B.data(), sizeof(float) * B.size(), cudaMemcpyHostToDevice));
+        CK(cudaMemcpy(h->BS, BS.data(), sizeof(float2) * BS.size(), cudaMemcpyHostToDevice));
         CK(cudaMemcpy(h->sig, sig.data(), sizeof(float) * sig.size(), cudaMemcpyHostToDevice));
         CK(cudaMemcpy(h->phq, phq.data(), sizeof(unsigned long long) * N, cudaMemcpyHostToDevice));
         CK(cudaMemcpy(h->omq, omq.data(), sizeof(unsigned long long) * N, cudaMemcpyHostToDevice));
@@ -335,10 +335,27 @@ int build_inlet(stg_lbm *h, const stg_rans_profile *r, uint64_t seed)
     return STG_OK;
 }
 
-// inlet plane of the step with this parity
-float *ubc_plane(const stg_lbm *h, int parity)
+// blocks of a step pass at most, their mass slots (one each and one per group) and counters
+size_t mass_slots(int nx, int ny, int nz)
 {
-    return h->ubc + (size_t)(parity & 1) * 3 * (size_t)h->d.ny * h->d.nz;
+    const int n = stg::step_grid_blocks(nx, ny, nz);
+    return (size_t)n + stg::mass_groups(n);
+}
+size_t mass_counters(int nx, int ny, int nz) { return (size_t)stg::mass_groups(stg::step_grid_blocks(nx, ny, nz)) + 1; }
+
+// runs of z planes whose statistics a sampling step leaves in stat_part
+int stat_runs(int nx, int ny, int nz)
+{
+    const int g = stg::stat_group(nx, ny, nz);
+    return (nz + g - 1) / g;
+}
+
+size_t plane_floats(const stg_lbm *h) { return 3 * (size_t)h->d.ny * h->d.nz; }
+
+// inlet plane of step t
+float *ubc_plane(const stg_lbm *h, int64_t t)
+{
+    return h->ubc + (size_t)(t & (stg::INLET_RING - 1)) * plane_floats(h);
 }
 
 // where the populations of the current state live (for probes and block reads)
@@ -374,6 +391,7 @@ stg::StepArgs step_args(const stg_lbm *h, int parity)
     a.ny = h->d.ny;
     a.nz = h->d.nz;
     a.P = (unsigned)h->P;
+    a.in_flight = std::max<int64_t>(h->in_flight, (int64_t)h->P);
     a.bc_x = h->d.bc_x;
     a.bc_y = h->d.bc_y;
     a.tau0 = (float)h->d.tau0;
@@ -382,16 +400,16 @@ stg::StepArgs step_args(const stg_lbm *h, int parity)
     a.Fy = (float)h->d.force[1];
     a.Fz = (float)h->d.force[2];
     a.has_force = (h->d.force[0] != 0.0 || h->d.force[1] != 0.0 || h->d.force[2] != 0.0);
-    a.ubc = ubc_plane(h, parity);
+    a.ubc = h->ubc;
     a.spf = h->spf;
     a.ctl = h->ctl;
     a.parity = parity;
     a.stats_every = h->d.stats_every;
     a.interior = h->interior;
     a.aa = h->aa ? 1 : 0;
-    a.tile_layout = h->tile.interior_layout;
     a.tile_zc = h->tile.interior_zc;
     a.tile_wall_zc = h->tile.wall_zc;
+    a.stat_group = stg::stat_group(h->d.nx, h->d.ny, h->d.nz);
     a.check_every = h->d.check_every;
     a.stat_mean = h->stat_mean;
     a.stat_rey = h->stat_rey;
@@ -408,9 +426,8 @@ stg::InletArgs inlet_args(const stg_lbm *h, int parity)
     a.ny = h->d.ny;
     a.nz = h->d.nz;
     a.N = h->N;
-    a.A = h->A;
-    a.B = h->B;
-    a.SQ = h->SQ;
+    a.AS = h->AS;
+    a.BS = h->BS;
     a.sig = h->sig;
     a.phq = h->phq;
     a.omq = h->omq;
@@ -418,8 +435,9 @@ stg::InletArgs inlet_args(const stg_lbm *h, int parity)
     a.u_int = h->u_int;
     a.a_filter = h->a_filter;
     a.uf = h->uf;
-    a.ubc = ubc_plane(h, parity ^ 1);  // the plane of the next step
-    a.ahead = 1;
+    a.ubc = h->ubc;
+    a.ahead = 1;  // the plane of the next step
+    a.planes = 1;
     a.ctl = h->ctl;
     a.parity = parity;
     return a;
@@ -447,12 +465,42 @@ namespace {
 namespace stg {
 namespace host {
 
-cudaError_t enqueue_step(stg_lbm *h, int parity, bool stats)
+// The inlet planes are computed beside the passes on a branch of their own, a few
+// for the next steps first (they are due when the first pass ends) and the rest of
+// the block, INLET_MAX_PLANES at a time, beside the passes that read those.  One
+// launch per step instead took 10 to 19 us each on lattices whose pass takes 4 to
+// 60, ahead of the pass or of its wall rows.
+cudaError_t enqueue_steps(stg_lbm *h, int64_t t, int n)
 {
-    const stg::InletArgs in = inlet_args(h, parity);
-    return stg::launch_step(step_args(h, parity), h->d.storage, h->d.collision, stats, h->stream, h->side,
-                            h->ev_fork, h->ev_join,
-                            h->inout ? &in : nullptr);
+    constexpr int FIRST = 4;
+    cudaError_t e = cudaSuccess;
+    int asked = 0;  // planes launched: those of the steps t + 1 .. t + asked
+    int due = 0;    // the first step whose plane has not been waited for
+    auto ask = [&](int k) {
+        k = std::min(k, n - asked);
+        stg::InletArgs in = inlet_args(h, (int)(t & 1));
+        in.from_block = asked > 0;
+        in.ahead = 1 + asked;
+        in.planes = k;
+        e = cudaEventRecord(h->ev_ifork, h->stream);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(h->inlet_side, h->ev_ifork, 0);
+        if (e == cudaSuccess) e = stg::launch_inlet(in, h->inlet_side);
+        if (e == cudaSuccess) e = cudaEventRecord(h->ev_ijoin, h->inlet_side);
+        asked += k;
+    };
+    for (int s = 0; s < n && e == cudaSuccess; ++s) {
+        if (h->inout && s == due) {
+            if (s > 0) e = cudaStreamWaitEvent(h->stream, h->ev_ijoin, 0);
+            due = asked + 1;
+            // the ring holds the planes that the coming passes read and as many again
+            if (e == cudaSuccess && asked < n) ask(s == 0 ? FIRST : stg::INLET_MAX_PLANES);
+        }
+        if (e == cudaSuccess)
+            e = stg::launch_step(step_args(h, (int)((t + s) & 1)), h->d.storage, h->d.collision, is_stats_step(h, t + s),
+                                 h->stream, h->side, h->ev_fork, h->ev_join);
+    }
+    if (e == cudaSuccess && h->inout && n > 0) e = cudaStreamWaitEvent(h->stream, h->ev_ijoin, 0);
+    return e;
 }
 
 }  // namespace host
@@ -460,21 +508,18 @@ cudaError_t enqueue_step(stg_lbm *h, int parity, bool stats)
 
 namespace {
 
-// Graph of `steps` steps starting with parity p0.  single_stats >= 0: one
-// step with that sampling flag; otherwise step s samples when (s + 1) is a
-// multiple of the sampling period (a block that starts at an aligned index).
-int capture(stg_lbm *h, int p0, int steps, int single_stats, cudaGraphExec_t *out)
+// Graph of `steps` steps from step index t0 on (of which only the parity and
+// the place in the sampling period matter).
+int capture(stg_lbm *h, int64_t t0, int steps, cudaGraphExec_t *out)
 {
     cudaGraph_t g = nullptr;
     CK(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-    cudaError_t e = cudaSuccess;
-    for (int s = 0; s < steps && e == cudaSuccess; ++s) {
-        const bool st = single_stats >= 0 ? single_stats != 0
-                                          : (h->d.stats_every > 0 && (s + 1) % h->d.stats_every == 0);
-        e = enqueue_step(h, (p0 + s) & 1, st);
-    }
+    cudaError_t e = enqueue_steps(h, t0, steps);
     cudaError_t e2 = cudaStreamEndCapture(h->stream, &g);
-    if (e != cudaSuccess) return cuda_fail(h, e, "kernel launch during capture");
+    if (e != cudaSuccess) {
+        if (g) cudaGraphDestroy(g);
+        return cuda_fail(h, e, "kernel launch during capture");
+    }
     if (e2 != cudaSuccess) return cuda_fail(h, e2, "cudaStreamEndCapture");
     e = cudaGraphInstantiate(out, g, cudaGraphInstantiateFlagUseNodePriority);
     cudaGraphDestroy(g);
@@ -502,11 +547,18 @@ int capture_all(stg_lbm *h)
 {
     destroy_graphs(h);
     int rc = STG_OK;
-    for (int p = 0; p < 2 && rc == STG_OK; ++p) {
-        rc = capture(h, p, 1, 0, &h->g_single[p][0]);
-        if (rc == STG_OK && h->d.stats_every > 0) rc = capture(h, p, 1, 1, &h->g_single[p][1]);
-        if (rc == STG_OK && h->block_steps > 0) rc = capture(h, p, h->block_steps, -1, &h->g_block[p]);
+    const int64_t shared = h->in_flight;
+    h->in_flight = 0;  // these graphs run the lattice alone
+    // one full cycle of step indices: parities and sampling flags that never meet
+    // (with an even sampling period, half of them) need no graph
+    const int k = std::max(h->d.stats_every, 1);
+    for (int64_t t = 0; t < 2 * (int64_t)k && rc == STG_OK; ++t) {
+        cudaGraphExec_t &g = h->g_single[t & 1][is_stats_step(h, t) ? 1 : 0];
+        if (!g) rc = capture(h, t, 1, &g);
+        if (rc == STG_OK && h->block_steps > 0 && t % k == 0 && !h->g_block[t & 1])
+            rc = capture(h, t, h->block_steps, &h->g_block[t & 1]);
     }
+    h->in_flight = shared;
     return rc;
 }
 
@@ -669,7 +721,6 @@ int reset_counters(stg_lbm *h, int64_t step)
     if (h->inout) {
         // the inlet plane of the restart step (later planes are computed one step ahead)
         stg::InletArgs in = inlet_args(h, (int)(step & 1));
-        in.ubc = ubc_plane(h, (int)(step & 1));
         in.ahead = 0;
         CK(stg::launch_inlet(in, h->stream));
     }
@@ -697,6 +748,9 @@ void release(stg_lbm *h)
     if (h->ev_fork) cudaEventDestroy(h->ev_fork);
     if (h->ev_join) cudaEventDestroy(h->ev_join);
     if (h->side) cudaStreamDestroy(h->side);
+    if (h->inlet_side) cudaStreamDestroy(h->inlet_side);
+    if (h->ev_ifork) cudaEventDestroy(h->ev_ifork);
+    if (h->ev_ijoin) cudaEventDestroy(h->ev_ijoin);
     if (h->ev_done) cudaEventDestroy(h->ev_done);
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
     delete h;
@@ -790,12 +844,15 @@ int stg_lbm_create(const stg_domain *domain, const stg_rans_profile *rans, const
         }
         h->own_stream = true;
     }
-    int lo_prio = 0, hi_prio = 0;  // the branch (wall rows, inlet plane) gets the highest priority: its blocks start first
+    int lo_prio = 0, hi_prio = 0;  // the branches (wall rows, inlet planes) get the highest priority: its blocks start first
     if (cudaEventCreateWithFlags(&h->ev_check, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming) != cudaSuccess ||
         cudaDeviceGetStreamPriorityRange(&lo_prio, &hi_prio) != cudaSuccess ||
         cudaStreamCreateWithPriority(&h->side, cudaStreamNonBlocking, hi_prio) != cudaSuccess ||
+        cudaStreamCreateWithPriority(&h->inlet_side, cudaStreamNonBlocking, hi_prio) != cudaSuccess ||
+        cudaEventCreateWithFlags(&h->ev_ifork, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&h->ev_ijoin, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&h->ev_done, cudaEventDisableTiming) != cudaSuccess ||
         !(h->h_pinned = pinned_slots().get())) {
         h->err = "event / pinned allocation failed";
@@ -811,20 +868,20 @@ int stg_lbm_create(const stg_domain *domain, const stg_rans_profile *rans, const
     h->aa = domain->streaming == STG_STREAM_AA;
     h->lat[0] = dalloc(h, 19 * h->P * h->elem);
     h->lat[1] = h->aa ? h->lat[0] : dalloc(h, 19 * h->P * h->elem);  // in place: one lattice
-    h->ubc = (float *)dalloc(h, sizeof(float) * 6 * (size_t)ny * nz);
+    h->ubc = (float *)dalloc(h, sizeof(float) * stg::INLET_RING * plane_floats(h));
     h->uf = (float *)dalloc(h, sizeof(float) * 3 * (size_t)ny * nz);
     h->ctl = (StepCtl *)dalloc(h, sizeof(StepCtl));
     h->stat_mean = (double *)dalloc(h, sizeof(double) * 3 * (size_t)nx * ny);
     h->stat_rey = (double *)dalloc(h, sizeof(double) * 6 * (size_t)nx * ny);
-    h->mass_partial = (double *)dalloc(h, sizeof(double) * stg::step_grid_blocks(nx, ny, nz));
+    h->mass_partial = (double *)dalloc(h, sizeof(double) * mass_slots(nx, ny, nz));
     if (domain->stats_every > 0) {
-        h->stat_part = (float *)dalloc(h, sizeof(float) * 9 * (size_t)nx * ny * ((nz + stg::STAT_GROUP - 1) / stg::STAT_GROUP));
+        h->stat_part = (float *)dalloc(h, sizeof(float) * 9 * (size_t)nx * ny * stat_runs(nx, ny, nz));
         if (!h->stat_part) {
             h->err = "device allocation failed";
             return bail(STG_ERR_NOMEM);
         }
     }
-    h->mass_counter = (unsigned *)dalloc(h, sizeof(unsigned) * 4);
+    h->mass_counter = (unsigned *)dalloc(h, sizeof(unsigned) * mass_counters(nx, ny, nz));
     h->mass_out = (double *)dalloc(h, sizeof(double) * 2);
     h->m_partial = (double *)dalloc(h, sizeof(double) * stg::mass_grid_blocks());
     h->m_counter = (unsigned *)dalloc(h, sizeof(unsigned) * 4);
@@ -849,10 +906,10 @@ int stg_lbm_create(const stg_domain *domain, const stg_rans_profile *rans, const
         return bail(STG_ERR_NOMEM);
     }
     cudaError_t e = cudaSuccess;
-    e = cudaMemsetAsync(h->mass_counter, 0, sizeof(unsigned) * 4, h->stream);
+    e = cudaMemsetAsync(h->mass_counter, 0, sizeof(unsigned) * mass_counters(nx, ny, nz), h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->m_counter, 0, sizeof(unsigned) * 4, h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->mass_out, 0, sizeof(double) * 2, h->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->ubc, 0, sizeof(float) * 6 * (size_t)ny * nz, h->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(h->ubc, 0, sizeof(float) * stg::INLET_RING * plane_floats(h), h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->uf, 0, sizeof(float) * 3 * (size_t)ny * nz, h->stream);
     if (e != cudaSuccess) {
         cuda_fail(h, e, "cudaMemsetAsync");
@@ -892,17 +949,17 @@ int stg_lbm_estimate_bytes(const stg_domain *d, const stg_params *p, int64_t *by
     const double nx = d->nx, ny = d->ny, nz = d->nz, P = nx * ny * nz;
     const double elem = d->storage == STG_FP32 ? 4.0 : 2.0;
     const double lattices = d->streaming == STG_STREAM_AA ? 1.0 : 2.0;
-    double b = lattices * r(19 * P * elem) + r(24 * ny * nz) + r(12 * ny * nz) + r(sizeof(StepCtl)) + r(24 * nx * ny) + r(48 * nx * ny) +
-               r(8.0 * stg::step_grid_blocks(d->nx, d->ny, d->nz)) + 2 * r(16) + 2 * r(16) +
+    double b = lattices * r(19 * P * elem) + r(12.0 * stg::INLET_RING * ny * nz) + r(12 * ny * nz) + r(sizeof(StepCtl)) + r(24 * nx * ny) + r(48 * nx * ny) +
+               r(8.0 * mass_slots(d->nx, d->ny, d->nz)) + r(4.0 * mass_counters(d->nx, d->ny, d->nz)) + 3 * r(16) +
                r(8.0 * stg::mass_grid_blocks());
     if (d->sponge_len > 0.0) b += r(4 * nx);
-    if (d->stats_every > 0) b += r(36.0 * nx * ny * std::ceil(nz / (double)stg::STAT_GROUP));
+    if (d->stats_every > 0) b += r(36.0 * nx * ny * stat_runs(d->nx, d->ny, d->nz));
     if (d->bc_x == STG_BC_X_INLET_OUTLET) {
         double N = 1.0;
         if (p && p->n_modes > 0) N = p->n_modes;
         else if (p && p->alpha > 0.0) N = std::ceil(std::log(1.5 * std::max(ny, 2.0)) / std::log(1.0 + p->alpha) + 1.0);
-        // A, B, SQ, sigma, the two phase words, a6, u_int, the FP64 stresses
-        b += r(4 * N * ny) + r(4 * N * nz) + r(4 * N * ny) + r(12 * N) + 2 * r(8 * N) + r(24 * ny) + r(4 * ny) +
+        // AS, BS, sigma, the two phase words, a6, u_int, the FP64 stresses
+        b += r(8 * N * ny) + r(8 * N * nz) + r(12 * N) + 2 * r(8 * N) + r(24 * ny) + r(4 * ny) +
              r(48 * ny);
     }
     *bytes = (int64_t)b;
@@ -1132,7 +1189,7 @@ int stg_lbm_save(stg_lbm *h, void *host, size_t bytes)
     p += hd.pop_bytes;
     CK(cudaMemcpy(p, h->uf, hd.uf_bytes, cudaMemcpyDeviceToHost));
     p += hd.uf_bytes;
-    CK(cudaMemcpy(p, ubc_plane(h, (int)(h->t & 1)), hd.plane_bytes, cudaMemcpyDeviceToHost));  // this step's inlet plane
+    CK(cudaMemcpy(p, ubc_plane(h, h->t), hd.plane_bytes, cudaMemcpyDeviceToHost));  // this step's inlet plane
     p += hd.plane_bytes;
     const size_t m = (size_t)h->d.nx * h->d.ny;
     CK(cudaMemcpy(p, h->stat_mean, sizeof(double) * 3 * m, cudaMemcpyDeviceToHost));
@@ -1161,7 +1218,7 @@ int stg_lbm_load(stg_lbm *h, const void *host, size_t bytes)
     p += hd.pop_bytes;
     CK(cudaMemcpy(h->uf, p, hd.uf_bytes, cudaMemcpyHostToDevice));
     p += hd.uf_bytes;
-    CK(cudaMemcpy(ubc_plane(h, (int)(hd.t & 1)), p, hd.plane_bytes, cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(ubc_plane(h, hd.t), p, hd.plane_bytes, cudaMemcpyHostToDevice));
     p += hd.plane_bytes;
     const size_t m = (size_t)h->d.nx * h->d.ny;
     CK(cudaMemcpy(h->stat_mean, p, sizeof(double) * 3 * m, cudaMemcpyHostToDevice));
@@ -1218,7 +1275,7 @@ int stg_lbm_get_inlet(stg_lbm *h, float *host_u)
     int rc = wait_stream(h);
     if (rc) return rc;
     // the plane of the last completed step
-    CK(cudaMemcpy(host_u, ubc_plane(h, (int)((h->t + 1) & 1)), sizeof(float) * 3 * (size_t)h->d.ny * h->d.nz,
+    CK(cudaMemcpy(host_u, ubc_plane(h, h->t - 1), sizeof(float) * 3 * (size_t)h->d.ny * h->d.nz,
                   cudaMemcpyDeviceToHost));
     return STG_OK;
 }
@@ -1227,7 +1284,7 @@ int stg_lbm_device_state(stg_lbm *h, void **pops, float **inlet_u)
 {
     if (!h) return fail(nullptr, STG_ERR_INVALID, "handle is NULL");
     if (pops) *pops = h->lat[h->t & 1];
-    if (inlet_u) *inlet_u = ubc_plane(h, (int)((h->t + 1) & 1));
+    if (inlet_u) *inlet_u = ubc_plane(h, h->t - 1);
     return STG_OK;
 }
 
@@ -1359,8 +1416,8 @@ int apply_tile(stg_lbm *h, const stg_tile &tile)
 
 const stg_tile *tile_candidates(int *n)
 {
-    static const stg_tile cand[] = {{1, 4, 24, 0},  {1, 6, 24, 0},  {1, 8, 24, 0},  {1, 12, 24, 0}, {1, 16, 24, 0},
-                                    {1, 8, 8, 0},   {0, 16, 24, 0}, {0, 24, 24, 0}, {0, 48, 24, 0}, {0, 0, 0, 0}};
+    // (the launches take runs of at most 8 planes by themselves)
+    static const stg_tile cand[] = {{1, 4, 24, 0}, {1, 6, 24, 0}, {1, 8, 24, 0}};
     *n = (int)(sizeof cand / sizeof cand[0]);
     return cand;
 }

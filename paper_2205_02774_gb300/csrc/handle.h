@@ -28,13 +28,14 @@ struct stg_lbm {
     std::vector<std::pair<void *, size_t>> allocs;
     size_t P = 0, elem = 4;
     void *lat[2] = {nullptr, nullptr};
-    float *ubc = nullptr, *uf = nullptr;  // ubc: inlet planes of steps t and t + 1, [2][3][nz][ny] by step parity
+    float *ubc = nullptr, *uf = nullptr;  // ubc: inlet planes [INLET_RING][3][nz][ny], step t in plane t mod INLET_RING
     float *spf = nullptr;  // sponge factor per column (nullptr: no sponge)
     int n_probes = 0;                     // velocity probes (stg_lbm_set_probes)
     int *probe_xyz = nullptr;             // device [3 n_probes]
     float *probe_buf = nullptr;           // device samples of one step_probed call
     size_t probe_cap = 0;                 // floats in probe_buf
-    float *A = nullptr, *B = nullptr, *SQ = nullptr, *sig = nullptr, *a6 = nullptr, *u_int = nullptr;
+    float2 *AS = nullptr, *BS = nullptr;
+    float *sig = nullptr, *a6 = nullptr, *u_int = nullptr;
     unsigned long long *phq = nullptr, *omq = nullptr;  // phi^n and omega^n as Q0.64 fractions of a turn
     int N = 0;
     float a_filter = 0.f;
@@ -47,8 +48,10 @@ struct stg_lbm {
     unsigned *m_counter = nullptr;
     double *h_pinned = nullptr;  // [0]: last checked mass
     cudaEvent_t ev_check = nullptr, ev_done = nullptr;
-    cudaStream_t side = nullptr;                       // branch for the edge kernel
+    cudaStream_t side = nullptr;                       // branch for the wall rows / edge kernel
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+    cudaStream_t inlet_side = nullptr;                 // branch for the inlet planes
+    cudaEvent_t ev_ifork = nullptr, ev_ijoin = nullptr;
     bool check_pending = false;
     int64_t t = 0, t0_stats = 0;
     double mass0 = 0.0;
@@ -63,6 +66,7 @@ struct stg_lbm {
     double timeout_s = 900.0;
     int interior = 0;  // STG_LBM_INTERIOR=scalar|pair overrides the interior kernel choice
     stg_tile tile{1, 8, 24, 0};
+    int64_t in_flight = 0;  // cells advanced together with this lattice's (a batch's total); 0: its own alone
     stg_batch *batch = nullptr;  // the batch this lattice belongs to (its steps run there)
 };
 
@@ -80,9 +84,10 @@ struct Range {
 
 int fail(stg_lbm *h, int code, const std::string &msg);
 int cuda_fail(stg_lbm *h, cudaError_t e, const char *what);
-// one step of h with the given parity on h->stream (and h->side); `stats`
-// selects the sampling-step kernels
-cudaError_t enqueue_step(stg_lbm *h, int parity, bool stats);
+// the n steps of h from step index t on (their inlet planes included) on
+// h->stream and h->side; of t only the parity and the place in the sampling
+// period matter
+cudaError_t enqueue_steps(stg_lbm *h, int64_t t, int n);
 bool is_stats_step(const stg_lbm *h, int64_t t);
 // evaluate the last completed mass check (non-blocking)
 int poll_check(stg_lbm *h);

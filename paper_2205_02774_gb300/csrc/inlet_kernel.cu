@@ -7,145 +7,184 @@
 //   u'  = a(j) v'                                                           eqs. (v_fluc), (cholesky)
 //   u_f = a u_f + (1 - a) u'   (first-order temporal filter; u_f = u' at the first step)
 //   u_bc = u_int(j) e_x + u_f                                               eqs. (u_phys), (u_transfer)
-// The phase is split into three parts each already reduced to [0, 2 pi):
-// the y part and the z part (tables built in FP64 on the host) and the time
-// part phi^n + omega^n t, kept as Q0.64 fractions of a turn and advanced by
-// wrapping 64-bit integer arithmetic (a phase accumulator: exact modulo a
-// turn for any step count, no floating point); their FP32 sum is below 6 pi
-// and is reduced to [-pi, pi] before the cosine.
+// By the addition theorem the cosine of the whole phase splits into factors of
+// one variable each,
+//   sqrt(6 q^n(j)) cos(A^n_j + B^n_k + th^n(t)) = ca cb' - sa sb',
+//   (ca, sa) = sqrt(6 q^n(j)) (cos, sin) A^n_j   A: y part, k^n d^n_y y_j
+//   (cb', sb') = (cos, sin)(B^n_k + th^n(t)), from the tables (cos, sin) B^n_k
+//                (z part) and (cos, sin) th^n(t) of the time phase,
+// so a mode term is two multiply-adds and three more into v' instead of a range
+// reduction and a cosine.  The static tables are built in FP64 on the host; the
+// time phase phi^n + omega^n t is a Q0.64 fraction of a turn advanced by
+// wrapping 64-bit integer arithmetic (exact modulo a turn for any step count).
 //
-// Work split: a block covers 32 consecutive j (one per lane) by 8 span nodes
-// k; its 8 warps are 4 pairs of span nodes times 2 halves of the mode sum
-// (modes of even and odd index within a chunk).  Everything a mode term
-// needs is staged in shared memory per chunk of INLET_CHUNK modes by
-// coalesced loads of the whole block (any mode count fits the fixed
-// footprint): the time phase and sigma^n, the block's 8 z parts, and its 32
-// y parts and amplitudes sqrt(6 q^n(j)).  A thread reads the y part and the
-// amplitude of a mode once and uses them for its two span nodes, so a mode
-// term costs a few shared-memory reads, the phase sum and its reduction, one
-// cosine and four multiply-adds; the two halves of the mode sum are added in
-// a fixed order at the end.
-// The plane of step t + 1 is computed during step t (ahead = 1), beside the
-// step pass that reads the plane of step t; the first plane after a reset is
-// computed with ahead = 0.
+// One launch computes the planes of `planes` consecutive steps (a block of steps
+// asks for them a few and then 16 at a time, beside its passes, instead of one
+// launch in every step).  A block of 8 warps covers 32 consecutive j (one per
+// lane) and ITEMS = 8 IPW pairs (span node, step), IPW per warp in registers:
+// IPW = 4 for more than 8 planes, 1 up to that, where the latency of the launch
+// counts.  Per chunk of modes the block stages the y factors, the time factors and
+// the items' (cb', sb') in shared memory; a mode then costs a warp 2 + IPW
+// shared-memory reads and 6 IPW multiplies and multiply-adds, and issuing those
+// bounds the kernel.  The sum over the modes is in mode order in every form, and
+// every multiply-add is written out, so a plane's bits do not depend on how many
+// were asked for.  The filter then runs over the steps in order, one thread per node.
 #include "internal.h"
 
 namespace stg {
 
 constexpr int INLET_J = 32;      // wall-normal nodes per block (one per lane)
-constexpr int INLET_KPT = 2;     // span nodes per thread
-constexpr int INLET_KG = 4;      // span-node pairs per block
-constexpr int INLET_H = 2;       // halves of the mode sum
-constexpr int INLET_WARPS = INLET_KG * INLET_H;
-constexpr int INLET_K = INLET_KPT * INLET_KG;  // span nodes per block
-constexpr int INLET_CHUNK = 128; // modes staged per pass through shared memory
+constexpr int INLET_WARPS = 8;
 
-// At least 4 blocks per SM caps the kernel at 64 registers, which it fits without
-// spilling; left to itself ptxas aims at the 5 blocks the shared memory allows and
-// spills to a stack frame, and with local memory the kernel no longer ran beside
-// the interior pass (0.75 ms more per step on 1536x256x384 in FP32).
-__global__ void __launch_bounds__(INLET_J * INLET_WARPS, 4) stg_inlet_kernel(const InletArgs a)
+template <int IPW>
+__global__ void __launch_bounds__(INLET_J * INLET_WARPS, 2) stg_inlet_kernel(const InletArgs a, int kb)
 {
-    __shared__ float4 ts[INLET_CHUNK];           // (time phase, sigma_x, sigma_y, sigma_z) per mode
-    __shared__ float2 bz[INLET_CHUNK][INLET_KG]; // z parts of the block's span nodes per mode
-    __shared__ float ay_s[INLET_CHUNK][INLET_J]; // y parts of the block's wall-normal nodes per mode
-    __shared__ float sq_s[INLET_CHUNK][INLET_J]; // amplitudes sqrt(6 q^n(j)) per mode
-    __shared__ float part[INLET_KG][INLET_KPT][3][INLET_J];  // second half of the mode sum
+    constexpr int ITEMS = IPW * INLET_WARPS;
+    constexpr int CHUNK = IPW == 1 ? 96 : 32;              // modes staged per pass through shared memory
+    constexpr int STEPS = IPW == 1 ? ITEMS : INLET_MAX_PLANES;
+    constexpr int NT = INLET_J * INLET_WARPS;
+    __shared__ float2 ys[CHUNK][INLET_J];                  // (ca, sa) per mode and wall-normal node
+    __shared__ float2 ts[CHUNK][STEPS];                    // (cos, sin) of the time phase per mode and step
+    __shared__ float2 is[CHUNK][ITEMS];                    // (cb', sb') per mode and item
+    __shared__ float4 sg[CHUNK];                           // sigma^n
+    __shared__ float vs[ITEMS][3][INLET_J];                // v' per item and node
     const int lane = threadIdx.x, w = threadIdx.y;
-    const int g = w % INLET_KG, h = w / INLET_KG;
     const int tid = w * INLET_J + lane;
-    const int ny = a.ny, nz = a.nz, N = a.N;
+    const int ny = a.ny, nz = a.nz, N = a.N, T = a.planes;
     const int j0 = blockIdx.x * INLET_J;
-    const int j = j0 + lane;
-    const int k0 = blockIdx.y * INLET_K;
-    const bool jl = j < ny;
-    const long long t = a.ctl->t[a.parity] + a.ahead;
-    const bool first = (t == a.ctl->t0_filter);
-    float v[INLET_KPT][3];
+    const int k0 = blockIdx.y * kb;   // the block's span nodes k0 .. k0 + kb - 1; item q = (k0 + q / T, step q % T)
+    const int items = kb * T;         // <= ITEMS
+    const float af = a.a_filter, bf = 1.0f - a.a_filter;
+    const size_t plane = (size_t)ny * nz;
+    float v[IPW][3];
 #pragma unroll
-    for (int q = 0; q < INLET_KPT; ++q) v[q][0] = v[q][1] = v[q][2] = 0.f;
-    for (int n0 = 0; n0 < N; n0 += INLET_CHUNK) {
-        const int cn = min(INLET_CHUNK, N - n0);
+    for (int q = 0; q < IPW; ++q) v[q][0] = v[q][1] = v[q][2] = 0.f;
+    // The table reads of a chunk are issued together, a chunk ahead of their use:
+    // their latency is most of what a chunk costs a launch of few blocks.
+    constexpr int NB = CHUNK * ITEMS / NT, NY = CHUNK * INLET_J / NT, NS = (CHUNK * STEPS + NT - 1) / NT;
+    float2 b[NB], y[NY];
+    unsigned long long ph[NS], om[NS];
+    float4 sgr;
+    auto fetch = [&](int n0) {
+        const int cn = min(CHUNK, N - n0);
+#pragma unroll
+        for (int i = 0; i < NS; ++i) {
+            const int m = (tid + i * NT) / T;
+            if (m < cn) ph[i] = a.phq[n0 + m], om[i] = a.omq[n0 + m];
+        }
+#pragma unroll
+        for (int i = 0; i < NB; ++i) {
+            const int e = tid + i * NT, m = e / ITEMS, q = e % ITEMS;
+            if (m < cn && q < items) b[i] = a.BS[(size_t)(n0 + m) * nz + min(k0 + q / T, nz - 1)];  // nodes past nz are not stored
+        }
+#pragma unroll
+        for (int i = 0; i < NY; ++i) {
+            const int m = w + i * INLET_WARPS;
+            if (m < cn) y[i] = a.AS[(size_t)(n0 + m) * ny + min(j0 + lane, ny - 1)];  // nor are rows past ny
+        }
+        if (tid < cn) sgr = make_float4(a.sig[3 * (n0 + tid)], a.sig[3 * (n0 + tid) + 1], a.sig[3 * (n0 + tid) + 2], 0.f);
+    };
+    // the filter state and tables of the thread's first node, early as well
+    float L[6], ui = 0.f, f[3];
+    auto fetch_node = [&](int e) {
+        const int j = j0 + e % INLET_J, k = k0 + e / INLET_J;
+        if (e >= kb * INLET_J || j >= ny || k >= nz) return false;
+#pragma unroll
+        for (int c = 0; c < 6; ++c) L[c] = a.a6[6 * j + c];
+        ui = a.u_int[j];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) f[c] = a.uf[c * plane + (size_t)k * ny + j];
+        return true;
+    };
+    fetch(0);
+    // step of the first plane: a later launch of a block of steps, beside which the
+    // step counter moves on, counts from the block's first one
+    const long long t = (a.from_block ? a.ctl->t_block : a.ctl->t[a.parity]) + a.ahead;
+    if (!a.from_block && blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) a.ctl->t_block = t - a.ahead;
+    const long long t0f = a.ctl->t0_filter;
+    bool mine = fetch_node(tid);
+    for (int n0 = 0; n0 < N; n0 += CHUNK) {
+        const int cn = min(CHUNK, N - n0);
         __syncthreads();  // the previous chunk is consumed
-        for (int m = tid; m < cn; m += INLET_J * INLET_WARPS) {
-            const int n = n0 + m;
-            // time part of the phase in turns: phi^n + omega^n t modulo one turn
-            const unsigned long long q = a.phq[n] + a.omq[n] * (unsigned long long)t;
-            const float th = (float)(unsigned)(q >> 32) * 1.4629180792671596e-09f;  // 2 pi / 2^32
-            ts[m] = make_float4(th, a.sig[3 * n + 0], a.sig[3 * n + 1], a.sig[3 * n + 2]);
+#pragma unroll
+        for (int i = 0; i < NS; ++i) {
+            const int e = tid + i * NT, m = e / T, s = e - m * T;
+            if (m >= cn) continue;
+            // time part of the phase modulo one turn; its top 32 bits as a signed
+            // fraction of half a turn
+            const unsigned long long q = ph[i] + om[i] * (unsigned long long)(t + s);
+            float sn, cs;
+            sincospif((float)(int)(unsigned)(q >> 32) * 4.656612873077393e-10f, &sn, &cs);  // 2^-31
+            ts[m][s] = make_float2(cs, sn);
         }
-        for (int e = tid; e < cn * INLET_K; e += INLET_J * INLET_WARPS) {
-            const int m = e / INLET_K, kk = e % INLET_K;
-            const int k = min(k0 + kk, nz - 1);  // span nodes past nz are computed and not stored
-            reinterpret_cast<float *>(&bz[m][0])[kk] = a.B[(size_t)(n0 + m) * nz + k];
+#pragma unroll
+        for (int i = 0; i < NY; ++i) {
+            const int m = w + i * INLET_WARPS;
+            if (m < cn) ys[m][lane] = y[i];
         }
-        for (int e = tid; e < cn * INLET_J; e += INLET_J * INLET_WARPS) {
-            const int m = e / INLET_J, jj = min(j0 + e % INLET_J, ny - 1);  // rows past ny are not stored
-            ay_s[m][e % INLET_J] = a.A[(size_t)(n0 + m) * ny + jj];
-            sq_s[m][e % INLET_J] = a.SQ[(size_t)(n0 + m) * ny + jj];
+        if (tid < cn) sg[tid] = sgr;
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < NB; ++i) {
+            const int e = tid + i * NT, m = e / ITEMS, q = e % ITEMS;
+            if (m >= cn || q >= items) continue;
+            const float2 th = ts[m][q % T];
+            is[m][q] = make_float2(fmaf(b[i].x, th.x, -__fmul_rn(b[i].y, th.y)),
+                                   fmaf(b[i].y, th.x, __fmul_rn(b[i].x, th.y)));
         }
+        if (n0 + CHUNK < N) fetch(n0 + CHUNK);
         __syncthreads();
 #pragma unroll 4
-        for (int m = h; m < cn; m += INLET_H) {
-            const float4 tm = ts[m];
-            const float ay = ay_s[m][lane] + tm.x;  // in [0, 4 pi)
-            const float sq = sq_s[m][lane];
-            const float2 b2 = bz[m][g];
-            const float bq[INLET_KPT] = {b2.x, b2.y};
+        for (int m = 0; m < cn; ++m) {
+            const float2 y = ys[m][lane];
+            const float4 s = sg[m];
 #pragma unroll
-            for (int q = 0; q < INLET_KPT; ++q) {
-                float arg = ay + bq[q];                           // in [0, 6 pi)
-                arg -= 6.2831853f * rintf(arg * 0.15915494f);     // to [-pi, pi]
-                const float amp = sq * __cosf(arg);
-                v[q][0] = fmaf(amp, tm.y, v[q][0]);
-                v[q][1] = fmaf(amp, tm.z, v[q][1]);
-                v[q][2] = fmaf(amp, tm.w, v[q][2]);
+            for (int q = 0; q < IPW; ++q) {
+                const float2 bq = is[m][w * IPW + q];
+                const float c = fmaf(y.x, bq.x, -__fmul_rn(y.y, bq.y));
+                v[q][0] = fmaf(c, s.x, v[q][0]);
+                v[q][1] = fmaf(c, s.y, v[q][1]);
+                v[q][2] = fmaf(c, s.z, v[q][2]);
             }
         }
     }
-    if (h == 1) {
 #pragma unroll
-        for (int q = 0; q < INLET_KPT; ++q)
+    for (int q = 0; q < IPW; ++q)
 #pragma unroll
-            for (int c = 0; c < 3; ++c) part[g][q][c][lane] = v[q][c];
-    }
+        for (int c = 0; c < 3; ++c) vs[w * IPW + q][c][lane] = v[q][c];
     __syncthreads();
-    if (h == 1 || !jl) return;
-    const float *L = a.a6 + 6 * j;
-    const float l11 = L[0], l21 = L[1], l22 = L[2], l31 = L[3], l32 = L[4], l33 = L[5];
-    const float af = a.a_filter, bf = 1.0f - a.a_filter, ui = a.u_int[j];
-    const size_t plane = (size_t)ny * nz;
+    for (int e = tid; e < kb * INLET_J; e += NT, mine = fetch_node(e)) {
+        if (!mine) continue;
+        const int jj = e % INLET_J, kk = e / INLET_J;
+        const size_t node = (size_t)(k0 + kk) * ny + j0 + jj;
+        for (int s = 0; s < T; ++s) {
+            const float *vq = &vs[kk * T + s][0][jj];
+            const float v0 = vq[0], v1 = vq[INLET_J], v2 = vq[2 * INLET_J];
+            const float u[3] = {__fmul_rn(L[0], v0), fmaf(L[2], v1, __fmul_rn(L[1], v0)),
+                                fmaf(L[5], v2, fmaf(L[4], v1, __fmul_rn(L[3], v0)))};
+            const bool first = (t + s == t0f);
+            float *o = a.ubc + (size_t)((t + s) & (INLET_RING - 1)) * 3 * plane + node;
 #pragma unroll
-    for (int q = 0; q < INLET_KPT; ++q) {
-        const int k = k0 + g * INLET_KPT + q;
-        if (k >= nz) break;
-        const float v0 = v[q][0] + part[g][q][0][lane];
-        const float v1 = v[q][1] + part[g][q][1][lane];
-        const float v2 = v[q][2] + part[g][q][2][lane];
-        const size_t node = (size_t)k * ny + j;
-        const float u0 = l11 * v0;
-        const float u1 = l21 * v0 + l22 * v1;
-        const float u2 = l31 * v0 + l32 * v1 + l33 * v2;
-        float f0 = u0, f1 = u1, f2 = u2;
-        if (!first) {
-            f0 = af * a.uf[node] + bf * u0;
-            f1 = af * a.uf[plane + node] + bf * u1;
-            f2 = af * a.uf[2 * plane + node] + bf * u2;
+            for (int c = 0; c < 3; ++c) {
+                f[c] = first ? u[c] : fmaf(af, f[c], __fmul_rn(bf, u[c]));
+                o[c * plane] = c == 0 ? ui + f[c] : f[c];
+            }
         }
-        a.uf[node] = f0;
-        a.uf[plane + node] = f1;
-        a.uf[2 * plane + node] = f2;
-        a.ubc[node] = ui + f0;
-        a.ubc[plane + node] = f1;
-        a.ubc[2 * plane + node] = f2;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) a.uf[c * plane + node] = f[c];
     }
 }
 
 cudaError_t launch_inlet(const InletArgs &a, cudaStream_t s)
 {
-    const dim3 grid((a.ny + INLET_J - 1) / INLET_J, (a.nz + INLET_K - 1) / INLET_K);
-    if (grid.y > 65535u) return cudaErrorInvalidConfiguration;  // nz > 524 280
-    stg_inlet_kernel<<<grid, dim3(INLET_J, INLET_WARPS), 0, s>>>(a);
+    if (a.planes < 1 || a.planes > INLET_MAX_PLANES) return cudaErrorInvalidValue;
+    const int ipw = a.planes > INLET_WARPS ? 4 : 1;
+    const int kb = ipw * INLET_WARPS / a.planes;
+    const dim3 grid((a.ny + INLET_J - 1) / INLET_J, (a.nz + kb - 1) / kb);
+    if (grid.y > 65535u) return cudaErrorInvalidConfiguration;
+    const dim3 block(INLET_J, INLET_WARPS);
+    if (ipw == 4) stg_inlet_kernel<4><<<grid, block, 0, s>>>(a, kb);
+    else stg_inlet_kernel<1><<<grid, block, 0, s>>>(a, kb);
     return cudaGetLastError();
 }
 

@@ -14,8 +14,14 @@ namespace stg {
 struct StepCtl {
     long long t[2];
     long long t0_filter;  // step at which the temporal filter restarts
+    long long t_block;    // step at which the current block of steps began
     unsigned long long err; // error bits set by kernels (none of the current kernels sets one)
 };
+
+// Inlet velocity planes are kept in a ring by step index (a power of two).  A
+// launch computes at most INLET_MAX_PLANES of them; the steps of a block read the
+// planes of one launch while the next launch writes its own.
+constexpr int INLET_RING = 32, INLET_MAX_PLANES = 16;
 
 struct StepArgs {
     const void *src;      // post-collision populations of the previous step
@@ -32,38 +38,37 @@ struct StepArgs {
     int il, ir;             // 32-wide x chunks [il, ir) of rows 1..ny-2 belong to the interior kernel
     int interior;           // interior kernel: 0 best available, 1 one cell per thread, 2 cell pairs
     int aa;                 // 1: one lattice updated in place (AA pattern; src == dst), 0: two lattices
-    // tile of the plain (non-sampling) vector launches: layout 0 = 8 z-warps on one 64-cell x chunk,
-    // layout 1 = 4 x-warps (256 cells) walking z together; zc / wall_zc = z planes per block of the
-    // rows 1..ny-2 / wall-row launch (0: the whole z column)
-    int tile_layout, tile_zc, tile_wall_zc;
+    // z planes per run of the plain (non-sampling) vector launches at most, inner / wall rows (0: the whole z column)
+    int tile_zc, tile_wall_zc;
+    int row_step;           // vector launches of the rows 0, row_step, ...
+    int stat_group;         // z planes per run of the sampling vector launches
     unsigned total_blocks;  // blocks of all step kernels of the pass (mass-check completion count)
     int slot_base;          // first mass-partial slot of this launch's blocks
-    int bump_t;             // this launch advances the device step counter
     int nx, ny, nz;
     unsigned P;           // cells per population plane (nx*ny*nz)
+    long long in_flight;  // cells of all lattices advanced together (a batch's members; else P)
     int bc_x, bc_y;       // STG_BC_X_*, STG_BC_Y_*
     float tau0, kq;       // kq = 18 sqrt(2) C  (eq. tau_eff)
     float Fx, Fy, Fz;
     int has_force;
-    const float *ubc;     // inlet velocity plane [3][nz][ny]
+    const float *ubc;     // inlet velocity planes [INLET_RING][3][nz][ny], step t in plane t mod INLET_RING
     const float *spf;     // sponge zone: viscosity factor per column x [nx] (eq. sponge_visco); nullptr: off
     StepCtl *ctl;
     int parity;
     int stats_every, check_every;
     double *stat_mean;    // [3][ny][nx]
     double *stat_rey;     // [6][ny][nx]
-    float *stat_part;     // sampling steps of the vector kernels: FP32 sums per group of
-                          // STAT_GROUP z planes, [ceil(nz / STAT_GROUP)][9][ny][nx]
-    double *mass_partial; // [gridDim.x * gridDim.y]
-    unsigned *mass_counter;
+    float *stat_part;     // sampling steps of the vector kernels: FP32 sums per run of
+                          // stat_group z planes, [ceil(nz / stat_group)][9][ny][nx]
+    double *mass_partial; // one slot per block, then one per MASS_GROUP blocks
+    unsigned *mass_counter;  // one per MASS_GROUP blocks, then one
     double *mass_out;     // [0]: last checked mass
 };
 
 struct InletArgs {
     int ny, nz, N;
-    const float *A;       // [N][ny]  k^n d^n_y (j + 1/2) mod 2 pi
-    const float *B;       // [N][nz]  k^n d^n_z k       mod 2 pi
-    const float *SQ;      // [N][ny]  sqrt(6 q^n(y_j))
+    const float2 *AS;     // [N][ny]  sqrt(6 q^n(y_j)) (cos, sin) of k^n d^n_y (j + 1/2)
+    const float2 *BS;     // [N][nz]  (cos, sin) of k^n d^n_z k
     const float *sig;     // [N][3]   sigma^n
     const unsigned long long *phq;  // [N] phi^n / (2 pi) as a Q0.64 fraction of a turn
     const unsigned long long *omq;  // [N] phase advance per step, -d^n_x U_b / max l_e turns, Q0.64
@@ -71,8 +76,9 @@ struct InletArgs {
     const float *u_int;   // [ny]     interpolated mean streamwise velocity
     float a_filter;
     float *uf;            // [3][nz][ny] filtered fluctuation (state)
-    float *ubc;           // [3][nz][ny] inlet velocity output
-    int ahead;            // the plane is for step t + ahead (t = ctl->t[parity])
+    float *ubc;           // inlet velocity planes, as in StepArgs (output)
+    int ahead, planes;    // the planes of steps t + ahead .. t + ahead + planes - 1
+    int from_block;       // t: 0 ctl->t[parity] (noted as ctl->t_block), 1 ctl->t_block
     StepCtl *ctl;
     int parity;
 };
@@ -89,13 +95,25 @@ struct MassArgs {
 // launchers (return the launch status)
 // `stats` must be true exactly on sampling steps ((t + 1) % stats_every == 0);
 // the host tracks t and decides.
-// inlet: the inlet kernel for the next step's plane (NULL: none), launched on the branch
 cudaError_t launch_step(const StepArgs &a, int storage, int collision, bool stats,
-                        cudaStream_t s, cudaStream_t side, cudaEvent_t fork, cudaEvent_t join,
-                        const InletArgs *inlet = nullptr);
+                        cudaStream_t s, cudaStream_t side, cudaEvent_t fork, cudaEvent_t join);
 // binary16 regularized unforced lattices take quads (four cells per lane)
 // when the rows split into whole quads
 inline bool quads_fit(int nx) { return nx % 4 == 0 && nx >= 8; }
+// Lattices of the vector kernels (the others take one cell per thread): rows of
+// whole pairs and 32-bit element offsets.  The in-place scheme exists for them
+// only (the host checks its conditions), so it ignores the interior override.
+inline bool vector_fits(const StepArgs &a)
+{
+    return (a.aa || a.interior == 0 || a.interior == 2) && a.nx % 2 == 0 && a.nx >= 4 &&
+           19.0 * a.nx * a.ny * a.nz < 4294967296.0 && (a.bc_x != 0 || a.nx >= 3);
+}
+// Whether a pass of the vector kernels (cpl cells per lane) is one launch of all
+// rows, and the z planes per run of its launches (step_kernel.cu).
+bool one_launch(const StepArgs &a, int cpl);
+int run_planes(const StepArgs &a, int cpl, int tile_zc, int elem, bool walls);
+// cells per lane of the vector kernels
+int lane_cells(const StepArgs &a, int storage, int collision);
 cudaError_t launch_inlet(const InletArgs &a, cudaStream_t s);
 // FP64 Cholesky factor of the lattice-unit Reynolds stress per inlet node (setup)
 cudaError_t launch_setup_nodes(int ny, const double *R6, float *a6, cudaStream_t s);
@@ -117,13 +135,18 @@ cudaError_t launch_probe(const void *src, int storage, const LatticeView &lv, in
 cudaError_t launch_gather_block(const void *src, int storage, const LatticeView &lv, int x0, int y0, int z0, int bx,
                                 int by, int bz, void *out, cudaStream_t s);
 
-// Upper bound of the mass-partial slots of one step pass over every tile
-// that set_tile accepts (z chunks of at least MIN_ZC planes).
+// shortest z chunk that set_tile accepts
 constexpr int MIN_ZC = 4;
-// z planes per block on sampling steps of the vector kernels (fixed, so the
-// statistics do not depend on the launch tile)
-constexpr int STAT_GROUP = 32;
+// z planes per run on sampling steps of the vector kernels, walked by STAT_WARPS
+// warps: a function of the lattice alone, so the statistics do not depend on the
+// launch tile
+constexpr int STAT_WARPS = 4;
+int stat_group(int nx, int ny, int nz);
+// Upper bound of the blocks of one step pass over every tile.
 int step_grid_blocks(int nx, int ny, int nz);
+// Blocks whose mass partials are added by the last of them to finish.
+constexpr int MASS_GROUP = 1024;
+inline int mass_groups(int blocks) { return (blocks + MASS_GROUP - 1) / MASS_GROUP; }
 int mass_grid_blocks();
 
 }  // namespace stg

@@ -1,12 +1,13 @@
-// Step kernels of shifted binary16 storage with the plain BGK collision (one of four
-// instantiation units of step_kernel.cuh, compiled in parallel).
+// Step kernels of shifted binary16 storage,
+// the plain BGK collision, two cells per lane (one of the instantiation units of step_kernel.cuh,
+// compiled in parallel).
 #include "step_kernel.cuh"
 
 namespace stg {
 
 bool launch_f16_bgk(const StepArgs &a, bool stats, cudaStream_t s, cudaStream_t side)
 {
-    return launch_typed<__half, false>(a, stats, s, side);
+    return launch_typed<__half, 2, false>(a, stats, s, side);
 }
 
 }  // namespace stg

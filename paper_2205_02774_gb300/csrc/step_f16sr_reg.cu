@@ -1,13 +1,13 @@
 // Step kernels of shifted binary16 storage written by stochastic rounding,
-// with the regularized collision (one of the instantiation units of
-// step_kernel.cuh, compiled in parallel).
+// the regularized collision, two cells per lane (one of the instantiation units of step_kernel.cuh,
+// compiled in parallel).
 #include "step_kernel.cuh"
 
 namespace stg {
 
 bool launch_f16sr_reg(const StepArgs &a, bool stats, cudaStream_t s, cudaStream_t side)
 {
-    return launch_typed<__half, true, true>(a, stats, s, side);
+    return launch_typed<__half, 2, true, true>(a, stats, s, side);
 }
 
 }  // namespace stg

@@ -1,6 +1,8 @@
 // Host-side launch of one fused step pass (the kernels: step_kernel.cuh and
 // its six instantiation units), the initial-state kernel, the statistics
 // reduction of sampling steps and the FP64 mass reduction.
+#include <algorithm>
+
 #include <cuda_fp16.h>
 
 #include "d3q19.cuh"
@@ -12,19 +14,79 @@ namespace stg {
 
 constexpr int BX = 32;
 
-// instantiation units (step_f32_*.cu, step_f16_*.cu, step_f16sr_*.cu; reg / bgk collision)
-bool launch_f32_reg(const StepArgs &a, bool stats, cudaStream_t s, cudaStream_t side);
-bool launch_f32_bgk(const StepArgs &a, bool stats, cudaStream_t s, cudaStream_t side);
-bool launch_f16_reg(const StepArgs &a, bool stats, cudaStream_t s, cudaStream_t side);
-bool launch_f16_bgk(const StepArgs &a, bool stats, cudaStream_t s, cudaStream_t side);
-bool launch_f16sr_reg(const StepArgs &a, bool stats, cudaStream_t s, cudaStream_t side);
-bool launch_f16sr_bgk(const StepArgs &a, bool stats, cudaStream_t s, cudaStream_t side);
+// instantiation units (step_<storage>_<collision>[_quad].cu)
+using Pass = bool (*)(const StepArgs &a, bool stats, cudaStream_t s, cudaStream_t side);
+bool launch_f32_reg(const StepArgs &, bool, cudaStream_t, cudaStream_t),
+    launch_f32_bgk(const StepArgs &, bool, cudaStream_t, cudaStream_t),
+    launch_f16_reg(const StepArgs &, bool, cudaStream_t, cudaStream_t),
+    launch_f16_reg_quad(const StepArgs &, bool, cudaStream_t, cudaStream_t),
+    launch_f16_bgk(const StepArgs &, bool, cudaStream_t, cudaStream_t),
+    launch_f16sr_reg(const StepArgs &, bool, cudaStream_t, cudaStream_t),
+    launch_f16sr_reg_quad(const StepArgs &, bool, cudaStream_t, cudaStream_t),
+    launch_f16sr_bgk(const StepArgs &, bool, cudaStream_t, cudaStream_t);
 
 int step_grid_blocks(int nx, int ny, int nz)
 {
-    const long long vec = (long long)((nx + 2 * BX - 1) / (2 * BX)) * ny * ((nz + MIN_ZC - 1) / MIN_ZC);
+    const long long vec = (long long)((nx + 2 * BX - 1) / (2 * BX)) * ny * nz;  // one plane per item
     const long long col = (long long)((nx + BX - 1) / BX) * ny;
     return (int)((vec > col ? vec : col) + 2LL * ny + 64);
+}
+
+// The longer a run, the less scratch a sampling step writes and reads (36 B each
+// per cell and run), and the longer the serial walk of its warps: 32 planes (8 per
+// warp), but less where that leaves the GPU's resident warps less than one and a
+// half chunks of 64 cells each (a plane takes a warp 2 to 4 us when little else is
+// in flight: 64x32x32 spent 160 us on a sampling step of one 32-plane run per warp).
+int stat_group(int nx, int ny, int nz)
+{
+    const long long rows = (long long)((nx + 2 * BX - 1) / (2 * BX)) * ny;
+    int g = 32;
+    while (g > STAT_WARPS && rows * ((nz + g - 1) / g) * STAT_WARPS < 152LL * 32 * 3 / 2 && nz / (g / 2) < 65535) g /= 2;
+    return g;
+}
+
+int lane_cells(const StepArgs &a, int storage, int collision)
+{
+    return storage != 0 && collision == 0 && !a.has_force && quads_fit(a.nx) && vector_fits(a) ? 4 : 2;
+}
+
+// Items: one x chunk (32 cpl cells) of one row and plane each, of all lattices
+// that advance together.  While the GPU's warps (16 per SM with the registers of
+// the kernel for any row) have only a few each, a pass is bound by launches and by
+// the latency of one plane, and one launch of all rows saves the branch of the wall
+// rows: 64x32x32 5.6 against 8.2 us per step, 240x40x60 FP32 (3.9 items per warp)
+// 18.0 against 21.0.  Above that the inner rows' own kernel, with more warps per SM,
+// is the faster one: 384x64x96 FP32 (15) 57 against 73 us, 324x54x81 FP16 (5.4) 30.6
+// against 35.0, 240x40x60 FP16 (2.0) 13.2 against 14.4.
+static long long items_of(const StepArgs &a, int cpl)
+{
+    const long long own = (long long)((a.nx + BX * cpl - 1) / (BX * cpl)) * a.ny * a.nz;
+    return std::max(own, a.in_flight / (BX * cpl));
+}
+
+bool one_launch(const StepArgs &a, int cpl)
+{
+    return a.ny < 3 || items_of(a, cpl) * 2 < 152LL * 16 * (cpl == 4 ? 3 : 8);
+}
+
+// A run of several planes costs one block start instead of several, but a pass
+// ends with its last runs, and a short pass needs every warp from the start: so
+// runs grow with the number of items per resident warp.  FP32 (256 B per row piece)
+// is fastest with runs of 1 or 2 (768x128x192: 415, 418, 425 us with 2, 4, 8;
+// 1536x256x384: 3.27, 3.29, 3.31, 3.34 ms with 1, 2, 4, 8), binary16 with 4 or 8
+// (1536x256x384: 1.82, 1.76, 1.72, 1.72 ms with 1, 2, 4, 8; 384x64x96: 2).
+// The wall rows, beside the inner launch, are spread over as many warps as their
+// latency needs: binary16 1, FP32 4 (768x128x192: FP16 226, 228, 230 us with
+// 1, 2, 4, and 236 with 24; FP32 420, 420, 418), and 4 among the members of a batch.
+int run_planes(const StepArgs &a, int cpl, int tile_zc, int elem, bool walls)
+{
+    const int most = tile_zc > 0 ? tile_zc : a.nz;
+    const int least = (a.nz + 65534) / 65535;  // a launch holds 65535 runs
+    if (walls) return std::max(least, std::min(most, elem == 4 || a.in_flight > a.P ? 4 : 1));
+    const long long per_warp = items_of(a, cpl) / (152 * (elem == 4 ? 32 : 20));
+    int zc = 1;
+    while (zc < (elem == 4 ? 2 : 8) && per_warp >= 5 * zc) zc *= 2;
+    return std::max(least, std::min(zc, most));
 }
 
 // Adds the z-group sums of a sampling step to the FP64 statistics, group by
@@ -39,7 +101,7 @@ __global__ void stats_reduce_kernel(const float *part, int groups, size_t m, dou
     // is a small fraction of its FP32 rate, and an FP64 conversion and add per
     // group made this kernel FP64-bound
     float hi = 0.f, lo = 0.f;
-#pragma unroll 4
+#pragma unroll 8
     for (int g = 0; g < groups; ++g) {
         const float x = __ldcs(part + (size_t)g * 9 * m + k);
         const float s = hi + x;
@@ -52,41 +114,26 @@ __global__ void stats_reduce_kernel(const float *part, int groups, size_t m, dou
     else stat_rey[k - 3 * m] += sum;
 }
 
-// One fused step pass.  With a side stream and two events the wall rows (or
-// the edge kernel on the scalar path) run on a forked branch concurrently
-// with the interior (they read and write disjoint slots: the previous and the
-// next lattice, or, in place, the slots of their own cells); `s` waits for
-// both.  `inlet`
-// (may be NULL) computes the next step's inlet plane on the branch.
+// One fused step pass.  The wall rows (or the edge kernel of the one-cell-per-
+// thread path) run on the forked branch `side` beside the inner rows (they write
+// disjoint slots); `s` waits for both.  A pass of one launch needs no branch.
 cudaError_t launch_step(const StepArgs &a, int storage, int collision, bool stats,
-                        cudaStream_t s, cudaStream_t side, cudaEvent_t fork, cudaEvent_t join, const InletArgs *inlet)
+                        cudaStream_t s, cudaStream_t side, cudaEvent_t fork, cudaEvent_t join)
 {
     cudaError_t e = cudaSuccess;
-    const bool forked = side != nullptr && fork != nullptr && join != nullptr;
+    const int cpl = lane_cells(a, storage, collision);
+    const bool one = vector_fits(a) && one_launch(a, cpl);
+    const bool forked = !one && side != nullptr && fork != nullptr && join != nullptr;
     if (forked) {
         if ((e = cudaEventRecord(fork, s)) != cudaSuccess) return e;
         if ((e = cudaStreamWaitEvent(side, fork, 0)) != cudaSuccess) return e;
     }
     cudaStream_t es = forked ? side : s;
-    // the inlet kernel writes the plane of the next step, which nothing in
-    // this pass reads, so it runs on the branch beside the interior; beside a
-    // quad interior (96-register warps filling the SMs' registers) its
-    // 256-thread blocks waited for room and the step ran slower than with the
-    // inlet ahead of the pass (FP16-SR 1.813 against 1.771 ms on 1536x256x384),
-    // so there it goes first on the main stream
-    const bool quad = storage != 0 && collision == 0 && !a.has_force && quads_fit(a.nx);
-    if (inlet && (e = launch_inlet(*inlet, quad ? s : es)) != cudaSuccess) return e;
-    bool reduce = false;
-    if (storage == 0) {
-        if (collision == 0) reduce = launch_f32_reg(a, stats, s, es);
-        else reduce = launch_f32_bgk(a, stats, s, es);
-    } else if (storage == 1) {
-        if (collision == 0) reduce = launch_f16_reg(a, stats, s, es);
-        else reduce = launch_f16_bgk(a, stats, s, es);
-    } else {
-        if (collision == 0) reduce = launch_f16sr_reg(a, stats, s, es);
-        else reduce = launch_f16sr_bgk(a, stats, s, es);
-    }
+    // by storage and collision, two and four cells per lane
+    static constexpr Pass passes[3][2][2] = {{{launch_f32_reg, nullptr}, {launch_f32_bgk, nullptr}},
+                                             {{launch_f16_reg, launch_f16_reg_quad}, {launch_f16_bgk, nullptr}},
+                                             {{launch_f16sr_reg, launch_f16sr_reg_quad}, {launch_f16sr_bgk, nullptr}}};
+    const bool reduce = passes[storage][collision][cpl == 4](a, stats, s, es);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (forked) {
         if ((e = cudaEventRecord(join, side)) != cudaSuccess) return e;
@@ -94,7 +141,7 @@ cudaError_t launch_step(const StepArgs &a, int storage, int collision, bool stat
     }
     if (reduce) {
         const size_t m = (size_t)a.nx * a.ny;
-        const int groups = (a.nz + STAT_GROUP - 1) / STAT_GROUP;
+        const int groups = (a.nz + a.stat_group - 1) / a.stat_group;
         const unsigned blocks = (unsigned)((9 * m + 255) / 256);
         stats_reduce_kernel<<<blocks, 256, 0, s>>>(a.stat_part, groups, m, a.stat_mean, a.stat_rey);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;

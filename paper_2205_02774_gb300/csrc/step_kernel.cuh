@@ -14,10 +14,11 @@
 // velocity statistics and the FP64 mass.
 //
 // Layout: SoA f[i][z][y][x].  The even-nx path (vector kernels) gives each
-// lane two consecutive x cells; plain steps cut the lattice into blocks of
-// (x chunk, row, z chunk) chosen by the launch tile, sampling steps into
-// fixed groups of z planes whose per-(x, y) sums are added in order.  The
-// odd-nx path (one cell per thread) keeps a block per (x chunk, row) column.
+// lane two or four consecutive x cells and a warp an x chunk of one row over a
+// run of z planes: on plain steps as long as the lattice's size makes best
+// (run_planes), on sampling steps a function of the lattice alone, whose
+// per-(x, y) sums are added in order.  The odd-nx path (one cell per thread)
+// keeps a block per (x chunk, row) column.
 //
 // Streaming schemes (vector kernels, MODE):
 //  PULL      two lattices: read src[i] at x - c_i, write dst[i] at x;
@@ -47,6 +48,16 @@
 namespace stg {
 
 constexpr int PULL = 0, AA_SHIFT = 1, AA_LOCAL = 2;
+
+// the place of this step's plane in StepArgs::ubc; the step index is read again
+// (an L1 hit, by the lanes that hold an inlet node) rather than kept in a
+// register over the plane loop, which several instances would spill for
+__device__ __forceinline__ size_t inlet_plane(const StepArgs &a)
+{
+    unsigned t;
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(t) : "l"(&a.ctl->t[a.parity]));
+    return (size_t)(t & (INLET_RING - 1));
+}
 
 // Stochastic rounding of binary16 stores (SR kernels): a value between two
 // binary16 neighbours goes to the upper one with probability equal to its
@@ -185,7 +196,8 @@ __device__ __forceinline__ void step_column(const StepArgs &a, int bx, int y)
                 gather_general<S>(src, P, nx, ny, x, y, z, xm, xp, xm_ok, xp_ok, ym, yp, ym_w, yp_w, zm, zp, here, g);
                 if (inout && (x == 0 || x == nx - 1)) {
                     if (x == 0) {
-                        const size_t pc = (size_t)z * ny + y, pl3 = (size_t)ny * nz;
+                        const size_t pl3 = (size_t)ny * nz;
+                        const size_t pc = inlet_plane(a) * 3 * pl3 + (size_t)z * ny + y;
                         const float ubx = a.ubc[pc], uby = a.ubc[pl3 + pc], ubz = a.ubc[2 * pl3 + pc];
                         // Zou-He density, eq. (density_bc): parallel set + 2 x leaving set.
                         // The weights of that combination sum to 1 (2/3 + 2 x 1/6), so
@@ -425,6 +437,7 @@ struct Vec<__half, 2> {
 
 template <>
 struct Vec<__half, 4> {
+    using Half = Vec<__half, 2>;
     using raw = uint2;  // x: cells 0, 1 (low half first); y: cells 2, 3
     // 8-byte read-only load with the 256-byte L2 fetch (a warp reads a 256 B row piece)
     static __device__ __forceinline__ raw ld(const __half *p)
@@ -434,23 +447,23 @@ struct Vec<__half, 4> {
         return v;
     }
     static __device__ __forceinline__ unsigned word(raw v, int j) { return j < 2 ? v.x : v.y; }
-    static __device__ __forceinline__ float cell(raw v, int j) { return Vec<__half, 2>::cell(word(v, j), j & 1); }
+    static __device__ __forceinline__ float cell(raw v, int j) { return Half::cell(word(v, j), j & 1); }
     // cells 2k and 2k + 1 in FP32
-    static __device__ __forceinline__ float2 pair(raw v, int k) { return Vec<__half, 2>::pair(k ? v.y : v.x); }
-    static __device__ __forceinline__ float add_h(raw v, int j, float c) { return Vec<__half, 2>::add_h(word(v, j), j & 1, c); }
-    static __device__ __forceinline__ float sub_h(raw v, int j, float c) { return Vec<__half, 2>::sub_h(word(v, j), j & 1, c); }
+    static __device__ __forceinline__ float2 pair(raw v, int k) { return Half::pair(k ? v.y : v.x); }
+    static __device__ __forceinline__ float add_h(raw v, int j, float c) { return Half::add_h(word(v, j), j & 1, c); }
+    static __device__ __forceinline__ float sub_h(raw v, int j, float c) { return Half::sub_h(word(v, j), j & 1, c); }
     // cells 2k, 2k + 1 <- lo, hi (round to nearest, or stochastic rounding with bits rb)
     static __device__ __forceinline__ void set_pair(raw &v, int k, float lo, float hi)
     {
-        (k ? v.y : v.x) = Vec<__half, 2>::pack(lo, hi);
+        (k ? v.y : v.x) = Half::pack(lo, hi);
     }
     static __device__ __forceinline__ void set_pair_rs(raw &v, int k, float lo, float hi, unsigned rb)
     {
-        (k ? v.y : v.x) = Vec<__half, 2>::pack_rs(lo, hi, rb);
+        (k ? v.y : v.x) = Half::pack_rs(lo, hi, rb);
     }
     static __device__ __forceinline__ void st(__half *p, raw v) { __stcs(reinterpret_cast<uint2 *>(p), v); }
     // cell j at p + j
-    static __device__ __forceinline__ void st1(__half *p, raw v, int j) { Vec<__half, 2>::st1(p + (j & 2), word(v, j), j & 1); }
+    static __device__ __forceinline__ void st1(__half *p, raw v, int j) { Half::st1(p + (j & 2), word(v, j), j & 1); }
     // cells 1 and 2 as one aligned pair at p
     static __device__ __forceinline__ void st_mid(__half *p, raw v)
     {
@@ -485,8 +498,8 @@ struct Vec<__half, 4> {
     }
 };
 
-// One vector column (CPL 32 cells wide) at row y over the planes z = zb,
-// zb + zs, ... below ze.  YEDGE rows
+// One vector column (CPL 32 cells wide) at row y over the planes zb, zb + zs, ...
+// below ze.  YEDGE rows
 // (y = 0 or ny-1) take the y neighbour by half-way bounce-back (walls: the
 // cell's own opposite population) or by the periodic wrap.  In inlet/outlet
 // mode the inlet node x = 0 is rebuilt by the regularized Zou-He
@@ -657,7 +670,8 @@ __device__ __forceinline__ float vec_loop(const StepArgs &a, float (*sacc)[9][BX
                     // Zou-He density, eq. (density_bc): parallel set + 2 x leaving set,
                     // rho_bc - 1 = (S_g + u_x)/(1 - u_x) in shifted variables; the
                     // unknowns (c_x > 0, their sources lie outside) are not read
-                    const size_t pc = (size_t)z * ny + y, pl3 = (size_t)ny * nz;
+                    const size_t pl3 = (size_t)ny * nz;
+                    const size_t pc = inlet_plane(a) * 3 * pl3 + (size_t)z * ny + y;
                     const float ubx = a.ubc[pc], uby = a.ubc[pl3 + pc], ubz = a.ubc[2 * pl3 + pc];
                     float par = 0.f, lv = 0.f;
 #pragma unroll
@@ -790,102 +804,70 @@ __device__ __forceinline__ float vec_loop(const StepArgs &a, float (*sacc)[9][BX
     return sdr;
 }
 
-// Sampling-step vector kernel over all x of rows 1..ny-2 (YEDGE false) or of
-// rows 0 and ny-1 (YEDGE true; that launch also advances the device step
-// counter).  Block (4 consecutive 64-cell x chunks, or one 128-cell quad
-// chunk, row, group of STAT_GROUP z planes); each warp walks the group's planes in order for its own chunk
-// (the plain kernel's layout 1), its lanes adding the velocity moments of
-// their cells to private shared-memory slots, and writes the group's FP32
-// sums per (x, y) to the group's slot of a.stat_part; stats_reduce_kernel
-// then adds the groups in order.  The decomposition is fixed (no tile), so
-// the statistics are deterministic and independent of the launch tile.
-// H16 as in vec_loop.  STATS is chosen on the host (it knows the step
-// count); plain steps use lbm_vec_zc_kernel.
-// warps (x chunks) per block of the layout-1 and sampling kernels: 4 with
-// pairs (256 cells), one with quads (128 cells: wider quad blocks leave warps
-// idle on rows that are not a multiple of their width, e.g. a quarter of them
-// on 768-cell rows, and were no faster on 1536-cell rows)
-constexpr int QUAD_NW = 1;
-template <int CPL>
-constexpr int chunk_warps() { return CPL == 4 ? QUAD_NW : 4; }
-template <typename S, int CPL, bool REG, bool FORCE, bool STATS, bool YEDGE, bool SP, bool H16, int MODE, bool SR>
-// (the wall rows, on the branch beside the interior launch, may take 128
-// registers so that they need no stack frame; binary16 quads take 96)
-__global__ void __launch_bounds__(BX *chunk_warps<CPL>(), (YEDGE ? 16 : ((REG && !FORCE) ? (CPL == 4 ? 20 : 32) : 24)) / chunk_warps<CPL>())
+// Rows of a vector launch: INNER, y = 1..ny-2, or ANY, y = 0, a.row_step, ...
+// (all rows, or the wall rows alone).
+constexpr int INNER = 0, ANY = 1;
+
+// Warps per block and the occupancy asked for.  The regularized unforced inner
+// rows fit 64 registers with pairs (32 warps per SM) and 96 with binary16 quads
+// (20 warps per SM: with 8-byte row pieces those warps keep as many bytes in
+// flight as FP32); BGK, forced and sampling pairs get 80; sampling quads, and the
+// launches of any rows (the wall rows beside the inner launch, all rows of a lattice too
+// small to fill the GPU) 128, so that they need no stack frame.
+template <int CPL, bool STATS>
+constexpr int block_warps() { return STATS ? STAT_WARPS : (CPL == 4 ? 1 : 4); }
+template <int CPL, bool LEAN, bool STATS, int ROWS>
+constexpr int warps_per_sm() { return ROWS != INNER ? 16 : (CPL == 4 ? (STATS ? 16 : 20) : (LEAN && !STATS ? 32 : 24)); }
+
+// The vector kernel: block (x chunks, row, run of z planes).
+// Plain steps (STATS false): the warps of a block take x chunks side by side
+// and each walks the run's a.tile_zc planes for its own.
+// Sampling steps: the STAT_WARPS warps take every STAT_WARPS-th plane of one
+// chunk's run of a.stat_group planes, a function of the lattice alone.  The lanes
+// add the velocity moments of their cells to private shared-memory slots, the
+// warps' slots are added in order, and the run's FP32 sums per (x, y) go to the
+// run's slot of a.stat_part, where stats_reduce_kernel adds the runs in order, so
+// the statistics are deterministic and independent of the launch tile.  H16 as in
+// vec_loop.  STATS is chosen on the host (it knows the step count).
+template <typename S, int CPL, bool REG, bool FORCE, bool STATS, int ROWS, bool SP, bool H16, int MODE, bool SR>
+__global__ void __launch_bounds__(BX *block_warps<CPL, STATS>(), warps_per_sm<CPL, REG && !FORCE, STATS, ROWS>() / block_warps<CPL, STATS>())
     lbm_vec_kernel(const StepArgs a)
 {
-    constexpr int STAT_NW = chunk_warps<CPL>();
-    __shared__ float sacc[STATS ? STAT_NW : 1][9][BX * CPL];  // per-thread statistics slots
+    constexpr int NW = block_warps<CPL, STATS>();
+    __shared__ float sacc[STATS ? NW : 1][9][BX * CPL];  // per-thread statistics slots
     const int nx = a.nx, ny = a.ny;
     const int lane = threadIdx.x, wi = threadIdx.y;
-    const int x0 = BX * CPL * (STAT_NW * blockIdx.x + wi);
-    const int y = YEDGE ? (blockIdx.y == 0 ? 0 : ny - 1) : blockIdx.y + 1;
+    const int y = ROWS == INNER ? blockIdx.y + 1 : blockIdx.y * a.row_step;
+    const int x0 = BX * CPL * (STATS ? blockIdx.x : blockDim.y * blockIdx.x + wi);
     const long long t = a.ctl->t[a.parity];
     const bool do_check = a.check_every > 0 && ((t + 1) % a.check_every) == 0;
+    const int zc = STATS ? a.stat_group : a.tile_zc;
+    const int zb = blockIdx.z * zc + (STATS ? wi : 0), ze = min((int)(blockIdx.z + 1) * zc, a.nz), zs = STATS ? NW : 1;
     if (STATS) {
 #pragma unroll
         for (int q = 0; q < 9; ++q)
 #pragma unroll
             for (int j = 0; j < CPL; ++j) sacc[wi][q][CPL * lane + j] = 0.f;
     }
-    const int zb = STATS ? blockIdx.z * STAT_GROUP : 0;
-    const float sdr = vec_loop<S, CPL, REG, FORCE, STATS, YEDGE, SP, H16, MODE, SR>(
-        a, sacc, x0, y, zb, STATS ? min(zb + STAT_GROUP, a.nz) : a.nz, 1);
+    float sdr;
+    if (ROWS == ANY && (y == 0 || y == ny - 1))
+        sdr = vec_loop<S, CPL, REG, FORCE, STATS, true, SP, H16, MODE, SR>(a, sacc, x0, y, zb, ze, zs);
+    else
+        sdr = vec_loop<S, CPL, REG, FORCE, STATS, false, SP, H16, MODE, SR>(a, sacc, x0, y, zb, ze, zs);
     if (STATS) {
-        // each thread wrote only its own slots: no barrier
+        __syncthreads();
         const size_t m = (size_t)nx * ny;
-        float *part = a.stat_part + (size_t)blockIdx.z * 9 * m;
+        float *part = a.stat_part + (size_t)blockIdx.z * 9 * m + (size_t)y * nx + x0;
+        for (int e = wi * BX + lane; e < 9 * BX * CPL; e += NW * BX) {
+            const int q = e / (BX * CPL), c = e % (BX * CPL);
+            float v = sacc[0][q][c];
 #pragma unroll
-        for (int j = 0; j < CPL; ++j) {
-            const int xc = x0 + CPL * lane + j;
-            if (xc >= nx) continue;
-            const size_t xy = (size_t)y * nx + xc;
-#pragma unroll
-            for (int q = 0; q < 9; ++q) part[q * m + xy] = sacc[wi][q][CPL * lane + j];
+            for (int k = 1; k < NW; ++k) v += sacc[k][q][c];
+            if (x0 + c < nx) part[q * m + c] = v;
         }
     }
-    if (do_check) mass_finish<BX * STAT_NW>(a, sdr);
-    if (YEDGE && a.bump_t && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && lane == 0 && wi == 0)
-        a.ctl->t[a.parity ^ 1] = t + 1;
-}
-
-// Plain-step vector kernel, tiled in z: block (x chunk, row, z chunk of
-// a.tile_zc planes, or of a.tile_wall_zc planes for the wall rows).  Many
-// short blocks instead of one block per z column keep the last wave of the
-// grid small.  LAYOUT 0: 8 warps on one 64-cell x chunk, warp w taking the
-// planes w, w + 8, ... of the chunk; LAYOUT 1: 4 warps on 4 consecutive x
-// chunks (256 cells), all walking the chunk's planes together (binary16
-// quads: one warp on one 128-cell chunk).  The regularized unforced interior variants fit 64
-// registers with pairs (32 warps per SM) and 96 with quads (20 warps per SM:
-// with 8-byte row pieces those warps keep as many bytes in flight as FP32);
-// BGK, forced and wall-row ones get 80 with pairs (24 warps per SM) and 128
-// with quads.
-template <int LAYOUT, bool LEAN, int CPL = 2>
-struct ZcShape {
-    static constexpr int NW = LAYOUT == 0 ? BZ : chunk_warps<CPL>();  // warps per block
-    static constexpr int MINB = (CPL == 4 ? (LEAN ? 20 : 16) : (LEAN ? 32 : 24)) / NW;  // resident blocks per SM
-};
-
-template <typename S, int CPL, bool REG, bool FORCE, int LAYOUT, bool YEDGE, bool SP, bool H16, int MODE, bool SR>
-__global__ void __launch_bounds__(BX *ZcShape<LAYOUT, REG && !FORCE && !YEDGE, CPL>::NW,
-                                  ZcShape<LAYOUT, REG && !FORCE && !YEDGE, CPL>::MINB)
-    lbm_vec_zc_kernel(const StepArgs a)
-{
-    constexpr int NW = ZcShape<LAYOUT, REG && !FORCE && !YEDGE, CPL>::NW;
-    const int wi = threadIdx.y;
-    const int y = YEDGE ? (blockIdx.y == 0 ? 0 : a.ny - 1) : blockIdx.y + 1;
-    const int zc0 = YEDGE ? a.tile_wall_zc : a.tile_zc;
-    const int zc = zc0 > 0 ? zc0 : a.nz;
-    const int zb = blockIdx.z * zc, ze = min(zb + zc, a.nz);
-    const long long t = a.ctl->t[a.parity];
-    const bool do_check = a.check_every > 0 && ((t + 1) % a.check_every) == 0;
-    float sdr;
-    if (LAYOUT == 0)
-        sdr = vec_loop<S, CPL, REG, FORCE, false, YEDGE, SP, H16, MODE, SR>(a, nullptr, BX * CPL * blockIdx.x, y, zb + wi, ze, NW);
-    else
-        sdr = vec_loop<S, CPL, REG, FORCE, false, YEDGE, SP, H16, MODE, SR>(a, nullptr, BX * CPL * (NW * blockIdx.x + wi), y, zb, ze, 1);
     if (do_check) mass_finish<BX * NW>(a, sdr);
-    if (YEDGE && a.bump_t && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0 && wi == 0)
+    if (ROWS != INNER && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && lane == 0 && wi == 0)
         a.ctl->t[a.parity ^ 1] = t + 1;
 }
 
@@ -912,31 +894,20 @@ __global__ void __launch_bounds__(BX *BZ, 2) lbm_edge_kernel(const StepArgs a)
     }
     const long long t = a.ctl->t[a.parity];
     step_column<S, REG, FORCE, true, SP, SR>(a, bx, y);
-    if (a.bump_t && b == 0 && threadIdx.x == 0 && threadIdx.y == 0) a.ctl->t[a.parity ^ 1] = t + 1;
+    if (b == 0 && threadIdx.x == 0 && threadIdx.y == 0) a.ctl->t[a.parity ^ 1] = t + 1;
 }
 
-// How a pass covers the lattice.
-//  vector split: vector kernel on rows 1..ny-2 and on rows {0, ny-1} (all x,
-//                inlet/outlet nodes included);
-//  scalar split: interior kernel (one cell per thread) on the
-//                32-wide chunks [1, nxc-1) of rows 1..ny-2, edge kernel on the
-//                rest.
+// How a pass of one cell per thread covers the lattice: interior kernel on the
+// 32-wide chunks [il, ir) of rows 1..ny-2, edge kernel on the rest.
 struct Split {
-    bool vec;
-    int il, ir, gx, gy;        // scalar split interior
+    int il, ir, gx, gy;
     int n_edge;
 };
 
-static Split split_of(const StepArgs &a, int cpl)
+static Split split_of(const StepArgs &a)
 {
     Split sp{};
-    const int nx = a.nx, ny = a.ny, nz = a.nz;
-    const int nxc = (nx + BX - 1) / BX;
-    // the in-place scheme exists for the vector kernels only (the host checks
-    // its lattice conditions), so it ignores the interior override
-    sp.vec = (a.aa || a.interior == 0 || a.interior == 2) && nx % cpl == 0 && nx >= 2 * cpl &&
-             19.0 * nx * ny * nz < 4294967296.0 && (a.bc_x != 0 || nx >= 3);
-    if (sp.vec) return sp;
+    const int nxc = (a.nx + BX - 1) / BX, ny = a.ny;
     if (nxc >= 3 && ny >= 3) {
         sp.il = 1;
         sp.ir = nxc - 1;
@@ -948,113 +919,92 @@ static Split split_of(const StepArgs &a, int cpl)
     return sp;
 }
 
-// Vector split of one pass in streaming mode MODE.
+template <typename S, int CPL, bool REG, bool FORCE, bool SP, int MODE, bool SR, int ROWS>
+static void launch_rows(const StepArgs &a, bool stats, dim3 grid, int nw, cudaStream_t s)
+{
+    // binary16 in an inlet/outlet lattice: x halo by 2-byte loads
+    // (the local in-place step reads no x neighbour)
+    constexpr bool H = sizeof(S) == 2 && MODE != AA_LOCAL;
+    const bool h16 = H && a.bc_x == 0;
+    const dim3 block(BX, nw);
+    if (stats && h16) lbm_vec_kernel<S, CPL, REG, FORCE, true, ROWS, SP, H, MODE, SR><<<grid, block, 0, s>>>(a);
+    else if (stats) lbm_vec_kernel<S, CPL, REG, FORCE, true, ROWS, SP, false, MODE, SR><<<grid, block, 0, s>>>(a);
+    else if (h16) lbm_vec_kernel<S, CPL, REG, FORCE, false, ROWS, SP, H, MODE, SR><<<grid, block, 0, s>>>(a);
+    else lbm_vec_kernel<S, CPL, REG, FORCE, false, ROWS, SP, false, MODE, SR><<<grid, block, 0, s>>>(a);
+}
+
+// The pass in streaming mode MODE: the inner rows on `s` and the wall rows on
+// `side` beside them, or, on a lattice that does not fill the GPU, all rows in
+// one launch.
 template <typename S, int CPL, bool REG, bool FORCE, bool SP, int MODE, bool SR>
 static void launch_vec(StepArgs a, bool stats, cudaStream_t s, cudaStream_t side)
 {
-    const dim3 block(BX, BZ);
-    {
-        constexpr int cpl = CPL;
-        const int nx = a.nx, ny = a.ny;
-        const int nxv = (nx + BX * cpl - 1) / (BX * cpl);  // vector chunks per row
-        const int rows_in = ny > 2 ? ny - 2 : 0, rows_edge = ny >= 2 ? 2 : 1;
-        const int nz = a.nz;
-        // grids: sampling steps take fixed groups of STAT_GROUP planes (their
-        // sums go to a.stat_part and are reduced after the pass); plain steps
-        // take the tile's z chunks
-        const int groups = (nz + STAT_GROUP - 1) / STAT_GROUP;
-        constexpr int STAT_NW = chunk_warps<CPL>();
-        const int nxs = (nx + BX * cpl * STAT_NW - 1) / (BX * cpl * STAT_NW);  // sampling blocks along x
-        dim3 gi(nxs, rows_in, groups), ge(nxs, rows_edge, groups);
-        const dim3 bs(BX, STAT_NW);
-        dim3 bi = block;
-        if (!stats) {
-            const int zc = a.tile_zc > 0 ? a.tile_zc : nz, wzc = a.tile_wall_zc > 0 ? a.tile_wall_zc : nz;
-            if (a.tile_layout == 1) {
-                constexpr int W = ZcShape<1, true, CPL>::NW;
-                gi = dim3((nx + BX * cpl * W - 1) / (BX * cpl * W), rows_in, (nz + zc - 1) / zc);
-                bi = dim3(BX, W);
-            } else {
-                gi = dim3(nxv, rows_in, (nz + zc - 1) / zc);
-            }
-            ge = dim3(nxv, rows_edge, (nz + wzc - 1) / wzc);
-        }
-        const int n_in = rows_in > 0 ? (int)(gi.x * gi.y * gi.z) : 0;
-        const int n_edge = (int)(ge.x * ge.y * ge.z);
-        // binary16 in an inlet/outlet lattice: x halo by 2-byte loads
-        // (the local in-place step reads no x neighbour)
-        constexpr bool H = sizeof(S) == 2 && MODE != AA_LOCAL;
-        const bool h16 = H && a.bc_x == 0;
-        a.total_blocks = (unsigned)(n_in + n_edge);
-        StepArgs ai = a, ae = a;
-        ai.slot_base = 0;
-        ae.slot_base = n_in;
-        ae.bump_t = 1;
-        if (n_in > 0) {
-            if (stats && h16) lbm_vec_kernel<S, CPL, REG, FORCE, true, false, SP, H, MODE, SR><<<gi, bs, 0, s>>>(ai);
-            else if (stats) lbm_vec_kernel<S, CPL, REG, FORCE, true, false, SP, false, MODE, SR><<<gi, bs, 0, s>>>(ai);
-            else if (h16 && a.tile_layout == 1) lbm_vec_zc_kernel<S, CPL, REG, FORCE, 1, false, SP, H, MODE, SR><<<gi, bi, 0, s>>>(ai);
-            else if (h16) lbm_vec_zc_kernel<S, CPL, REG, FORCE, 0, false, SP, H, MODE, SR><<<gi, bi, 0, s>>>(ai);
-            else if (a.tile_layout == 1) lbm_vec_zc_kernel<S, CPL, REG, FORCE, 1, false, SP, false, MODE, SR><<<gi, bi, 0, s>>>(ai);
-            else lbm_vec_zc_kernel<S, CPL, REG, FORCE, 0, false, SP, false, MODE, SR><<<gi, bi, 0, s>>>(ai);
-        }
-        if (stats && h16) lbm_vec_kernel<S, CPL, REG, FORCE, true, true, SP, H, MODE, SR><<<ge, bs, 0, side>>>(ae);
-        else if (stats) lbm_vec_kernel<S, CPL, REG, FORCE, true, true, SP, false, MODE, SR><<<ge, bs, 0, side>>>(ae);
-        else if (h16) lbm_vec_zc_kernel<S, CPL, REG, FORCE, 0, true, SP, H, MODE, SR><<<ge, block, 0, side>>>(ae);
-        else lbm_vec_zc_kernel<S, CPL, REG, FORCE, 0, true, SP, false, MODE, SR><<<ge, block, 0, side>>>(ae);
+    const int chunks = (a.nx + BX * CPL - 1) / (BX * CPL);
+    int nw = block_warps<CPL, false>();
+    // chunks per block: as many as leave the fewest warps idle
+    for (int k = nw - 1; k > 0; --k)
+        if ((chunks + k - 1) / k * k < (chunks + nw - 1) / nw * nw) nw = k;
+    const bool one = one_launch(a, CPL);
+    StepArgs w = a;
+    a.tile_zc = stats ? a.stat_group : run_planes(a, CPL, a.tile_zc, sizeof(S), false);
+    w.tile_zc = stats ? a.stat_group : run_planes(a, CPL, a.tile_wall_zc, sizeof(S), true);
+    if (stats) nw = STAT_WARPS;
+    auto grid_of = [&](int rows, int zc) {
+        return dim3(stats ? chunks : (chunks + nw - 1) / nw, rows, (a.nz + zc - 1) / zc);
+    };
+    const dim3 gi = grid_of(one ? a.ny : a.ny - 2, a.tile_zc), gw = grid_of(2, w.tile_zc);
+    const unsigned ni = gi.x * gi.y * gi.z, nwall = one ? 0 : gw.x * gw.y * gw.z;
+    a.slot_base = 0;
+    w.slot_base = ni;
+    a.total_blocks = w.total_blocks = ni + nwall;
+    a.row_step = 1;
+    w.row_step = a.ny - 1;
+    if (one) {
+        launch_rows<S, CPL, REG, FORCE, SP, MODE, SR, ANY>(a, stats, gi, nw, s);
+    } else {
+        launch_rows<S, CPL, REG, FORCE, SP, MODE, SR, INNER>(a, stats, gi, nw, s);
+        launch_rows<S, CPL, REG, FORCE, SP, MODE, SR, ANY>(w, stats, gw, nw, side);
     }
 }
 
 // Returns true when the pass left z-group statistics in a.stat_part.
-template <typename S, bool REG, bool FORCE, bool SP, bool SR>
-static bool launch_forced(StepArgs a, const Split &sp, bool stats, cudaStream_t s,
-                          cudaStream_t side)
+template <typename S, int CPL, bool REG, bool FORCE, bool SP, bool SR>
+static bool launch_forced(StepArgs a, bool stats, cudaStream_t s, cudaStream_t side)
 {
-    const dim3 block(BX, BZ);
-    if (sp.vec) {
-        // binary16, regularized unforced, rows of whole quads: four cells per lane
-        constexpr bool QUAD = sizeof(S) == 2 && REG && !FORCE;
+    if (CPL == 4 || vector_fits(a)) {
         // in place: steps with even index shift, steps with odd index stay local
-        const int mode = !a.aa ? PULL : (a.parity == 0 ? AA_SHIFT : AA_LOCAL);
-        if (QUAD && quads_fit(a.nx)) {
-            if constexpr (QUAD) {
-                if (mode == PULL) launch_vec<S, 4, REG, FORCE, SP, PULL, SR>(a, stats, s, side);
-                else if (mode == AA_SHIFT) launch_vec<S, 4, REG, FORCE, SP, AA_SHIFT, SR>(a, stats, s, side);
-                else launch_vec<S, 4, REG, FORCE, SP, AA_LOCAL, SR>(a, stats, s, side);
-            }
-        } else {
-            if (mode == PULL) launch_vec<S, 2, REG, FORCE, SP, PULL, SR>(a, stats, s, side);
-            else if (mode == AA_SHIFT) launch_vec<S, 2, REG, FORCE, SP, AA_SHIFT, SR>(a, stats, s, side);
-            else launch_vec<S, 2, REG, FORCE, SP, AA_LOCAL, SR>(a, stats, s, side);
-        }
+        if (!a.aa) launch_vec<S, CPL, REG, FORCE, SP, PULL, SR>(a, stats, s, side);
+        else if (a.parity == 0) launch_vec<S, CPL, REG, FORCE, SP, AA_SHIFT, SR>(a, stats, s, side);
+        else launch_vec<S, CPL, REG, FORCE, SP, AA_LOCAL, SR>(a, stats, s, side);
         return stats;
     }
-    const int n_in = sp.gy > 0 ? sp.gx * sp.gy : 0;
-    a.il = sp.il;
-    a.ir = sp.ir;
-    a.total_blocks = (unsigned)(n_in + sp.n_edge);
-    StepArgs ai = a, ae = a;
-    ai.slot_base = 0;
-    ae.slot_base = n_in;
-    ae.bump_t = 1;
-    lbm_edge_kernel<S, REG, FORCE, SP, SR><<<sp.n_edge, block, 0, side>>>(ae);
-    if (n_in > 0) {
-        lbm_step_kernel<S, REG, FORCE, SP, SR><<<dim3(sp.gx, sp.gy), block, 0, s>>>(ai);
+    if constexpr (CPL == 2) {
+        const dim3 block(BX, BZ);
+        const Split sp = split_of(a);
+        const int n_in = sp.gy > 0 ? sp.gx * sp.gy : 0;
+        a.il = sp.il;
+        a.ir = sp.ir;
+        a.total_blocks = (unsigned)(n_in + sp.n_edge);
+        StepArgs ai = a, ae = a;
+        ai.slot_base = 0;
+        ae.slot_base = n_in;
+        lbm_edge_kernel<S, REG, FORCE, SP, SR><<<sp.n_edge, block, 0, side>>>(ae);
+        if (n_in > 0) lbm_step_kernel<S, REG, FORCE, SP, SR><<<dim3(sp.gx, sp.gy), block, 0, s>>>(ai);
     }
     return false;
 }
 
-// SR: binary16 stores by stochastic rounding (S = __half only)
-template <typename S, bool REG, bool SR = false>
-bool launch_typed(const StepArgs &a0, bool stats, cudaStream_t s, cudaStream_t side)
+// CPL: cells per lane of the vector kernels (2, with the one-cell-per-thread
+// kernels, or 4); SR: binary16 stores by stochastic rounding (S = __half only)
+template <typename S, int CPL, bool REG, bool SR = false>
+bool launch_typed(const StepArgs &a, bool stats, cudaStream_t s, cudaStream_t side)
 {
-    const Split sp = split_of(a0, 2);
-    StepArgs a = a0;
-    a.bump_t = 0;
     // the sponge is only compiled for unforced lattices (the host refuses a sponge with a force)
-    if (a.spf) return launch_forced<S, REG, false, true, SR>(a, sp, stats, s, side);
-    if (a.has_force) return launch_forced<S, REG, true, false, SR>(a, sp, stats, s, side);
-    return launch_forced<S, REG, false, false, SR>(a, sp, stats, s, side);
+    if (a.spf) return launch_forced<S, CPL, REG, false, true, SR>(a, stats, s, side);
+    if constexpr (CPL == 2) {
+        if (a.has_force) return launch_forced<S, CPL, REG, true, false, SR>(a, stats, s, side);
+    }
+    return launch_forced<S, CPL, REG, false, false, SR>(a, stats, s, side);
 }
 
 }  // namespace stg
