@@ -97,7 +97,7 @@ struct MassArgs {
 // the host tracks t and decides.
 cudaError_t launch_step(const StepArgs &a, int storage, int collision, bool stats,
                         cudaStream_t s, cudaStream_t side, cudaEvent_t fork, cudaEvent_t join);
-// binary16 regularized unforced lattices take quads (four cells per lane)
+// binary16 lattices take quads (four cells per lane)
 // when the rows split into whole quads
 inline bool quads_fit(int nx) { return nx % 4 == 0 && nx >= 8; }
 // Lattices of the vector kernels (the others take one cell per thread): rows of
@@ -113,7 +113,7 @@ inline bool vector_fits(const StepArgs &a)
 bool one_launch(const StepArgs &a, int cpl);
 int run_planes(const StepArgs &a, int cpl, int tile_zc, int elem, bool walls);
 // cells per lane of the vector kernels
-int lane_cells(const StepArgs &a, int storage, int collision);
+int lane_cells(const StepArgs &a, int storage);
 cudaError_t launch_inlet(const InletArgs &a, cudaStream_t s);
 // FP64 Cholesky factor of the lattice-unit Reynolds stress per inlet node (setup)
 cudaError_t launch_setup_nodes(int ny, const double *R6, float *a6, cudaStream_t s);

@@ -1,15 +1,17 @@
-// The regularized collision of lbm_cell.cuh (collide_sd, unforced) for the
-// two cells a lane of the vector kernels holds, computed together: every
-// float2 operation below acts on both cells (.x the lane's first cell, .y its
-// second) through the packed FP32 instructions of sm_100 and later
-// (add/sub/mul/fma .f32x2: one instruction, two roundings, each the IEEE
-// result of the scalar operation).  Only the reciprocals and square roots go
-// cell by cell.  The update is collide_sd's
-//     g*_i = w_i [a0 + c_i.B + c_i.A.c_i]
+// The collisions of lbm_cell.cuh (collide_sd) for two cells of a lane of the
+// vector kernels, computed together: every float2 operation below acts on both
+// cells (.x the first, .y the second) through the packed FP32 instructions of
+// sm_100 and later (add/sub/mul/fma .f32x2: one instruction, two roundings, each
+// the IEEE result of the scalar operation).  Only the reciprocals and square
+// roots go cell by cell.  The update is collide_sd's
+//     g*_i = K g_i + w_i [a0 + c_i.B + c_i.A.c_i]
 // written with B = 3 b and A = 4.5 A' so that the factors 3 and 4.5 join the
 // weights in the output stage:
-//     a0 = drho - 1.5 (rho u.u + km tr Pi_neq),  b = rho u,
-//     A' = rho u u + km Pi_neq,                  km = 1 - 1/tau_eff.
+//   regularized: a0 = drho - 1.5 (rho u.u + km tr Pi_neq) - 3 kf u.F,  K = 0,
+//                b = rho u + (kf - km/2) F,  A' = rho u u + km Pi_neq + kf (u F + F u)
+//   BGK:         a0 = om (drho - 1.5 rho u.u) - 3 kf u.F,  K = km,
+//                b = om rho u + kf F,  A' = om rho u u + kf (u F + F u)
+// with om = 1/tau_eff, km = 1 - om and, with a force, kf = 1 - om/2 (else 0).
 #pragma once
 
 #include "d3q19.cuh"
@@ -132,17 +134,21 @@ __device__ __forceinline__ PairMoments pair_moments(Pop2 pop)
 }
 
 // Smagorinsky relaxation (eq. tau_eff, with the sponge factor nuf of eq.
-// sponge_visco when SP) and regularized collision of the pair; out(i, r)
-// receives the result r of population i (both cells) in the order
-// i = 0, 1, ..., 18.  Returns the density excess and velocity per cell.
-template <bool SP, typename Out>
-__device__ __forceinline__ void collide_pair(const PairMoments &m, float tau0, float kq, float2 nuf, Out out,
-                                             float2 &drho_o, float2 &ux_o, float2 &uy_o, float2 &uz_o)
+// sponge_visco when SP) and collision of the pair; pop(i) gives population i of
+// both cells (read again by the BGK collision), out(i, r) receives the result r
+// of population i (both cells) in the order i = 0, 1, ..., 18.  Returns the
+// density excess and velocity per cell.
+template <bool REG, bool FORCE, bool SP, typename Pop2, typename Out>
+__device__ __forceinline__ void collide_pair(const PairMoments &m, Pop2 pop, float tau0, float kq, float2 nuf, float Fx,
+                                             float Fy, float Fz, Out out, float2 &drho_o, float2 &ux_o, float2 &uy_o,
+                                             float2 &uz_o)
 {
     const float2 drho = m.drho;
     const float2 rho = p_add(drho, p_k(1.0f));
     const float2 irho = make_float2(1.0f / rho.x, 1.0f / rho.y);
-    const float2 ux = p_mul(m.jx, irho), uy = p_mul(m.jy, irho), uz = p_mul(m.jz, irho);
+    const float2 ux = p_mul(FORCE ? p_add(m.jx, p_k(0.5f * Fx)) : m.jx, irho);
+    const float2 uy = p_mul(FORCE ? p_add(m.jy, p_k(0.5f * Fy)) : m.jy, irho);
+    const float2 uz = p_mul(FORCE ? p_add(m.jz, p_k(0.5f * Fz)) : m.jz, irho);
     // rho u u and Pi_neq = sum c c g - drho/3 I - rho u u
     const float2 rux = p_mul(rho, ux), ruy = p_mul(rho, uy), ruz = p_mul(rho, uz);
     const float2 Pxx = p_mul(rux, ux), Pyy = p_mul(ruy, uy), Pzz = p_mul(ruz, uz);
@@ -160,53 +166,80 @@ __device__ __forceinline__ void collide_pair(const PairMoments &m, float tau0, f
     const float2 rad = p_fma(p_k(kq), p_mul(qh, p_mul(irho, irho)), p_k(tau0 * tau0));
     float2 tau = p_fma(p_k(0.5f), make_float2(sqrtf(rad.x), sqrtf(rad.y)), p_k(0.5f * tau0));
     if (SP) tau = p_fma(nuf, p_sub(tau, p_k(0.5f)), p_k(0.5f));
-    const float2 km = p_sub(p_k(1.0f), make_float2(1.0f / tau.x, 1.0f / tau.y));
+    const float2 om = make_float2(1.0f / tau.x, 1.0f / tau.y);
+    const float2 km = p_sub(p_k(1.0f), om);
     const float2 uu = p_fma(uz, uz, p_fma(uy, uy, p_mul(ux, ux)));
-    const float2 a0 = p_fma(p_k(-1.5f), p_fma(km, p_add(p_add(nxx, nyy), nzz), p_mul(rho, uu)), drho);
-    const float2 Axx = p_fma(km, nxx, Pxx), Ayy = p_fma(km, nyy, Pyy), Azz = p_fma(km, nzz, Pzz);
-    const float2 Axy = p_fma(km, nxy, Pxy), Axz = p_fma(km, nxz, Pxz), Ayz = p_fma(km, nyz, Pyz);
+    float2 a0, bx, by, bz, Axx, Ayy, Azz, Axy, Axz, Ayz;
+    if (REG) {
+        a0 = p_fma(p_k(-1.5f), p_fma(km, p_add(p_add(nxx, nyy), nzz), p_mul(rho, uu)), drho);
+        bx = rux, by = ruy, bz = ruz;
+        Axx = p_fma(km, nxx, Pxx), Ayy = p_fma(km, nyy, Pyy), Azz = p_fma(km, nzz, Pzz);
+        Axy = p_fma(km, nxy, Pxy), Axz = p_fma(km, nxz, Pxz), Ayz = p_fma(km, nyz, Pyz);
+    } else {
+        a0 = p_mul(om, p_fma(p_k(-1.5f), p_mul(rho, uu), drho));
+        bx = p_mul(om, rux), by = p_mul(om, ruy), bz = p_mul(om, ruz);
+        Axx = p_mul(om, Pxx), Ayy = p_mul(om, Pyy), Azz = p_mul(om, Pzz);
+        Axy = p_mul(om, Pxy), Axz = p_mul(om, Pxz), Ayz = p_mul(om, Pyz);
+    }
+    if (FORCE) {
+        const float2 kf = p_fma(p_k(-0.5f), om, p_k(1.0f));  // Guo prefactor
+        const float2 uF = p_fma(uz, p_k(Fz), p_fma(uy, p_k(Fy), p_mul(ux, p_k(Fx))));
+        a0 = p_fma(p_mul(p_k(-3.0f), kf), uF, a0);
+        // regularized: the first-order neq part -F/2 is kept
+        const float2 kb = REG ? p_fma(p_k(-0.5f), km, kf) : kf;
+        bx = p_fma(kb, p_k(Fx), bx), by = p_fma(kb, p_k(Fy), by), bz = p_fma(kb, p_k(Fz), bz);
+        const float2 kx = p_mul(kf, p_k(Fx)), ky = p_mul(kf, p_k(Fy)), kz = p_mul(kf, p_k(Fz));
+        Axx = p_fma(p_add(kx, kx), ux, Axx), Ayy = p_fma(p_add(ky, ky), uy, Ayy), Azz = p_fma(p_add(kz, kz), uz, Azz);
+        Axy = p_fma(kx, uy, p_fma(ky, ux, Axy));
+        Axz = p_fma(kx, uz, p_fma(kz, ux, Axz));
+        Ayz = p_fma(ky, uz, p_fma(kz, uy, Ayz));
+    }
+    auto put = [&](int i, float2 v) {
+        if (REG) out(i, v);
+        else out(i, p_fma(km, pop(i), v));
+    };
     constexpr float W0 = 1.0f / 3.0f, W1 = 1.0f / 18.0f, W2 = 1.0f / 36.0f;
     // rest population
-    out(0, p_mul(p_k(W0), a0));
+    put(0, p_mul(p_k(W0), a0));
     // axis pairs (1,2) +-x, (3,4) +-y, (5,6) +-z
     {
         const float2 w1a0 = p_mul(p_k(W1), a0);
-        const float2 ex = p_fma(p_k(4.5f * W1), Axx, w1a0), ox = p_mul(p_k(3.0f * W1), rux);
-        out(1, p_add(ex, ox));
-        out(2, p_sub(ex, ox));
-        const float2 ey = p_fma(p_k(4.5f * W1), Ayy, w1a0), oy = p_mul(p_k(3.0f * W1), ruy);
-        out(3, p_add(ey, oy));
-        out(4, p_sub(ey, oy));
-        const float2 ez = p_fma(p_k(4.5f * W1), Azz, w1a0), oz = p_mul(p_k(3.0f * W1), ruz);
-        out(5, p_add(ez, oz));
-        out(6, p_sub(ez, oz));
+        const float2 ex = p_fma(p_k(4.5f * W1), Axx, w1a0), ox = p_mul(p_k(3.0f * W1), bx);
+        put(1, p_add(ex, ox));
+        put(2, p_sub(ex, ox));
+        const float2 ey = p_fma(p_k(4.5f * W1), Ayy, w1a0), oy = p_mul(p_k(3.0f * W1), by);
+        put(3, p_add(ey, oy));
+        put(4, p_sub(ey, oy));
+        const float2 ez = p_fma(p_k(4.5f * W1), Azz, w1a0), oz = p_mul(p_k(3.0f * W1), bz);
+        put(5, p_add(ez, oz));
+        put(6, p_sub(ez, oz));
     }
     // edge pairs: (7,8) +-(1,1,0), (9,10) +-(1,-1,0), (11,12) +-(1,0,1), (13,14) +-(1,0,-1),
     //             (15,16) +-(0,1,1), (17,18) +-(0,1,-1)
     {
         const float2 w2a0 = p_mul(p_k(W2), a0);
-        const float2 bx = p_mul(p_k(3.0f * W2), rux), by = p_mul(p_k(3.0f * W2), ruy), bz = p_mul(p_k(3.0f * W2), ruz);
+        const float2 ex = p_mul(p_k(3.0f * W2), bx), ey = p_mul(p_k(3.0f * W2), by), ez = p_mul(p_k(3.0f * W2), bz);
         const float2 sxy = p_fma(p_k(4.5f * W2), p_add(Axx, Ayy), w2a0), txy = p_mul(p_k(9.0f * W2), Axy);
-        const float2 e7 = p_add(sxy, txy), o7 = p_add(bx, by);
-        out(7, p_add(e7, o7));
-        out(8, p_sub(e7, o7));
-        const float2 e9 = p_sub(sxy, txy), o9 = p_sub(bx, by);
-        out(9, p_add(e9, o9));
-        out(10, p_sub(e9, o9));
+        const float2 e7 = p_add(sxy, txy), o7 = p_add(ex, ey);
+        put(7, p_add(e7, o7));
+        put(8, p_sub(e7, o7));
+        const float2 e9 = p_sub(sxy, txy), o9 = p_sub(ex, ey);
+        put(9, p_add(e9, o9));
+        put(10, p_sub(e9, o9));
         const float2 sxz = p_fma(p_k(4.5f * W2), p_add(Axx, Azz), w2a0), txz = p_mul(p_k(9.0f * W2), Axz);
-        const float2 e11 = p_add(sxz, txz), o11 = p_add(bx, bz);
-        out(11, p_add(e11, o11));
-        out(12, p_sub(e11, o11));
-        const float2 e13 = p_sub(sxz, txz), o13 = p_sub(bx, bz);
-        out(13, p_add(e13, o13));
-        out(14, p_sub(e13, o13));
+        const float2 e11 = p_add(sxz, txz), o11 = p_add(ex, ez);
+        put(11, p_add(e11, o11));
+        put(12, p_sub(e11, o11));
+        const float2 e13 = p_sub(sxz, txz), o13 = p_sub(ex, ez);
+        put(13, p_add(e13, o13));
+        put(14, p_sub(e13, o13));
         const float2 syz = p_fma(p_k(4.5f * W2), p_add(Ayy, Azz), w2a0), tyz = p_mul(p_k(9.0f * W2), Ayz);
-        const float2 e15 = p_add(syz, tyz), o15 = p_add(by, bz);
-        out(15, p_add(e15, o15));
-        out(16, p_sub(e15, o15));
-        const float2 e17 = p_sub(syz, tyz), o17 = p_sub(by, bz);
-        out(17, p_add(e17, o17));
-        out(18, p_sub(e17, o17));
+        const float2 e15 = p_add(syz, tyz), o15 = p_add(ey, ez);
+        put(15, p_add(e15, o15));
+        put(16, p_sub(e15, o15));
+        const float2 e17 = p_sub(syz, tyz), o17 = p_sub(ey, ez);
+        put(17, p_add(e17, o17));
+        put(18, p_sub(e17, o17));
     }
     drho_o = drho;
     ux_o = ux;

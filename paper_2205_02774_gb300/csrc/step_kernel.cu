@@ -21,9 +21,11 @@ bool launch_f32_reg(const StepArgs &, bool, cudaStream_t, cudaStream_t),
     launch_f16_reg(const StepArgs &, bool, cudaStream_t, cudaStream_t),
     launch_f16_reg_quad(const StepArgs &, bool, cudaStream_t, cudaStream_t),
     launch_f16_bgk(const StepArgs &, bool, cudaStream_t, cudaStream_t),
+    launch_f16_bgk_quad(const StepArgs &, bool, cudaStream_t, cudaStream_t),
     launch_f16sr_reg(const StepArgs &, bool, cudaStream_t, cudaStream_t),
     launch_f16sr_reg_quad(const StepArgs &, bool, cudaStream_t, cudaStream_t),
-    launch_f16sr_bgk(const StepArgs &, bool, cudaStream_t, cudaStream_t);
+    launch_f16sr_bgk(const StepArgs &, bool, cudaStream_t, cudaStream_t),
+    launch_f16sr_bgk_quad(const StepArgs &, bool, cudaStream_t, cudaStream_t);
 
 int step_grid_blocks(int nx, int ny, int nz)
 {
@@ -45,9 +47,9 @@ int stat_group(int nx, int ny, int nz)
     return g;
 }
 
-int lane_cells(const StepArgs &a, int storage, int collision)
+int lane_cells(const StepArgs &a, int storage)
 {
-    return storage != 0 && collision == 0 && !a.has_force && quads_fit(a.nx) && vector_fits(a) ? 4 : 2;
+    return storage != 0 && quads_fit(a.nx) && vector_fits(a) ? 4 : 2;
 }
 
 // Items: one x chunk (32 cpl cells) of one row and plane each, of all lattices
@@ -121,7 +123,7 @@ cudaError_t launch_step(const StepArgs &a, int storage, int collision, bool stat
                         cudaStream_t s, cudaStream_t side, cudaEvent_t fork, cudaEvent_t join)
 {
     cudaError_t e = cudaSuccess;
-    const int cpl = lane_cells(a, storage, collision);
+    const int cpl = lane_cells(a, storage);
     const bool one = vector_fits(a) && one_launch(a, cpl);
     const bool forked = !one && side != nullptr && fork != nullptr && join != nullptr;
     if (forked) {
@@ -131,8 +133,8 @@ cudaError_t launch_step(const StepArgs &a, int storage, int collision, bool stat
     cudaStream_t es = forked ? side : s;
     // by storage and collision, two and four cells per lane
     static constexpr Pass passes[3][2][2] = {{{launch_f32_reg, nullptr}, {launch_f32_bgk, nullptr}},
-                                             {{launch_f16_reg, launch_f16_reg_quad}, {launch_f16_bgk, nullptr}},
-                                             {{launch_f16sr_reg, launch_f16sr_reg_quad}, {launch_f16sr_bgk, nullptr}}};
+                                             {{launch_f16_reg, launch_f16_reg_quad}, {launch_f16_bgk, launch_f16_bgk_quad}},
+                                             {{launch_f16sr_reg, launch_f16sr_reg_quad}, {launch_f16sr_bgk, launch_f16sr_bgk_quad}}};
     const bool reduce = passes[storage][collision][cpl == 4](a, stats, s, es);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (forked) {

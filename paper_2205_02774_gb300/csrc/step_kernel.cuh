@@ -524,13 +524,12 @@ __device__ __forceinline__ float vec_loop(const StepArgs &a, float (*sacc)[9][BX
     using raw = typename V::raw;
     // binary16, regularized collision: pair sums by mixed-precision adds
     constexpr bool MIXED = REG && sizeof(S) == 2;
-    // binary16, regularized unforced collision: the lane's cells go through
-    // the collision two at a time in packed FP32 (lbm_pair.cuh) wherever the
-    // warp's 32 CPL cells hold no inlet or outlet node; the warps that do, the
-    // other collisions and FP32 storage (whose step is bound by memory either
-    // way) update cell by cell.  A warp's chunk is the same in every kernel and
+    // binary16: the lane's cells go through the collision two at a time in
+    // packed FP32 (lbm_pair.cuh) wherever the warp's 32 CPL cells hold no inlet
+    // or outlet node; the warps that do and FP32 storage (whose step is bound by
+    // memory either way) update cell by cell.  A warp's chunk is the same in every kernel and
     // tile, so each cell always takes the same form.
-    constexpr bool PACKED = REG && !FORCE && sizeof(S) == 2;
+    constexpr bool PACKED = sizeof(S) == 2;
     const int nx = a.nx, ny = a.ny, nz = a.nz;
     const int nxy = nx * ny;
     const int lane = threadIdx.x, wi = threadIdx.y;
@@ -634,9 +633,10 @@ __device__ __forceinline__ float vec_loop(const StepArgs &a, float (*sacc)[9][BX
                 float2 nuf = make_float2(1.0f, 1.0f);
                 if (SP && active) nuf = __ldg(reinterpret_cast<const float2 *>(a.spf + x + 2 * k));
                 const unsigned seed = seed_of(k);
-                const PairMoments m = pair_moments([&](int i) { return V::pair(v[i], k); });
+                auto pop = [&](int i) { return V::pair(v[i], k); };
+                const PairMoments m = pair_moments(pop);
                 float2 drho, ux, uy, uz;
-                collide_pair<SP>(m, tau0, kq, nuf, [&](int i, float2 r) {
+                collide_pair<REG, FORCE, SP>(m, pop, tau0, kq, nuf, Fx, Fy, Fz, [&](int i, float2 r) {
                     if constexpr (SR) V::set_pair_rs(v[i], k, r.x, r.y, sr_bits(seed, i));
                     else V::set_pair(v[i], k, r.x, r.y);
                 }, drho, ux, uy, uz);
@@ -808,16 +808,21 @@ __device__ __forceinline__ float vec_loop(const StepArgs &a, float (*sacc)[9][BX
 // (all rows, or the wall rows alone).
 constexpr int INNER = 0, ANY = 1;
 
-// Warps per block and the occupancy asked for.  The regularized unforced inner
-// rows fit 64 registers with pairs (32 warps per SM) and 96 with binary16 quads
-// (20 warps per SM: with 8-byte row pieces those warps keep as many bytes in
-// flight as FP32); BGK, forced and sampling pairs get 80; sampling quads, and the
-// launches of any rows (the wall rows beside the inner launch, all rows of a lattice too
-// small to fill the GPU) 128, so that they need no stack frame.
+// Warps per block and the occupancy asked for.  The regularized inner rows fit 96
+// registers with binary16 quads (20 warps per SM: with 8-byte row pieces those
+// warps keep as many bytes in flight as FP32) and, unforced, 64 with pairs (32
+// warps per SM); BGK, forced and sampling pairs get 80; BGK and sampling quads 128
+// (BGK FP16-SR on 768x128x192 260 us per step, 274 with the spills of 96 and as
+// pairs), as do the launches of any rows (the wall rows beside the inner launch,
+// all rows of a lattice too small to fill the GPU), so that they need no stack frame.
 template <int CPL, bool STATS>
 constexpr int block_warps() { return STATS ? STAT_WARPS : (CPL == 4 ? 1 : 4); }
-template <int CPL, bool LEAN, bool STATS, int ROWS>
-constexpr int warps_per_sm() { return ROWS != INNER ? 16 : (CPL == 4 ? (STATS ? 16 : 20) : (LEAN && !STATS ? 32 : 24)); }
+template <int CPL, bool REG, bool FORCE, bool STATS, int ROWS>
+constexpr int warps_per_sm()
+{
+    if (ROWS != INNER || (CPL == 4 && (STATS || !REG))) return 16;
+    return CPL == 4 ? 20 : (REG && !FORCE && !STATS ? 32 : 24);
+}
 
 // The vector kernel: block (x chunks, row, run of z planes).
 // Plain steps (STATS false): the warps of a block take x chunks side by side
@@ -830,7 +835,7 @@ constexpr int warps_per_sm() { return ROWS != INNER ? 16 : (CPL == 4 ? (STATS ? 
 // the statistics are deterministic and independent of the launch tile.  H16 as in
 // vec_loop.  STATS is chosen on the host (it knows the step count).
 template <typename S, int CPL, bool REG, bool FORCE, bool STATS, int ROWS, bool SP, bool H16, int MODE, bool SR>
-__global__ void __launch_bounds__(BX *block_warps<CPL, STATS>(), warps_per_sm<CPL, REG && !FORCE, STATS, ROWS>() / block_warps<CPL, STATS>())
+__global__ void __launch_bounds__(BX *block_warps<CPL, STATS>(), warps_per_sm<CPL, REG, FORCE, STATS, ROWS>() / block_warps<CPL, STATS>())
     lbm_vec_kernel(const StepArgs a)
 {
     constexpr int NW = block_warps<CPL, STATS>();
@@ -1001,9 +1006,7 @@ bool launch_typed(const StepArgs &a, bool stats, cudaStream_t s, cudaStream_t si
 {
     // the sponge is only compiled for unforced lattices (the host refuses a sponge with a force)
     if (a.spf) return launch_forced<S, CPL, REG, false, true, SR>(a, stats, s, side);
-    if constexpr (CPL == 2) {
-        if (a.has_force) return launch_forced<S, CPL, REG, true, false, SR>(a, stats, s, side);
-    }
+    if (a.has_force) return launch_forced<S, CPL, REG, true, false, SR>(a, stats, s, side);
     return launch_forced<S, CPL, REG, false, false, SR>(a, stats, s, side);
 }
 
