@@ -18,7 +18,8 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libstglbm.so")
 STEP_TUS = ["step_f32_reg.cu", "step_f32_bgk.cu", "step_f16_reg.cu", "step_f16_reg_quad.cu",
             "step_f16_bgk.cu", "step_f16_bgk_quad.cu", "step_f16sr_reg.cu", "step_f16sr_reg_quad.cu", "step_f16sr_bgk.cu",
-            "step_f16sr_bgk_quad.cu"]
+            "step_f16sr_bgk_quad.cu", "step_f32_reg_row.cu", "step_f32_bgk_row.cu", "step_f16_reg_row.cu",
+            "step_f16_bgk_row.cu", "step_f16sr_reg_row.cu", "step_f16sr_bgk_row.cu"]
 SOURCES = ["capi.cu", "step_kernel.cu", *STEP_TUS, "inlet_kernel.cu", "noalloc.cu", "batch.cu", "serve.cu", "probe.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-I", CSRC, "-I", INCLUDE,

@@ -112,8 +112,9 @@ inline bool vector_fits(const StepArgs &a)
 // rows, and the z planes per run of its launches (step_kernel.cu).
 bool one_launch(const StepArgs &a, int cpl);
 int run_planes(const StepArgs &a, int cpl, int tile_zc, int elem, bool walls);
-// cells per lane of the vector kernels
+// cells per lane of the vector kernels, and whether they lie 32 apart
 int lane_cells(const StepArgs &a, int storage);
+bool row_lanes(const StepArgs &a, int storage);
 cudaError_t launch_inlet(const InletArgs &a, cudaStream_t s);
 // FP64 Cholesky factor of the lattice-unit Reynolds stress per inlet node (setup)
 cudaError_t launch_setup_nodes(int ny, const double *R6, float *a6, cudaStream_t s);

@@ -1,0 +1,14 @@
+// Step kernels of FP32 storage,
+// the plain BGK collision, lanes 32 cells apart (one of the
+// instantiation units of step_kernel.cuh, compiled in parallel).
+#include "step_kernel.cuh"
+
+namespace stg {
+
+bool launch_f32_bgk_row(const StepArgs &a, bool stats, cudaStream_t s, cudaStream_t side)
+{
+    if (lane_cells(a, 0) == 1) return launch_row<float, 1, false>(a, stats, s, side);
+    return launch_row<float, 2, false>(a, stats, s, side);
+}
+
+}  // namespace stg

@@ -14,7 +14,7 @@ namespace stg {
 
 constexpr int BX = 32;
 
-// instantiation units (step_<storage>_<collision>[_quad].cu)
+// instantiation units (step_<storage>_<collision>[_quad|_row].cu)
 using Pass = bool (*)(const StepArgs &a, bool stats, cudaStream_t s, cudaStream_t side);
 bool launch_f32_reg(const StepArgs &, bool, cudaStream_t, cudaStream_t),
     launch_f32_bgk(const StepArgs &, bool, cudaStream_t, cudaStream_t),
@@ -25,11 +25,17 @@ bool launch_f32_reg(const StepArgs &, bool, cudaStream_t, cudaStream_t),
     launch_f16sr_reg(const StepArgs &, bool, cudaStream_t, cudaStream_t),
     launch_f16sr_reg_quad(const StepArgs &, bool, cudaStream_t, cudaStream_t),
     launch_f16sr_bgk(const StepArgs &, bool, cudaStream_t, cudaStream_t),
-    launch_f16sr_bgk_quad(const StepArgs &, bool, cudaStream_t, cudaStream_t);
+    launch_f16sr_bgk_quad(const StepArgs &, bool, cudaStream_t, cudaStream_t),
+    launch_f32_reg_row(const StepArgs &, bool, cudaStream_t, cudaStream_t),
+    launch_f32_bgk_row(const StepArgs &, bool, cudaStream_t, cudaStream_t),
+    launch_f16_reg_row(const StepArgs &, bool, cudaStream_t, cudaStream_t),
+    launch_f16_bgk_row(const StepArgs &, bool, cudaStream_t, cudaStream_t),
+    launch_f16sr_reg_row(const StepArgs &, bool, cudaStream_t, cudaStream_t),
+    launch_f16sr_bgk_row(const StepArgs &, bool, cudaStream_t, cudaStream_t);
 
 int step_grid_blocks(int nx, int ny, int nz)
 {
-    const long long vec = (long long)((nx + 2 * BX - 1) / (2 * BX)) * ny * nz;  // one plane per item
+    const long long vec = (long long)((nx + BX - 1) / BX) * ny * nz;  // one plane and 32 cells per item
     const long long col = (long long)((nx + BX - 1) / BX) * ny;
     return (int)((vec > col ? vec : col) + 2LL * ny + 64);
 }
@@ -47,8 +53,24 @@ int stat_group(int nx, int ny, int nz)
     return g;
 }
 
+// FP32 lattices with fewer than 4 cells per resident lane (32 warps per SM): one
+// cell per lane halves the serial work of a warp (64x32x32 5.3 against 6.2 us per
+// step, 144x24x36 7.0 against 8.1, 240x40x60 15.4 against 18.2, 241x41x61 16.9
+// against 19.3; 325x55x81, just above, 44.1 against 42.3).
+static bool small_row(const StepArgs &a)
+{
+    return std::max<long long>(a.P, a.in_flight) < 4LL * 152 * 32 * 32;
+}
+
+bool row_lanes(const StepArgs &a, int storage)
+{
+    if (a.aa || a.interior != 0 || 19.0 * a.P >= 4294967296.0) return false;
+    return a.nx % 2 != 0 || a.nx < 4 || (storage == 0 && small_row(a));
+}
+
 int lane_cells(const StepArgs &a, int storage)
 {
+    if (row_lanes(a, storage)) return storage != 0 ? 4 : (small_row(a) ? 1 : 2);
     return storage != 0 && quads_fit(a.nx) && vector_fits(a) ? 4 : 2;
 }
 
@@ -124,18 +146,20 @@ cudaError_t launch_step(const StepArgs &a, int storage, int collision, bool stat
 {
     cudaError_t e = cudaSuccess;
     const int cpl = lane_cells(a, storage);
-    const bool one = vector_fits(a) && one_launch(a, cpl);
+    const bool one = (vector_fits(a) || row_lanes(a, storage)) && one_launch(a, cpl);
     const bool forked = !one && side != nullptr && fork != nullptr && join != nullptr;
     if (forked) {
         if ((e = cudaEventRecord(fork, s)) != cudaSuccess) return e;
         if ((e = cudaStreamWaitEvent(side, fork, 0)) != cudaSuccess) return e;
     }
     cudaStream_t es = forked ? side : s;
-    // by storage and collision, two and four cells per lane
-    static constexpr Pass passes[3][2][2] = {{{launch_f32_reg, nullptr}, {launch_f32_bgk, nullptr}},
-                                             {{launch_f16_reg, launch_f16_reg_quad}, {launch_f16_bgk, launch_f16_bgk_quad}},
-                                             {{launch_f16sr_reg, launch_f16sr_reg_quad}, {launch_f16sr_bgk, launch_f16sr_bgk_quad}}};
-    const bool reduce = passes[storage][collision][cpl == 4](a, stats, s, es);
+    // by storage and collision: pairs (or one cell per thread), quads, lanes 32 cells apart
+    static constexpr Pass passes[3][2][3] = {
+        {{launch_f32_reg, nullptr, launch_f32_reg_row}, {launch_f32_bgk, nullptr, launch_f32_bgk_row}},
+        {{launch_f16_reg, launch_f16_reg_quad, launch_f16_reg_row}, {launch_f16_bgk, launch_f16_bgk_quad, launch_f16_bgk_row}},
+        {{launch_f16sr_reg, launch_f16sr_reg_quad, launch_f16sr_reg_row},
+         {launch_f16sr_bgk, launch_f16sr_bgk_quad, launch_f16sr_bgk_row}}};
+    const bool reduce = passes[storage][collision][row_lanes(a, storage) ? 2 : (cpl == 4 ? 1 : 0)](a, stats, s, es);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (forked) {
         if ((e = cudaEventRecord(join, side)) != cudaSuccess) return e;

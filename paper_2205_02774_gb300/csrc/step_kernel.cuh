@@ -48,6 +48,8 @@
 namespace stg {
 
 constexpr int PULL = 0, AA_SHIFT = 1, AA_LOCAL = 2;
+// two lattices as PULL, lanes 32 cells apart (lbm_row.cuh)
+constexpr int ROW = 3;
 
 // the place of this step's plane in StepArgs::ubc; the step index is read again
 // (an L1 hit, by the lanes that hold an inlet node) rather than kept in a
@@ -57,6 +59,25 @@ __device__ __forceinline__ size_t inlet_plane(const StepArgs &a)
     unsigned t;
     asm volatile("ld.global.u32 %0, [%1];" : "=r"(t) : "l"(&a.ctl->t[a.parity]));
     return (size_t)(t & (INLET_RING - 1));
+}
+
+// The inlet node x = 0 from its streamed populations g (the unknown ones, c_x > 0,
+// are not read); node: its place in a velocity plane.  Zou-He density, eq.
+// (density_bc): parallel set + 2 x leaving set.  The weights of that combination
+// sum to 1 (2/3 + 2 x 1/6), so rho_bc - 1 = (S_g + u_x)/(1 - u_x) with S_g the same
+// sum of the shifted populations.
+__device__ __forceinline__ void inlet_node(const StepArgs &a, float (&g)[Q], size_t node)
+{
+    const size_t pl3 = (size_t)a.ny * a.nz;
+    const size_t pc = inlet_plane(a) * 3 * pl3 + node;
+    const float ubx = a.ubc[pc], uby = a.ubc[pl3 + pc], ubz = a.ubc[2 * pl3 + pc];
+    float par = 0.f, lv = 0.f;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        if (cx_of(i) == 0) par += g[i];
+        if (cx_of(i) < 0) lv += g[i];
+    }
+    rebuild<1>(g, (fmaf(2.0f, lv, par) + ubx) / (1.0f - ubx), ubx, uby, ubz);
 }
 
 // Stochastic rounding of binary16 stores (SR kernels): a value between two
@@ -202,20 +223,7 @@ __device__ __forceinline__ void step_column(const StepArgs &a, int bx, int y)
                 gather_general<S>(src, P, nx, ny, x, y, z, xm, xp, xm_ok, xp_ok, ym, yp, ym_w, yp_w, zm, zp, here, g);
                 if (inout && (x == 0 || x == nx - 1)) {
                     if (x == 0) {
-                        const size_t pl3 = (size_t)ny * nz;
-                        const size_t pc = inlet_plane(a) * 3 * pl3 + (size_t)z * ny + y;
-                        const float ubx = a.ubc[pc], uby = a.ubc[pl3 + pc], ubz = a.ubc[2 * pl3 + pc];
-                        // Zou-He density, eq. (density_bc): parallel set + 2 x leaving set.
-                        // The weights of that combination sum to 1 (2/3 + 2 x 1/6), so
-                        // rho_bc - 1 = (S_g + u_x)/(1 - u_x) with S_g the same sum of g.
-                        float par = 0.f, lv = 0.f;
-#pragma unroll
-                        for (int i = 0; i < Q; ++i) {
-                            if (cx_of(i) == 0) par += g[i];
-                            if (cx_of(i) < 0) lv += g[i];
-                        }
-                        const float drb = (fmaf(2.0f, lv, par) + ubx) / (1.0f - ubx);
-                        rebuild<1>(g, drb, ubx, uby, ubz);
+                        inlet_node(a, g, (size_t)z * ny + y);
                     } else {
                         // zero-gradient pressure outlet: rho = 1 and the velocity of the
                         // neighbour x = nx-2 at this step, from its streamed populations
@@ -673,19 +681,7 @@ __device__ __forceinline__ float vec_loop(const StepArgs &a, float (*sacc)[9][BX
             const bool node = (j == 0 && at_inlet) || (j == CPL - 1 && at_outlet);
             auto rebuild_node = [&](float (&gg)[Q]) {
                 if (j == 0 && at_inlet) {
-                    // Zou-He density, eq. (density_bc): parallel set + 2 x leaving set,
-                    // rho_bc - 1 = (S_g + u_x)/(1 - u_x) in shifted variables; the
-                    // unknowns (c_x > 0, their sources lie outside) are not read
-                    const size_t pl3 = (size_t)ny * nz;
-                    const size_t pc = inlet_plane(a) * 3 * pl3 + (size_t)z * ny + y;
-                    const float ubx = a.ubc[pc], uby = a.ubc[pl3 + pc], ubz = a.ubc[2 * pl3 + pc];
-                    float par = 0.f, lv = 0.f;
-#pragma unroll
-                    for (int i = 0; i < Q; ++i) {
-                        if (cx_of(i) == 0) par += gg[i];
-                        if (cx_of(i) < 0) lv += gg[i];
-                    }
-                    rebuild<1>(gg, (fmaf(2.0f, lv, par) + ubx) / (1.0f - ubx), ubx, uby, ubz);
+                    inlet_node(a, gg, (size_t)z * ny + y);
                 }
                 if (j == CPL - 1 && at_outlet) {
                     // zero-gradient pressure outlet: rho = 1 and the velocity of the
@@ -810,6 +806,12 @@ __device__ __forceinline__ float vec_loop(const StepArgs &a, float (*sacc)[9][BX
     return sdr;
 }
 
+}  // namespace stg
+
+#include "lbm_row.cuh"
+
+namespace stg {
+
 // Rows of a vector launch: INNER, y = 1..ny-2, or ANY, y = 0, a.row_step, ...
 // (all rows, or the wall rows alone).
 constexpr int INNER = 0, ANY = 1;
@@ -849,7 +851,7 @@ __global__ void __launch_bounds__(BX *block_warps<CPL, STATS>(), warps_per_sm<CP
     const int nx = a.nx, ny = a.ny;
     const int lane = threadIdx.x, wi = threadIdx.y;
     const int y = ROWS == INNER ? blockIdx.y + 1 : blockIdx.y * a.row_step;
-    const int x0 = BX * CPL * (STATS ? blockIdx.x : blockDim.y * blockIdx.x + wi);
+    const int x0 = BX * CPL * (STATS ? blockIdx.x : blockDim.y * blockIdx.x + wi) - (MODE == ROW ? row_shift(nx, H16) : 0);
     const long long t = a.ctl->t[a.parity];
     const bool do_check = a.check_every > 0 && ((t + 1) % a.check_every) == 0;
     const int zc = STATS ? a.stat_group : a.tile_zc;
@@ -861,10 +863,16 @@ __global__ void __launch_bounds__(BX *block_warps<CPL, STATS>(), warps_per_sm<CP
             for (int j = 0; j < CPL; ++j) sacc[wi][q][CPL * lane + j] = 0.f;
     }
     float sdr;
-    if (ROWS == ANY && (y == 0 || y == ny - 1))
-        sdr = vec_loop<S, CPL, REG, FORCE, STATS, true, SP, H16, MODE, SR>(a, sacc, x0, y, zb, ze, zs);
-    else
-        sdr = vec_loop<S, CPL, REG, FORCE, STATS, false, SP, H16, MODE, SR>(a, sacc, x0, y, zb, ze, zs);
+    const bool edge = ROWS == ANY && (y == 0 || y == ny - 1);
+    if constexpr (MODE == ROW) {
+        __shared__ unsigned keep_all[NW][2][Q];  // inputs of the pairs with a boundary node (binary16)
+        unsigned (*keep)[Q] = keep_all[wi];
+        if (edge) sdr = row_loop<S, CPL, REG, FORCE, STATS, true, SP, H16, SR>(a, sacc, keep, x0, y, zb, ze, zs);
+        else sdr = row_loop<S, CPL, REG, FORCE, STATS, false, SP, H16, SR>(a, sacc, keep, x0, y, zb, ze, zs);
+    } else {
+        if (edge) sdr = vec_loop<S, CPL, REG, FORCE, STATS, true, SP, H16, MODE, SR>(a, sacc, x0, y, zb, ze, zs);
+        else sdr = vec_loop<S, CPL, REG, FORCE, STATS, false, SP, H16, MODE, SR>(a, sacc, x0, y, zb, ze, zs);
+    }
     if (STATS) {
         __syncthreads();
         const size_t m = (size_t)nx * ny;
@@ -874,7 +882,7 @@ __global__ void __launch_bounds__(BX *block_warps<CPL, STATS>(), warps_per_sm<CP
             float v = sacc[0][q][c];
 #pragma unroll
             for (int k = 1; k < NW; ++k) v += sacc[k][q][c];
-            if (x0 + c < nx) part[q * m + c] = v;
+            if ((unsigned)(x0 + c) < (unsigned)nx) part[q * m + c] = v;
         }
     }
     if (do_check) mass_finish<BX * NW>(a, sdr);
@@ -933,9 +941,9 @@ static Split split_of(const StepArgs &a)
 template <typename S, int CPL, bool REG, bool FORCE, bool SP, int MODE, bool SR, int ROWS>
 static void launch_rows(const StepArgs &a, bool stats, dim3 grid, int nw, cudaStream_t s)
 {
-    // binary16 in an inlet/outlet lattice: x halo by 2-byte loads
-    // (the local in-place step reads no x neighbour)
-    constexpr bool H = sizeof(S) == 2 && MODE != AA_LOCAL;
+    // binary16 in an inlet/outlet lattice: x halo by 2-byte loads (the local
+    // in-place step reads no x neighbour)
+    constexpr bool H = MODE == ROW || (sizeof(S) == 2 && MODE != AA_LOCAL);
     const bool h16 = H && a.bc_x == 0;
     const dim3 block(BX, nw);
     if (stats && h16) lbm_vec_kernel<S, CPL, REG, FORCE, true, ROWS, SP, H, MODE, SR><<<grid, block, 0, s>>>(a);
@@ -950,7 +958,7 @@ static void launch_rows(const StepArgs &a, bool stats, dim3 grid, int nw, cudaSt
 template <typename S, int CPL, bool REG, bool FORCE, bool SP, int MODE, bool SR>
 static void launch_vec(StepArgs a, bool stats, cudaStream_t s, cudaStream_t side)
 {
-    const int chunks = (a.nx + BX * CPL - 1) / (BX * CPL);
+    const int chunks = (a.nx + BX * CPL - 1) / (BX * CPL);  // (a row's shift adds none)
     int nw = block_warps<CPL, false>();
     // chunks per block: as many as leave the fewest warps idle
     for (int k = nw - 1; k > 0; --k)
@@ -1003,6 +1011,16 @@ static bool launch_forced(StepArgs a, bool stats, cudaStream_t s, cudaStream_t s
         if (n_in > 0) lbm_step_kernel<S, REG, FORCE, SP, SR><<<dim3(sp.gx, sp.gy), block, 0, s>>>(ai);
     }
     return false;
+}
+
+// The same for lanes 32 cells apart.
+template <typename S, int CPL, bool REG, bool SR = false>
+bool launch_row(const StepArgs &a, bool stats, cudaStream_t s, cudaStream_t side)
+{
+    if (a.spf) launch_vec<S, CPL, REG, false, true, ROW, SR>(a, stats, s, side);
+    else if (a.has_force) launch_vec<S, CPL, REG, true, false, ROW, SR>(a, stats, s, side);
+    else launch_vec<S, CPL, REG, false, false, ROW, SR>(a, stats, s, side);
+    return stats;
 }
 
 // CPL: cells per lane of the vector kernels (2, with the one-cell-per-thread
