@@ -539,10 +539,10 @@ __device__ __forceinline__ float vec_loop(const StepArgs &a, float (*sacc)[9][BX
     // binary16, regularized collision: pair sums by mixed-precision adds
     constexpr bool MIXED = REG && sizeof(S) == 2;
     // binary16: the lane's cells go through the collision two at a time in
-    // packed FP32 (lbm_pair.cuh) wherever the warp's 32 CPL cells hold no inlet
-    // or outlet node; the warps that do and FP32 storage (whose step is bound by
-    // memory either way) update cell by cell.  A warp's chunk is the same in every kernel and
-    // tile, so each cell always takes the same form.
+    // packed FP32 (lbm_pair.cuh) unless one of the warp's lanes holds an inlet or
+    // outlet node in that pair; those pairs and FP32 storage (whose step is bound
+    // by memory either way) go cell by cell.  A warp's chunk is the same in every
+    // kernel and tile, so each cell always takes the same form.
     constexpr bool PACKED = sizeof(S) == 2;
     const int nx = a.nx, ny = a.ny, nz = a.nz;
     const int nxy = nx * ny;
@@ -560,7 +560,10 @@ __device__ __forceinline__ float vec_loop(const StepArgs &a, float (*sacc)[9][BX
     // CPL); both are rebuilt here from the values already in registers
     const bool at_inlet = inout && x == 0;
     const bool at_outlet = inout && active && x + CPL == nx;
-    const bool node_warp = inout && (x0 == 0 || x0 + BX * CPL >= nx);
+    // pairs k of the warp's lanes among which a node is (the first or the last pairs)
+    auto pair_has_node = [&](int k) {
+        return inout && ((k == 0 && x0 == 0) || (k == CPL / 2 - 1 && x0 + BX * CPL >= nx));
+    };
     // y neighbours of this row (YEDGE rows only)
     bool ym_bb = false, yp_bb = false;
     int ym_off = nx, yp_off = -nx;  // element offset of the source row for c_y = +1 / -1 (subtracted)
@@ -640,13 +643,28 @@ __device__ __forceinline__ float vec_loop(const StepArgs &a, float (*sacc)[9][BX
         // stochastic rounding: the bits of a pair's conversion depend on the
         // pair's first cell, so pairs and quads round a lattice alike
         auto seed_of = [&](int k) { return SR ? sr_seed(here + 2 * k, tmix) : 0u; };
-        if (PACKED && !node_warp) {
-            // the lane's cells two at a time (packed FP32 pairs)
+        auto count = [&](int j, float drho, float ux, float uy, float uz) {
+            if (!active) return;
+            if (STATS) {
+                // explicit fused multiply-adds: every kernel instance rounds the sums
+                // alike (the compiler would otherwise fuse them or not depending on
+                // how it shares the products with the collision)
+                float *sp = &sacc[wi][0][CPL * lane + j];
+                constexpr int L = BX * CPL;
+                sp[0 * L] += ux; sp[1 * L] += uy; sp[2 * L] += uz;
+                sp[3 * L] = __fmaf_rn(ux, ux, sp[3 * L]); sp[4 * L] = __fmaf_rn(uy, uy, sp[4 * L]);
+                sp[5 * L] = __fmaf_rn(uz, uz, sp[5 * L]); sp[6 * L] = __fmaf_rn(ux, uy, sp[6 * L]);
+                sp[7 * L] = __fmaf_rn(ux, uz, sp[7 * L]); sp[8 * L] = __fmaf_rn(uy, uz, sp[8 * L]);
+            }
+            sdr += drho;
+        };
 #pragma unroll
-            for (int k = 0; k < CPL / 2; ++k) {
+        for (int k = 0; k < CPL / 2; ++k) {
+            const unsigned seed = seed_of(k);
+            if (PACKED && !pair_has_node(k)) {
+                // both cells of the pair in packed FP32
                 float2 nuf = make_float2(1.0f, 1.0f);
                 if (SP && active) nuf = __ldg(reinterpret_cast<const float2 *>(a.spf + x + 2 * k));
-                const unsigned seed = seed_of(k);
                 auto pop = [&](int i) { return V::pair(v[i], k); };
                 const PairMoments m = pair_moments(pop);
                 float2 drho, ux, uy, uz;
@@ -654,101 +672,71 @@ __device__ __forceinline__ float vec_loop(const StepArgs &a, float (*sacc)[9][BX
                     if constexpr (SR) V::set_pair_rs(v[i], k, r.x, r.y, sr_bits(seed, i));
                     else V::set_pair(v[i], k, r.x, r.y);
                 }, drho, ux, uy, uz);
-                if (active) {
-                    if (STATS) {
-                        constexpr int L = BX * CPL;
-#pragma unroll
-                        for (int j = 0; j < 2; ++j) {
-                            float *sp = &sacc[wi][0][CPL * lane + 2 * k + j];
-                            const float vx = j ? ux.y : ux.x, vy = j ? uy.y : uy.x, vz = j ? uz.y : uz.x;
-                            sp[0 * L] += vx; sp[1 * L] += vy; sp[2 * L] += vz;
-                            sp[3 * L] = __fmaf_rn(vx, vx, sp[3 * L]); sp[4 * L] = __fmaf_rn(vy, vy, sp[4 * L]);
-                            sp[5 * L] = __fmaf_rn(vz, vz, sp[5 * L]); sp[6 * L] = __fmaf_rn(vx, vy, sp[6 * L]);
-                            sp[7 * L] = __fmaf_rn(vx, vz, sp[7 * L]); sp[8 * L] = __fmaf_rn(vy, vz, sp[8 * L]);
-                        }
-                    }
-                    sdr += drho.x;
-                    sdr += drho.y;
-                }
+                count(2 * k, drho.x, ux.x, uy.x, uz.x);
+                count(2 * k + 1, drho.y, ux.y, uy.y, uz.y);
+                continue;
             }
-        } else {
-        float upx = 0.f, upy = 0.f, upz = 0.f;  // velocity of the lane's previous cell
-        float gp[Q];                            // results of the pair's first cell
+            float upx = 0.f, upy = 0.f, upz = 0.f;  // velocity of the pair's first cell
+            float gp[Q];                            // its results
 #pragma unroll
-        for (int j = 0; j < CPL; ++j) {
-            float g[Q];
-            // boundary nodes of this cell (inlet x = 0 at j = 0, outlet x = nx-1 at the last j)
-            const bool node = (j == 0 && at_inlet) || (j == CPL - 1 && at_outlet);
-            auto rebuild_node = [&](float (&gg)[Q]) {
-                if (j == 0 && at_inlet) {
-                    inlet_node(a, gg, (size_t)z * ny + y);
-                }
-                if (j == CPL - 1 && at_outlet) {
-                    // zero-gradient pressure outlet: rho = 1 and the velocity of the
-                    // neighbour x = nx-2 (this lane's previous cell) at this step
-                    rebuild<-1>(gg, 0.0f, upx, upy, upz);
-                }
-            };
-            float drho, ux, uy, uz;
-            const float nuf = SP && active ? __ldg(a.spf + x + j) : 1.0f;
-            if constexpr (MIXED) {
-                // regularized collision of binary16 pairs: only the pair sums and
-                // differences enter, formed with one conversion per pair
-                float s[9], d[9], drho0;
-                if (node) {
+            for (int j = 2 * k; j < 2 * k + 2; ++j) {
+                float g[Q];
+                // boundary nodes of this cell (inlet x = 0 at j = 0, outlet x = nx-1 at the last j:
+                // rho = 1 and the velocity of the neighbour x = nx-2, the pair's first cell)
+                const bool in = j == 0 && at_inlet, out = j == CPL - 1 && at_outlet;
+                auto rebuild_node = [&](float (&gg)[Q]) {
+                    if (in) inlet_node(a, gg, (size_t)z * ny + y);
+                    if (out) rebuild<-1>(gg, 0.0f, upx, upy, upz);
+                };
+                float drho, ux, uy, uz;
+                const float nuf = SP && active ? __ldg(a.spf + x + j) : 1.0f;
+                if constexpr (MIXED) {
+                    // regularized collision of binary16 pairs: only the pair sums and
+                    // differences enter, formed with one conversion per pair
+                    float s[9], d[9], drho0;
+                    if (in || out) {
 #pragma unroll
-                    for (int i = 0; i < Q; ++i) g[i] = V::cell(v[i], j);
-                    rebuild_node(g);
+                        for (int i = 0; i < Q; ++i) g[i] = V::cell(v[i], j);
+                        rebuild_node(g);
 #pragma unroll
-                    for (int p = 0; p < 9; ++p) {
-                        s[p] = g[2 * p + 1] + g[2 * p + 2];
-                        d[p] = g[2 * p + 1] - g[2 * p + 2];
+                        for (int p = 0; p < 9; ++p) {
+                            s[p] = g[2 * p + 1] + g[2 * p + 2];
+                            d[p] = g[2 * p + 1] - g[2 * p + 2];
+                        }
+                        drho0 = g[0] + s[0];
+                    } else {
+#pragma unroll
+                        for (int p = 0; p < 9; ++p) {
+                            const float b = V::cell(v[2 * p + 2], j);
+                            s[p] = V::add_h(v[2 * p + 1], j, b);
+                            d[p] = V::sub_h(v[2 * p + 1], j, b);
+                        }
+                        drho0 = V::add_h(v[0], j, s[0]);
                     }
-                    drho0 = g[0] + s[0];
+                    collide_sd<REG, FORCE, SP>(g, s, d, drho0, tau0, kq, Fx, Fy, Fz, drho, ux, uy, uz, nuf);
                 } else {
 #pragma unroll
-                    for (int p = 0; p < 9; ++p) {
-                        const float b = V::cell(v[2 * p + 2], j);
-                        s[p] = V::add_h(v[2 * p + 1], j, b);
-                        d[p] = V::sub_h(v[2 * p + 1], j, b);
-                    }
-                    drho0 = V::add_h(v[0], j, s[0]);
+                    for (int i = 0; i < Q; ++i) g[i] = V::cell(v[i], j);
+                    if (in || out) rebuild_node(g);
+                    collide<REG, FORCE, SP>(g, tau0, kq, Fx, Fy, Fz, drho, ux, uy, uz, nuf);
                 }
-                collide_sd<REG, FORCE, SP>(g, s, d, drho0, tau0, kq, Fx, Fy, Fz, drho, ux, uy, uz, nuf);
-            } else {
+                upx = ux;
+                upy = uy;
+                upz = uz;
+                // the first cell waits in FP32; the second completes the pair, which
+                // replaces the pair's (already read) inputs
 #pragma unroll
-                for (int i = 0; i < Q; ++i) g[i] = V::cell(v[i], j);
-                if (node) rebuild_node(g);
-                collide<REG, FORCE, SP>(g, tau0, kq, Fx, Fy, Fz, drho, ux, uy, uz, nuf);
+                for (int i = 0; i < Q; ++i) {
+                    if (j == 2 * k) gp[i] = g[i];
+                    else if constexpr (SR) V::set_pair_rs(v[i], k, gp[i], g[i], sr_bits(seed, i));
+                    else V::set_pair(v[i], k, gp[i], g[i]);
+                }
+                count(j, drho, ux, uy, uz);
             }
-            upx = ux;
-            upy = uy;
-            upz = uz;
-            // the pair's first cell waits in FP32; the second completes the pair,
-            // which replaces the pair's (already read) inputs
-            const unsigned seed = (j & 1) ? seed_of(j >> 1) : 0u;
-#pragma unroll
-            for (int i = 0; i < Q; ++i) {
-                if ((j & 1) == 0) gp[i] = g[i];
-                else if constexpr (SR) V::set_pair_rs(v[i], j >> 1, gp[i], g[i], sr_bits(seed, i));
-                else V::set_pair(v[i], j >> 1, gp[i], g[i]);
-            }
-            const bool counted = active;
-            if (STATS && counted) {
-                float *sp = &sacc[wi][0][CPL * lane + j];
-                constexpr int L = BX * CPL;
-                // explicit fused multiply-adds: every kernel instance rounds the sums
-                // alike (the compiler would otherwise fuse them or not depending on
-                // how it shares the products with the collision)
-                sp[0 * L] += ux; sp[1 * L] += uy; sp[2 * L] += uz;
-                sp[3 * L] = __fmaf_rn(ux, ux, sp[3 * L]); sp[4 * L] = __fmaf_rn(uy, uy, sp[4 * L]);
-                sp[5 * L] = __fmaf_rn(uz, uz, sp[5 * L]); sp[6 * L] = __fmaf_rn(ux, uy, sp[6 * L]);
-                sp[7 * L] = __fmaf_rn(ux, uz, sp[7 * L]); sp[8 * L] = __fmaf_rn(uy, uz, sp[8 * L]);
-            }
-            if (counted) sdr += drho;
         }
-        }
-        if (active) {
+        // (in place, even steps: the quads go through shuffles of the whole warp)
+        constexpr bool SHIFT4 = MODE == AA_SHIFT && CPL == 4;
+        if (SHIFT4 || active) {
 #pragma unroll
             for (int i = 0; i < Q; ++i) {
                 if (MODE == PULL) {
@@ -768,7 +756,7 @@ __device__ __forceinline__ float vec_loop(const StepArgs &a, float (*sacc)[9][BX
                 const int cx = cx_of(i), cz = cz_of(i), cy = cy_of(i);
                 const bool yout = YEDGE && ((cy > 0 && yp_bb) || (cy < 0 && ym_bb));
                 if (yout) {
-                    V::st(own_slot(i), v[i]);
+                    if (active) V::st(own_slot(i), v[i]);
                     continue;
                 }
                 // target row (y + c_y, z + c_z): the source row of population opp(i)
@@ -777,28 +765,43 @@ __device__ __forceinline__ float vec_loop(const StepArgs &a, float (*sacc)[9][BX
                 S *trow = reinterpret_cast<S *>(reinterpret_cast<char *>(dbase + (row0 + tz + ty)) + (size_t)i * Pb);
                 S *tx = trow + x;
                 if (cx == 0) {
-                    V::st(tx, v[i]);
-                } else if (cx < 0) {
-                    // cells x + 1 .. x + CPL - 1 -> x .. x + CPL - 2 (quads: cells 1, 2
-                    // as one aligned pair), cell x -> x - 1; the row's first cell
-                    // (lanes with x = 0 only): outside at the inlet (the own slot),
-                    // wraps to x = nx - 1 when x is periodic
-                    if constexpr (CPL == 4) {
-                        V::st_mid(tx, v[i]);
-                        V::st1(tx - 1, v[i], 3);
+                    if (active) V::st(tx, v[i]);
+                } else if constexpr (SHIFT4) {
+                    // the target quad x .. x + 3 from the lane's own cells and one of the
+                    // lane beside it; where that lane is in another warp (or the row ends)
+                    // the own cells alone, cells 1 and 2 as one aligned pair, and the cell
+                    // that leaves the warp's quads by itself: outside at the open ends (the
+                    // own slot), wrapped when x is periodic
+                    const unsigned beside = cx < 0 ? __shfl_down_sync(0xffffffffu, v[i].x, 1)
+                                                   : __shfl_up_sync(0xffffffffu, v[i].y, 1);
+                    if (!active) continue;
+                    const unsigned mid = __byte_perm(v[i].x, v[i].y, 0x5432);
+                    if (cx < 0) {
+                        if (!side_r) V::st(tx, make_uint2(mid, __byte_perm(v[i].y, beside, 0x5432)));
+                        else {
+                            V::st_mid(tx, v[i]);
+                            V::st1(tx - 1, v[i], 3);
+                        }
+                        if (lane == 0) V::st1(x > 0 ? tx - 1 : (inout ? own_slot(i) : tx + (nx - 1)), v[i], 0);
                     } else {
-                        V::st1(tx - 1, v[i], 1);
+                        if (lane > 0) V::st(tx, make_uint2(__byte_perm(beside, v[i].x, 0x5432), mid));
+                        else {
+                            V::st1(tx + 1, v[i], 0);
+                            V::st_mid(tx + 2, v[i]);
+                        }
+                        if (side_r) V::st1(x + CPL < nx ? tx + 1 : (inout ? own_slot(i) : tx - (x + CPL - 1)), v[i], CPL - 1);
                     }
-                    if (x > 0) V::st1(tx - 1, v[i], 0);
-                    else V::st1(inout ? own_slot(i) : tx + (nx - 1), v[i], 0);
+                } else if (cx < 0) {
+                    // cell x + 1 -> x, cell x -> x - 1; the row's first cell (lanes with
+                    // x = 0 only): outside at the inlet (the own slot), wraps to
+                    // x = nx - 1 when x is periodic
+                    V::st1(tx - 1, v[i], 1);
+                    V::st1(x > 0 ? tx - 1 : (inout ? own_slot(i) : tx + (nx - 1)), v[i], 0);
                 } else {
-                    // cells x .. x + CPL - 2 -> x + 1 .. x + CPL - 1 (quads: cells 1, 2
-                    // as one aligned pair), cell x + CPL - 1 -> x + CPL; the row's last
-                    // cell (lanes with x = nx - CPL only): outside at the outlet, wraps to 0
+                    // cell x -> x + 1, cell x + 1 -> x + 2; the row's last cell (lanes with
+                    // x = nx - 2 only): outside at the outlet, wraps to 0
                     V::st1(tx + 1, v[i], 0);
-                    if constexpr (CPL == 4) V::st_mid(tx + 2, v[i]);
-                    if (x + CPL < nx) V::st1(tx + 1, v[i], CPL - 1);
-                    else V::st1(inout ? own_slot(i) : tx - (x + CPL - 1), v[i], CPL - 1);
+                    V::st1(x + CPL < nx ? tx + 1 : (inout ? own_slot(i) : tx - (x + CPL - 1)), v[i], CPL - 1);
                 }
             }
         }
