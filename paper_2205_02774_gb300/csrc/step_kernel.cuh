@@ -88,12 +88,9 @@ __device__ __forceinline__ void inlet_node(const StepArgs &a, float (&g)[Q], siz
 // half: bits 0-12 for the low half, 16-28 for the high half.  The bits are a
 // fixed function of (first cell of the pair, step, population), so a run is
 // reproducible and independent of the launch decomposition: a per-pair seed
-// from two multiply-xorshift rounds, then one multiply per population by an odd
-// constant of its own.  The 19 constants were drawn at random and kept where the
-// 38 13-bit fields of a pair are uncorrelated (below 0.005 in size over 2 10^6
-// pairs and two steps, the sampling noise being 0.003; neighbouring cells, rows,
-// planes and steps: noise), which an earlier form (the middle of a 64-bit product
-// of the seed plus a Weyl sequence, three instructions, 0.049) was less.
+// from two multiply-xorshift rounds, then, per population, the middle 32 bits
+// of the 64-bit product of the seed (offset by a Weyl sequence in i) with an
+// odd constant.
 __device__ __forceinline__ unsigned sr_seed(unsigned cell, unsigned tmix)
 {
     unsigned s = (cell * 0x9E3779B1u) ^ tmix;
@@ -101,14 +98,11 @@ __device__ __forceinline__ unsigned sr_seed(unsigned cell, unsigned tmix)
     return s ^ (s >> 12);
 }
 __device__ __forceinline__ unsigned sr_tmix(long long t) { return (unsigned)t * 0x85EBCA77u; }
-__host__ __device__ constexpr unsigned sr_mul(int i)
+__device__ __forceinline__ unsigned sr_bits(unsigned seed, int i)
 {
-    constexpr unsigned c[Q] = {0xB0FD574Du, 0xD133612Fu, 0x8BAD9A3Bu, 0xA741942Fu, 0x5497A305u, 0x6C022F1Du, 0x1ADDB539u,
-                               0x1BB3AC7Bu, 0x3DD5F2EFu, 0x86535593u, 0xF62F10F1u, 0x48AFC469u, 0xEFF946C3u, 0xB1EA3ACFu,
-                               0x6DB5CBB1u, 0x61DB376Du, 0x19602FB5u, 0x91B89277u, 0x31E8B3CDu};
-    return c[i];
+    const unsigned long long p = (unsigned long long)(seed ^ (0x9E3779B9u * (unsigned)(i + 1))) * 0xD168AAADull;
+    return (unsigned)(p >> 16);
 }
-__device__ __forceinline__ unsigned sr_bits(unsigned seed, int i) { return seed * sr_mul(i); }
 // one binary16 by stochastic rounding (the low half of the pair conversion)
 __device__ __forceinline__ void st_half_rs(__half *p, float g, unsigned rb)
 {
