@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <chrono>
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -470,7 +471,15 @@ namespace host {
 // the block, INLET_MAX_PLANES at a time, beside the passes that read those.  One
 // launch per step instead took 10 to 19 us each on lattices whose pass takes 4 to
 // 60, ahead of the pass or of its wall rows.
-cudaError_t enqueue_steps(stg_lbm *h, int64_t t, int n)
+cudaError_t enqueue_probes(stg_lbm *h, int64_t t, cudaStream_t s)
+{
+    stg::LatticeView v = lattice_view(h);
+    v.t = t;
+    return stg::launch_probe(h->lat[t & 1], h->d.storage, v, h->n_probes, h->probe_xyz, (float)h->d.force[0],
+                             (float)h->d.force[1], (float)h->d.force[2], h->ctl, s);
+}
+
+cudaError_t enqueue_steps(stg_lbm *h, int64_t t, int n, bool probed)
 {
     constexpr int FIRST = 4;
     cudaError_t e = cudaSuccess;
@@ -495,10 +504,24 @@ cudaError_t enqueue_steps(stg_lbm *h, int64_t t, int n)
             // the ring holds the planes that the coming passes read and as many again
             if (e == cudaSuccess && asked < n) ask(s == 0 ? FIRST : stg::INLET_MAX_PLANES);
         }
+        // two lattices: the samples of a step are taken beside the next one, which
+        // reads the same lattice, and before the one after, which writes it
+        if (e == cudaSuccess && probed && s >= 2 && !h->aa) e = cudaStreamWaitEvent(h->stream, h->ev_pjoin[s & 1], 0);
         if (e == cudaSuccess)
             e = stg::launch_step(step_args(h, (int)((t + s) & 1)), h->d.storage, h->d.collision, is_stats_step(h, t + s),
                                  h->stream, h->side, h->ev_fork, h->ev_join);
+        if (!probed || e != cudaSuccess) continue;
+        if (h->aa) {
+            e = enqueue_probes(h, t + s + 1, h->stream);
+            continue;
+        }
+        e = cudaEventRecord(h->ev_pfork, h->stream);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(h->side, h->ev_pfork, 0);
+        if (e == cudaSuccess) e = enqueue_probes(h, t + s + 1, h->side);
+        if (e == cudaSuccess) e = cudaEventRecord(h->ev_pjoin[s & 1], h->side);
     }
+    for (int s = std::max(0, n - 2); s < n && probed && !h->aa && e == cudaSuccess; ++s)
+        e = cudaStreamWaitEvent(h->stream, h->ev_pjoin[s & 1], 0);
     if (e == cudaSuccess && h->inout && n > 0) e = cudaStreamWaitEvent(h->stream, h->ev_ijoin, 0);
     return e;
 }
@@ -510,11 +533,11 @@ namespace {
 
 // Graph of `steps` steps from step index t0 on (of which only the parity and
 // the place in the sampling period matter).
-int capture(stg_lbm *h, int64_t t0, int steps, cudaGraphExec_t *out)
+int capture(stg_lbm *h, int64_t t0, int steps, cudaGraphExec_t *out, bool probed = false)
 {
     cudaGraph_t g = nullptr;
     CK(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-    cudaError_t e = enqueue_steps(h, t0, steps);
+    cudaError_t e = enqueue_steps(h, t0, steps, probed);
     cudaError_t e2 = cudaStreamEndCapture(h->stream, &g);
     if (e != cudaSuccess) {
         if (g) cudaGraphDestroy(g);
@@ -539,7 +562,27 @@ void destroy_graphs(stg_lbm *h)
         }
         if (h->g_block[p]) cudaGraphExecDestroy(h->g_block[p]);
         h->g_block[p] = nullptr;
+        if (h->g_probed[p]) cudaGraphExecDestroy(h->g_probed[p]);
+        h->g_probed[p] = nullptr;
     }
+}
+
+// The block graphs with probes, if there are probes.
+int capture_probed(stg_lbm *h)
+{
+    int rc = STG_OK;
+    const int64_t shared = h->in_flight;
+    h->in_flight = 0;
+    const int k = std::max(h->d.stats_every, 1);
+    for (int q = 0; q < 2 && rc == STG_OK; ++q) {
+        cudaGraphExec_t &g = h->g_probed[(q * k) & 1];
+        if (q > 0 && (k & 1) == 0) break;  // blocks of an even period begin at even steps
+        if (g) cudaGraphExecDestroy(g);
+        g = nullptr;
+        if (h->n_probes > 0 && h->block_steps > 0) rc = capture(h, q * k, h->block_steps, &g, true);
+    }
+    h->in_flight = shared;
+    return rc;
 }
 
 // Single-step graphs by [parity][sampling] and the block graphs by parity.
@@ -559,6 +602,7 @@ int capture_all(stg_lbm *h)
             rc = capture(h, t, h->block_steps, &h->g_block[t & 1]);
     }
     h->in_flight = shared;
+    if (rc == STG_OK) rc = capture_probed(h);
     return rc;
 }
 
@@ -631,9 +675,8 @@ namespace host {
 
 int queue_check_readback(stg_lbm *h, int64_t t_before)
 {
-    (void)t_before;
-    // read back the last check only once a check step has run since the reset
-    if (h->d.check_every > 0 && h->t / h->d.check_every > h->t0_stats / h->d.check_every) {
+    // only when a check step has run: the result of an earlier one is on its way already
+    if (h->d.check_every > 0 && h->t / h->d.check_every > t_before / h->d.check_every) {
         CK(cudaMemcpyAsync(h->h_pinned, h->mass_out, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
         CK(cudaEventRecord(h->ev_check, h->stream));
         h->check_pending = true;
@@ -751,6 +794,8 @@ void release(stg_lbm *h)
     if (h->inlet_side) cudaStreamDestroy(h->inlet_side);
     if (h->ev_ifork) cudaEventDestroy(h->ev_ifork);
     if (h->ev_ijoin) cudaEventDestroy(h->ev_ijoin);
+    for (cudaEvent_t e : {h->ev_pfork, h->ev_pjoin[0], h->ev_pjoin[1]})
+        if (e) cudaEventDestroy(e);
     if (h->ev_done) cudaEventDestroy(h->ev_done);
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
     delete h;
@@ -853,6 +898,9 @@ int stg_lbm_create(const stg_domain *domain, const stg_rans_profile *rans, const
         cudaStreamCreateWithPriority(&h->inlet_side, cudaStreamNonBlocking, hi_prio) != cudaSuccess ||
         cudaEventCreateWithFlags(&h->ev_ifork, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&h->ev_ijoin, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&h->ev_pfork, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&h->ev_pjoin[0], cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&h->ev_pjoin[1], cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&h->ev_done, cudaEventDisableTiming) != cudaSuccess ||
         !(h->h_pinned = pinned_slots().get())) {
         h->err = "event / pinned allocation failed";
@@ -975,6 +1023,7 @@ int stg_lbm_step(stg_lbm *h, int64_t n)
     int rc = poll_check(h);
     if (rc) return rc;
     if (h->sticky) return fail(h, h->sticky, "an earlier check failed; reset the state first");
+    const int64_t t_before = h->t;
     const int per = h->d.stats_every;
     while (n > 0) {
         cudaGraphExec_t g;
@@ -991,7 +1040,7 @@ int stg_lbm_step(stg_lbm *h, int64_t n)
         h->t += k;
         n -= k;
     }
-    return queue_check_readback(h, h->t);
+    return queue_check_readback(h, t_before);
 }
 
 int stg_lbm_step_timed(stg_lbm *h, int64_t n, double *ms_step, double *ms_inlet)
@@ -1319,7 +1368,7 @@ int stg_lbm_set_probes(stg_lbm *h, int32_t n, const int32_t *xyz)
     }
     if (n > 0) CK(cudaMemcpy(h->probe_xyz, xyz, sizeof(int) * 3 * (size_t)n, cudaMemcpyHostToDevice));
     h->n_probes = n;
-    return STG_OK;
+    return capture_probed(h);
 }
 
 int stg_lbm_step_probed(stg_lbm *h, int64_t n, float *u_host)
@@ -1340,13 +1389,28 @@ int stg_lbm_step_probed(stg_lbm *h, int64_t n, float *u_host)
         }
         h->probe_cap = need;
     }
+    // where the call's samples go (the words are free again: the call waits for its work)
     const int64_t t_before = h->t;
-    for (int64_t s = 0; s < n; ++s) {
+    struct {
+        long long t;
+        float *out;
+    } series{h->t, h->probe_buf};
+    static_assert(sizeof series == 2 * sizeof(double) && offsetof(StepCtl, probe_out) == offsetof(StepCtl, t_probe) + 8, "layout");
+    std::memcpy(h->h_pinned + 2, &series, sizeof series);
+    CK(cudaMemcpyAsync(&h->ctl->t_probe, h->h_pinned + 2, sizeof series, cudaMemcpyHostToDevice, h->stream));
+    const int per = h->d.stats_every;
+    for (int64_t s = 0; s < n;) {
+        cudaGraphExec_t g = h->g_probed[h->t & 1];
+        if (g && n - s >= h->block_steps && (per <= 0 || h->t % per == 0)) {
+            CK(cudaGraphLaunch(g, h->stream));
+            h->t += h->block_steps;
+            s += h->block_steps;
+            continue;
+        }
         CK(cudaGraphLaunch(h->g_single[h->t & 1][is_stats_step(h, h->t) ? 1 : 0], h->stream));
         h->t += 1;
-        CK(stg::launch_probe(h->lat[h->t & 1], h->d.storage, lattice_view(h), h->n_probes, h->probe_xyz,
-                             (float)h->d.force[0], (float)h->d.force[1], (float)h->d.force[2],
-                             h->probe_buf + (size_t)s * h->n_probes * 3, h->stream));
+        s += 1;
+        CK(enqueue_probes(h, h->t, h->stream));
     }
     rc = queue_check_readback(h, t_before);
     if (rc) return rc;

@@ -52,6 +52,7 @@ struct stg_lbm {
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     cudaStream_t inlet_side = nullptr;                 // branch for the inlet planes
     cudaEvent_t ev_ifork = nullptr, ev_ijoin = nullptr;
+    cudaEvent_t ev_pfork = nullptr, ev_pjoin[2] = {nullptr, nullptr};  // probes beside the next step
     bool check_pending = false;
     int64_t t = 0, t0_stats = 0;
     double mass0 = 0.0;
@@ -61,6 +62,7 @@ struct stg_lbm {
     // start at a step index divisible by the sampling period, by parity
     cudaGraphExec_t g_single[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
     cudaGraphExec_t g_block[2] = {nullptr, nullptr};
+    cudaGraphExec_t g_probed[2] = {nullptr, nullptr};  // blocks with the probes sampled after every step
     int block_steps = 16;
     stg_info info{};
     double timeout_s = 900.0;
@@ -87,7 +89,8 @@ int cuda_fail(stg_lbm *h, cudaError_t e, const char *what);
 // the n steps of h from step index t on (their inlet planes included) on
 // h->stream and h->side; of t only the parity and the place in the sampling
 // period matter
-cudaError_t enqueue_steps(stg_lbm *h, int64_t t, int n);
+// (probed: with the probes sampled after every step)
+cudaError_t enqueue_steps(stg_lbm *h, int64_t t, int n, bool probed = false);
 bool is_stats_step(const stg_lbm *h, int64_t t);
 // evaluate the last completed mass check (non-blocking)
 int poll_check(stg_lbm *h);

@@ -15,6 +15,8 @@ struct StepCtl {
     long long t[2];
     long long t0_filter;  // step at which the temporal filter restarts
     long long t_block;    // step at which the current block of steps began
+    long long t_probe;    // probed steps: step index before the first one of the call
+    float *probe_out;     // and its samples [steps][3 n]
     unsigned long long err; // error bits set by kernels (none of the current kernels sets one)
 };
 
@@ -129,9 +131,10 @@ struct LatticeView {
     size_t P;
     long long t;
 };
-// velocity of n cells (xyz: device int triples) of a stored lattice into out[3 n]
+// velocity of n cells (xyz: device int triples) of the lattice stored after lv.t
+// steps, into the place of that step in ctl->probe_out
 cudaError_t launch_probe(const void *src, int storage, const LatticeView &lv, int n, const int *xyz, float Fx,
-                         float Fy, float Fz, float *out, cudaStream_t s);
+                         float Fy, float Fz, const StepCtl *ctl, cudaStream_t s);
 // canonical sub-block [19][bz][by][bx] of a stored lattice into device memory `out`
 cudaError_t launch_gather_block(const void *src, int storage, const LatticeView &lv, int x0, int y0, int z0, int bx,
                                 int by, int bz, void *out, cudaStream_t s);
