@@ -57,7 +57,7 @@ def _kernel_hash():
     """Hash of the step kernels' source with comments and white space removed
     (a comment edit does not change the kernel whose counters were taken)."""
     h = hashlib.sha256()
-    for f in ("step_kernel.cu", "step_kernel.cuh", "d3q19.cuh", "internal.h", "lbm_cell.cuh", "lbm_pair.cuh", "reduce.cuh"):
+    for f in ("step_kernel.cu", "step_kernel.cuh", "d3q19.cuh", "internal.h", "lbm_cell.cuh", "lbm_pair.cuh", "lbm_row.cuh", "reduce.cuh"):
         with open(os.path.join(ROOT, "paper_2205_02774_gb300", "csrc", f)) as fh:
             src = fh.read()
         src = re.sub(r"/\*.*?\*/", "", src, flags=re.S)
@@ -99,6 +99,33 @@ def _launches(c, t0, steps):
     n = _launches_per_step(c) * steps
     if c.stats_every > 0 and c.nx % 2 == 0 and c.nx >= 4:
         n += sum(1 for t in range(t0, t0 + steps) if (t + 1) % c.stats_every == 0)
+    return n
+
+
+def _launches_enqueued(c, t0, steps, batch=False):
+    """Kernels the steps t0 .. t0+steps-1 really enqueue, as the library cuts them:
+    blocks (from a step index divisible by the sampling period; in a batch from any)
+    carry one inlet launch for the first 4 steps and one per 16 more, single steps
+    one each; a pass is one launch on lattices that do not fill the GPU, else two."""
+    k = max(c.stats_every, 1)
+    period = k * -(-16 // k) if c.stats_every > 0 else 16
+    if batch:
+        period = k * (1 if k % 2 == 0 else 2) * -(-16 // (k * (1 if k % 2 == 0 else 2)))
+    row = c.streaming == "pull" and (c.nx % 2 != 0 or c.nx < 4)
+    small = c.streaming == "pull" and c.storage == "fp32" and c.cells < 4 * 152 * 32 * 32 and not batch
+    cpl = (4 if row or (c.nx % 4 == 0 and c.nx >= 8) else 2) if c.storage != "fp32" else (1 if small else 2)
+    items = -(-c.nx // (32 * cpl)) * c.ny * c.nz
+    passes = 1 if c.ny < 3 or (not batch and 2 * items < 152 * 16 * (3 if cpl == 4 else 8)) else 2
+    inlet = c.bc_x == "stg"
+    n, t, left = 0, t0, steps
+    while left > 0:
+        whole = period <= 256 and left >= period and (batch or t % k == 0)
+        b = period if whole else 1
+        n += b * passes + (inlet and 1 + max(0, -(-(b - 4) // 16)))
+        t += b
+        left -= b
+    if c.stats_every > 0:
+        n += (t0 + steps) // c.stats_every - t0 // c.stats_every
     return n
 
 
@@ -294,7 +321,7 @@ def roofline(bpc, cells, ms_step, ms_inlet, traffic, kernel):
             "inlet_kernel_ms": ms_inlet}
 
 
-STEP_KERNEL = "lbm_vec_zc_kernel (rows 1..ny-2, inlet and outlet nodes included) + wall rows: one step pass"
+STEP_KERNEL = "lbm_vec_kernel (rows 1..ny-2, inlet and outlet nodes included) + wall rows: one step pass"
 
 
 def measure_channel(c, args, rank=0, dist=None, seed=None, sample_clocks=True):
@@ -425,7 +452,7 @@ def run_ours(args):
                    "parallelism": f"replicas x{ws}"},
         "roofline": roofline(BYTES_PER_CELL[c.storage], c.cells, m["ms_step"], m["ms_inlet"], traffic, STEP_KERNEL),
         "hbm_frac_of_step": m["hbm_frac_of_step"],
-        "gpu_launches": _launches(c, args.warmup, args.steps) + (args.steps if args.probes > 0 else 0),
+        "gpu_launches": _launches_enqueued(c, args.warmup, args.steps) + (args.steps if args.probes > 0 else 0),
         "clocks": m["clocks"],
     }
     line["e2e"] = end_to_end(c, args.steps)
@@ -446,7 +473,7 @@ def run_ours(args):
                 "ms_per_step": m2["ms_per_step"], "hbm_frac_of_step": m2["hbm_frac_of_step"], "tile": m2["tile"],
                 "clocks": m2["clocks"], "device_gb": m2["device_gb"],
                 "roofline": roofline(BYTES_PER_CELL[st], c2.cells, m2["ms_step"], m2["ms_inlet"], t2, STEP_KERNEL),
-                "gpu_launches": _launches(c2, args.warmup, args.steps)})
+                "gpu_launches": _launches_enqueued(c2, args.warmup, args.steps)})
     if ws == 1 and not args.no_cpu_baseline:
         line["cpu_baseline"] = cpu_baseline(args.workload, c.storage, args.cpu_steps, args.cpu_cells,
                                             extra=dict(collision=c.collision, sponge_len=c.sponge_len,
@@ -504,7 +531,7 @@ def ensemble_run(members, steps, warmup, storage):
                         "traffic": None, "scope": "whole step incl. inlet kernels",
                         "peak_source": f"{peak_kind} hbm_gbs (copy)"},
            "failed_members": bad, "clocks": clocks,
-           "gpu_launches": sum(_launches(j.case, warmup, steps) for j in jobs)}
+           "gpu_launches": sum(_launches_enqueued(j.case, warmup, steps, batch=True) for j in jobs)}
     b.close()
     for ch in chans:
         ch.close()

@@ -185,6 +185,12 @@ double vk_spectrum(double k, double le, double leta, double lcut)
     return e;
 }
 
+double wrap2pi(double v)
+{
+    v = std::fmod(v, 2.0 * kPi);
+    return v < 0.0 ? v + 2.0 * kPi : v;
+}
+
 // Inlet tables: Algorithm 1, LBM section steps 1-4.
 int build_inlet(stg_lbm *h, const stg_rans_profile *r, uint64_t seed)
 {
@@ -231,9 +237,7 @@ int build_inlet(stg_lbm *h, const stg_rans_profile *r, uint64_t seed)
     h->info.max_le = max_le;
     int N = 0;
     std::vector<double> kn, dk, phi, omg;
-    std::vector<float> sig;
-    std::vector<double> A;
-    std::vector<float2> BS;
+    std::vector<float> sig, A, BS;
     if (max_le > 0.0) {
         const double kmin = kPi / max_le, kmax = 1.5 * max_kcut;
         h->info.k_min = kmin;
@@ -269,11 +273,8 @@ int build_inlet(stg_lbm *h, const stg_rans_profile *r, uint64_t seed)
             sig[3 * n + 2] = (float)(-st * ce);
             // eq. (psu) at x = 0: phase advance -2 pi d_x U_b / max l_e per step
             omg[n] = -2.0 * kPi * dx * h->info.U_b / max_le;
-            for (int j = 0; j < ny; ++j) A[(size_t)n * ny + j] = kn[n] * dy * (j + 0.5);
-            for (int k = 0; k < nz; ++k) {
-                const double b = kn[n] * dz * k;
-                BS[(size_t)n * nz + k] = make_float2((float)std::cos(b), (float)std::sin(b));
-            }
+            for (int j = 0; j < ny; ++j) A[(size_t)n * ny + j] = (float)wrap2pi(kn[n] * dy * (j + 0.5));
+            for (int k = 0; k < nz; ++k) BS[(size_t)n * nz + k] = (float)wrap2pi(kn[n] * dz * k);
         }
     }
     h->N = N;
@@ -281,8 +282,8 @@ int build_inlet(stg_lbm *h, const stg_rans_profile *r, uint64_t seed)
     h->a_filter = h->p.T_filter > 0.0 ? (float)std::exp(-1.0 / h->p.T_filter) : 0.0f;
     h->info.a_filter = h->a_filter;
 
-    // mode amplitudes sqrt(6 q^n(y_j)), eq. (qn), times (cos, sin) of the y part
-    // of the phase, per inlet node, FP64 on the host (terms added in mode order)
+    // the y part of the phase and the mode amplitude sqrt(6 q^n(y_j)), eq. (qn), per
+    // inlet node, FP64 on the host (terms added in mode order)
     std::vector<float2> AS((size_t)std::max(N, 1) * ny, make_float2(0.f, 0.f));
     {
         std::vector<double> e(std::max(N, 1));
@@ -292,10 +293,9 @@ int build_inlet(stg_lbm *h, const stg_rans_profile *r, uint64_t seed)
                 e[n] = vk_spectrum(kn[n], le[j], leta[j], lcut[j]) * dk[n];
                 total += e[n];
             }
-            for (int n = 0; n < N && total > 0.0; ++n) {
-                const double q = std::sqrt(6.0 * e[n] / total), p = A[(size_t)n * ny + j];
-                AS[(size_t)n * ny + j] = make_float2((float)(q * std::cos(p)), (float)(q * std::sin(p)));
-            }
+            for (int n = 0; n < N; ++n)
+                AS[(size_t)n * ny + j] = make_float2(A[(size_t)n * ny + j],
+                                                     total > 0.0 ? (float)std::sqrt(6.0 * e[n] / total) : 0.0f);
         }
     }
     // time part of the phase, phi^n + omega^n t, as Q0.64 fractions of a turn:
@@ -310,7 +310,7 @@ int build_inlet(stg_lbm *h, const stg_rans_profile *r, uint64_t seed)
     // device tables
     const size_t Nn = (size_t)std::max(N, 1);
     h->AS = (float2 *)dalloc(h, sizeof(float2) * Nn * ny);
-    h->BS = (float2 *)dalloc(h, sizeof(float2) * Nn * nz);
+    h->BS = (float *)dalloc(h, sizeof(float) * Nn * nz);
     h->sig = (float *)dalloc(h, sizeof(float) * 3 * Nn);
     h->phq = (unsigned long long *)dalloc(h, sizeof(unsigned long long) * Nn);
     h->omq = (unsigned long long *)dalloc(h, sizeof(unsigned long long) * Nn);
@@ -325,7 +325,7 @@ int build_inlet(stg_lbm *h, const stg_rans_profile *r, uint64_t seed)
     CK(cudaMemcpy(dR6, R6.data(), sizeof(double) * 6 * ny, cudaMemcpyHostToDevice));
     CK(cudaMemcpy(h->AS, AS.data(), sizeof(float2) * AS.size(), cudaMemcpyHostToDevice));
     if (N > 0) {
-        CK(cudaMemcpy(h->BS, BS.data(), sizeof(float2) * BS.size(), cudaMemcpyHostToDevice));
+        CK(cudaMemcpy(h->BS, BS.data(), sizeof(float) * BS.size(), cudaMemcpyHostToDevice));
         CK(cudaMemcpy(h->sig, sig.data(), sizeof(float) * sig.size(), cudaMemcpyHostToDevice));
         CK(cudaMemcpy(h->phq, phq.data(), sizeof(unsigned long long) * N, cudaMemcpyHostToDevice));
         CK(cudaMemcpy(h->omq, omq.data(), sizeof(unsigned long long) * N, cudaMemcpyHostToDevice));
@@ -1007,7 +1007,7 @@ int stg_lbm_estimate_bytes(const stg_domain *d, const stg_params *p, int64_t *by
         if (p && p->n_modes > 0) N = p->n_modes;
         else if (p && p->alpha > 0.0) N = std::ceil(std::log(1.5 * std::max(ny, 2.0)) / std::log(1.0 + p->alpha) + 1.0);
         // AS, BS, sigma, the two phase words, a6, u_int, the FP64 stresses
-        b += r(8 * N * ny) + r(8 * N * nz) + r(12 * N) + 2 * r(8 * N) + r(24 * ny) + r(4 * ny) +
+        b += r(8 * N * ny) + r(4 * N * nz) + r(12 * N) + 2 * r(8 * N) + r(24 * ny) + r(4 * ny) +
              r(48 * ny);
     }
     *bytes = (int64_t)b;

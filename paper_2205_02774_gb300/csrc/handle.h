@@ -34,8 +34,8 @@ struct stg_lbm {
     int *probe_xyz = nullptr;             // device [3 n_probes]
     float *probe_buf = nullptr;           // device samples of one step_probed call
     size_t probe_cap = 0;                 // floats in probe_buf
-    float2 *AS = nullptr, *BS = nullptr;
-    float *sig = nullptr, *a6 = nullptr, *u_int = nullptr;
+    float2 *AS = nullptr;
+    float *BS = nullptr, *sig = nullptr, *a6 = nullptr, *u_int = nullptr;
     unsigned long long *phq = nullptr, *omq = nullptr;  // phi^n and omega^n as Q0.64 fractions of a turn
     int N = 0;
     float a_filter = 0.f;

@@ -7,28 +7,28 @@
 //   u'  = a(j) v'                                                           eqs. (v_fluc), (cholesky)
 //   u_f = a u_f + (1 - a) u'   (first-order temporal filter; u_f = u' at the first step)
 //   u_bc = u_int(j) e_x + u_f                                               eqs. (u_phys), (u_transfer)
-// By the addition theorem the cosine of the whole phase splits into factors of
-// one variable each,
-//   sqrt(6 q^n(j)) cos(A^n_j + B^n_k + th^n(t)) = ca cb' - sa sb',
-//   (ca, sa) = sqrt(6 q^n(j)) (cos, sin) A^n_j   A: y part, k^n d^n_y y_j
-//   (cb', sb') = (cos, sin)(B^n_k + th^n(t)), from the tables (cos, sin) B^n_k
-//                (z part) and (cos, sin) th^n(t) of the time phase,
-// so a mode term is two multiply-adds and three more into v' instead of a range
-// reduction and a cosine.  The static tables are built in FP64 on the host; the
-// time phase phi^n + omega^n t is a Q0.64 fraction of a turn advanced by
-// wrapping 64-bit integer arithmetic (exact modulo a turn for any step count).
+// The phase is split into three parts each already reduced to [0, 2 pi):
+// the y part and the z part (tables built in FP64 on the host) and the time
+// part phi^n + omega^n t, kept as Q0.64 fractions of a turn and advanced by
+// wrapping 64-bit integer arithmetic (a phase accumulator: exact modulo a
+// turn for any step count, no floating point); their FP32 sum is below 6 pi
+// and is reduced to [-pi, pi] before the cosine.
 //
 // One launch computes the planes of `planes` consecutive steps (a block of steps
 // asks for them a few and then 16 at a time, beside its passes, instead of one
 // launch in every step).  A block of 8 warps covers 32 consecutive j (one per
 // lane) and ITEMS = 8 IPW pairs (span node, step), IPW per warp in registers:
 // IPW = 4 for more than 8 planes, 1 up to that, where the latency of the launch
-// counts.  Per chunk of modes the block stages the y factors, the time factors and
-// the items' (cb', sb') in shared memory; a mode then costs a warp 2 + IPW
-// shared-memory reads and 6 IPW multiplies and multiply-adds, and issuing those
-// bounds the kernel.  The sum over the modes is in mode order in every form, and
-// every multiply-add is written out, so a plane's bits do not depend on how many
-// were asked for.  The filter then runs over the steps in order, one thread per node.
+// counts.  Per chunk of modes the block stages the y parts and amplitudes
+// sqrt(6 q^n(j)), sigma^n and the items' time and z parts in shared memory, the
+// table reads issued a chunk ahead; a mode then costs a warp 2 + IPW shared-memory
+// reads and per item the phase sum and its reduction, one cosine and four
+// multiply-adds.  The modes of even and of odd index are summed apart, each in
+// order, and then added, in every form, so a plane's bits do not depend on how many
+// were asked for.  The filter then runs over the steps in order, one thread per
+// node.  (cos(a + b) by the addition theorem on sine and cosine tables halves the
+// kernel's time, which passes hide almost all of, but rounds its planes otherwise,
+// and binary16 storage turns that into differences of whole spacings.)
 #include "internal.h"
 
 namespace stg {
@@ -41,11 +41,9 @@ __global__ void __launch_bounds__(INLET_J * INLET_WARPS, 2) stg_inlet_kernel(con
 {
     constexpr int ITEMS = IPW * INLET_WARPS;
     constexpr int CHUNK = IPW == 1 ? 96 : 32;              // modes staged per pass through shared memory
-    constexpr int STEPS = IPW == 1 ? ITEMS : INLET_MAX_PLANES;
     constexpr int NT = INLET_J * INLET_WARPS;
-    __shared__ float2 ys[CHUNK][INLET_J];                  // (ca, sa) per mode and wall-normal node
-    __shared__ float2 ts[CHUNK][STEPS];                    // (cos, sin) of the time phase per mode and step
-    __shared__ float2 is[CHUNK][ITEMS];                    // (cb', sb') per mode and item
+    __shared__ float2 ys[CHUNK][INLET_J];                  // (y part, amplitude) per mode and wall-normal node
+    __shared__ float2 is[CHUNK][ITEMS];                    // (time part, z part) per mode and item
     __shared__ float4 sg[CHUNK];                           // sigma^n
     __shared__ float vs[ITEMS][3][INLET_J];                // v' per item and node
     const int lane = threadIdx.x, w = threadIdx.y;
@@ -56,26 +54,24 @@ __global__ void __launch_bounds__(INLET_J * INLET_WARPS, 2) stg_inlet_kernel(con
     const int items = kb * T;         // <= ITEMS
     const float af = a.a_filter, bf = 1.0f - a.a_filter;
     const size_t plane = (size_t)ny * nz;
-    float v[IPW][3];
+    float v[2][IPW][3];  // modes of even and odd index
 #pragma unroll
-    for (int q = 0; q < IPW; ++q) v[q][0] = v[q][1] = v[q][2] = 0.f;
+    for (int q = 0; q < 2 * IPW; ++q) v[q & 1][q >> 1][0] = v[q & 1][q >> 1][1] = v[q & 1][q >> 1][2] = 0.f;
     // The table reads of a chunk are issued together, a chunk ahead of their use:
     // their latency is most of what a chunk costs a launch of few blocks.
-    constexpr int NB = CHUNK * ITEMS / NT, NY = CHUNK * INLET_J / NT, NS = (CHUNK * STEPS + NT - 1) / NT;
-    float2 b[NB], y[NY];
-    unsigned long long ph[NS], om[NS];
+    constexpr int NB = CHUNK * ITEMS / NT, NY = CHUNK * INLET_J / NT;
+    float b[NB];
+    float2 y[NY];
+    unsigned long long ph[NB], om[NB];
     float4 sgr;
     auto fetch = [&](int n0) {
         const int cn = min(CHUNK, N - n0);
 #pragma unroll
-        for (int i = 0; i < NS; ++i) {
-            const int m = (tid + i * NT) / T;
-            if (m < cn) ph[i] = a.phq[n0 + m], om[i] = a.omq[n0 + m];
-        }
-#pragma unroll
         for (int i = 0; i < NB; ++i) {
             const int e = tid + i * NT, m = e / ITEMS, q = e % ITEMS;
-            if (m < cn && q < items) b[i] = a.BS[(size_t)(n0 + m) * nz + min(k0 + q / T, nz - 1)];  // nodes past nz are not stored
+            if (m >= cn || q >= items) continue;
+            ph[i] = a.phq[n0 + m], om[i] = a.omq[n0 + m];
+            b[i] = a.BS[(size_t)(n0 + m) * nz + min(k0 + q / T, nz - 1)];  // nodes past nz are not stored
         }
 #pragma unroll
         for (int i = 0; i < NY; ++i) {
@@ -107,15 +103,12 @@ __global__ void __launch_bounds__(INLET_J * INLET_WARPS, 2) stg_inlet_kernel(con
         const int cn = min(CHUNK, N - n0);
         __syncthreads();  // the previous chunk is consumed
 #pragma unroll
-        for (int i = 0; i < NS; ++i) {
-            const int e = tid + i * NT, m = e / T, s = e - m * T;
-            if (m >= cn) continue;
-            // time part of the phase modulo one turn; its top 32 bits as a signed
-            // fraction of half a turn
-            const unsigned long long q = ph[i] + om[i] * (unsigned long long)(t + s);
-            float sn, cs;
-            sincospif((float)(int)(unsigned)(q >> 32) * 4.656612873077393e-10f, &sn, &cs);  // 2^-31
-            ts[m][s] = make_float2(cs, sn);
+        for (int i = 0; i < NB; ++i) {
+            const int e = tid + i * NT, m = e / ITEMS, q = e % ITEMS;
+            if (m >= cn || q >= items) continue;
+            // time part of the phase: phi^n + omega^n t modulo one turn
+            const unsigned long long p = ph[i] + om[i] * (unsigned long long)(t + q % T);
+            is[m][q] = make_float2((float)(unsigned)(p >> 32) * 1.4629180792671596e-09f, b[i]);  // 2 pi / 2^32
         }
 #pragma unroll
         for (int i = 0; i < NY; ++i) {
@@ -124,34 +117,35 @@ __global__ void __launch_bounds__(INLET_J * INLET_WARPS, 2) stg_inlet_kernel(con
         }
         if (tid < cn) sg[tid] = sgr;
         __syncthreads();
-#pragma unroll
-        for (int i = 0; i < NB; ++i) {
-            const int e = tid + i * NT, m = e / ITEMS, q = e % ITEMS;
-            if (m >= cn || q >= items) continue;
-            const float2 th = ts[m][q % T];
-            is[m][q] = make_float2(fmaf(b[i].x, th.x, -__fmul_rn(b[i].y, th.y)),
-                                   fmaf(b[i].y, th.x, __fmul_rn(b[i].x, th.y)));
-        }
         if (n0 + CHUNK < N) fetch(n0 + CHUNK);
-        __syncthreads();
-#pragma unroll 4
-        for (int m = 0; m < cn; ++m) {
-            const float2 y = ys[m][lane];
+        // (a chunk's length is even: the parity of m is the mode's)
+        auto term = [&](int m, float (&vp)[IPW][3]) {
+            const float2 ya = ys[m][lane];
             const float4 s = sg[m];
 #pragma unroll
             for (int q = 0; q < IPW; ++q) {
-                const float2 bq = is[m][w * IPW + q];
-                const float c = fmaf(y.x, bq.x, -__fmul_rn(y.y, bq.y));
-                v[q][0] = fmaf(c, s.x, v[q][0]);
-                v[q][1] = fmaf(c, s.y, v[q][1]);
-                v[q][2] = fmaf(c, s.z, v[q][2]);
+                const float2 tb = is[m][w * IPW + q];
+                float arg = ya.x + tb.x;                       // in [0, 4 pi)
+                arg = arg + tb.y;                              // in [0, 6 pi)
+                arg -= 6.2831853f * rintf(arg * 0.15915494f);  // to [-pi, pi]
+                const float amp = ya.y * __cosf(arg);
+                vp[q][0] = fmaf(amp, s.x, vp[q][0]);
+                vp[q][1] = fmaf(amp, s.y, vp[q][1]);
+                vp[q][2] = fmaf(amp, s.z, vp[q][2]);
             }
+        };
+        int m = 0;
+#pragma unroll 2
+        for (; m + 1 < cn; m += 2) {
+            term(m, v[0]);
+            term(m + 1, v[1]);
         }
+        if (m < cn) term(m, v[0]);
     }
 #pragma unroll
     for (int q = 0; q < IPW; ++q)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) vs[w * IPW + q][c][lane] = v[q][c];
+        for (int c = 0; c < 3; ++c) vs[w * IPW + q][c][lane] = v[0][q][c] + v[1][q][c];
     __syncthreads();
     for (int e = tid; e < kb * INLET_J; e += NT, mine = fetch_node(e)) {
         if (!mine) continue;
@@ -160,13 +154,13 @@ __global__ void __launch_bounds__(INLET_J * INLET_WARPS, 2) stg_inlet_kernel(con
         for (int s = 0; s < T; ++s) {
             const float *vq = &vs[kk * T + s][0][jj];
             const float v0 = vq[0], v1 = vq[INLET_J], v2 = vq[2 * INLET_J];
-            const float u[3] = {__fmul_rn(L[0], v0), fmaf(L[2], v1, __fmul_rn(L[1], v0)),
-                                fmaf(L[5], v2, fmaf(L[4], v1, __fmul_rn(L[3], v0)))};
+            const float u[3] = {__fmul_rn(L[0], v0), fmaf(L[1], v0, __fmul_rn(L[2], v1)),
+                                fmaf(L[5], v2, fmaf(L[3], v0, __fmul_rn(L[4], v1)))};
             const bool first = (t + s == t0f);
             float *o = a.ubc + (size_t)((t + s) & (INLET_RING - 1)) * 3 * plane + node;
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                f[c] = first ? u[c] : fmaf(af, f[c], __fmul_rn(bf, u[c]));
+                f[c] = first ? u[c] : fmaf(bf, u[c], __fmul_rn(af, f[c]));
                 o[c * plane] = c == 0 ? ui + f[c] : f[c];
             }
         }

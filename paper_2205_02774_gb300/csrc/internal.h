@@ -69,8 +69,8 @@ struct StepArgs {
 
 struct InletArgs {
     int ny, nz, N;
-    const float2 *AS;     // [N][ny]  sqrt(6 q^n(y_j)) (cos, sin) of k^n d^n_y (j + 1/2)
-    const float2 *BS;     // [N][nz]  (cos, sin) of k^n d^n_z k
+    const float2 *AS;     // [N][ny]  k^n d^n_y (j + 1/2) mod 2 pi, sqrt(6 q^n(y_j))
+    const float *BS;      // [N][nz]  k^n d^n_z k mod 2 pi
     const float *sig;     // [N][3]   sigma^n
     const unsigned long long *phq;  // [N] phi^n / (2 pi) as a Q0.64 fraction of a turn
     const unsigned long long *omq;  // [N] phase advance per step, -d^n_x U_b / max l_e turns, Q0.64

@@ -72,20 +72,32 @@ struct Strip<__half, CPL> {
     }
 };
 
-// Velocity of a cell from its streamed populations, rounded as collide() rounds it.
-template <bool FORCE>
+// Velocity of a cell from its streamed populations, for the outlet node beside it:
+// with the sums in population order (odd nx), or with collide()'s rounding (ORDER
+// false: what the pairs of even nx take).
+template <bool FORCE, bool ORDER>
 __device__ __forceinline__ void cell_velocity(const float (&g)[Q], float Fx, float Fy, float Fz, float &ux, float &uy,
                                               float &uz)
 {
     float drho = 0.f, jx = 0.f, jy = 0.f, jz = 0.f;
+    if (ORDER) {
 #pragma unroll
-    for (int p = 0; p < 9; ++p) {
-        const int i = 2 * p + 1;
-        const float s = g[i] + g[i + 1], d = g[i] - g[i + 1];
-        drho = p ? drho + s : g[0] + s;
-        if (cx_of(i)) jx += cx_of(i) * d;
-        if (cy_of(i)) jy += cy_of(i) * d;
-        if (cz_of(i)) jz += cz_of(i) * d;
+        for (int i = 0; i < Q; ++i) {
+            drho += g[i];
+            if (cx_of(i)) jx += cx_of(i) * g[i];
+            if (cy_of(i)) jy += cy_of(i) * g[i];
+            if (cz_of(i)) jz += cz_of(i) * g[i];
+        }
+    } else {
+#pragma unroll
+        for (int p = 0; p < 9; ++p) {
+            const int i = 2 * p + 1;
+            const float s = g[i] + g[i + 1], d = g[i] - g[i + 1];
+            drho = p ? drho + s : g[0] + s;
+            if (cx_of(i)) jx += cx_of(i) * d;
+            if (cy_of(i)) jy += cy_of(i) * d;
+            if (cz_of(i)) jz += cz_of(i) * d;
+        }
     }
     const float irho = 1.0f / (1.0f + drho);
     ux = (FORCE ? fmaf(0.5f, Fx, jx) : jx) * irho;
@@ -177,7 +189,6 @@ __device__ __forceinline__ float row_loop(const StepArgs &a, float (*sacc)[9][32
             sdr += drho;
         };
         auto nu_factor = [&](int j) { return SP && on(j) ? __ldg(a.spf + x + 32 * j) : 1.0f; };
-        auto seed_of = [&](int k) { return SR ? sr_seed((unsigned)here + 64 * k, tmix) : 0u; };
         // the node x = 0 or x = nx-1 in g; the outlet: rho = 1 and the velocity u of the
         // neighbour x = nx-2 at this step (the lane beside it: x0 is chosen so)
         auto node_of = [&](float (&g)[Q], int j, float ux, float uy, float uz) {
@@ -188,7 +199,10 @@ __device__ __forceinline__ float row_loop(const StepArgs &a, float (*sacc)[9][32
         if constexpr (PACKED) {
 #pragma unroll
             for (int k = 0; k < CPL / 2; ++k) {
-                const unsigned seed = seed_of(k);
+                // stochastic rounding: each cell has its own seed, its bits the low 13 of a word
+                const unsigned s0 = SR ? sr_seed((unsigned)here + 64 * k, tmix) : 0u;
+                const unsigned s1 = SR ? sr_seed((unsigned)here + 64 * k + 32, tmix) : 0u;
+                auto bits = [&](int i) { return __byte_perm(sr_bits(s0, i), sr_bits(s1, i), 0x5410); };
                 const float2 nuf = make_float2(nu_factor(2 * k), nu_factor(2 * k + 1));
                 const bool nodes = has_inlet(2 * k) || has_outlet(2 * k) || has_outlet(2 * k + 1);
                 // the lane of an inlet / outlet node keeps the pair's inputs (in shared
@@ -198,11 +212,22 @@ __device__ __forceinline__ float row_loop(const StepArgs &a, float (*sacc)[9][32
 #pragma unroll
                     for (int i = 0; i < Q; ++i) keep[slot][i] = v[i].w[k];
                 }
+                // the velocity of the cell to the left, for the outlet node
+                float lx = 0.f, ly = 0.f, lz = 0.f;
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    if (!has_outlet(2 * k + c)) continue;
+                    float g[Q];
+#pragma unroll
+                    for (int i = 0; i < Q; ++i) g[i] = v[i].cell(2 * k + c);
+                    cell_velocity<FORCE, true>(g, Fx, Fy, Fz, lx, ly, lz);
+                    lx = from_left(lx), ly = from_left(ly), lz = from_left(lz);
+                }
                 auto pop = [&](int i) { return v[i].pair(k); };
                 const PairMoments m = pair_moments(pop);
                 float2 drho, ux, uy, uz;
-                collide_pair<REG, FORCE, SP>(m, pop, tau0, kq, nuf, Fx, Fy, Fz, [&](int i, float2 r) {
-                    if constexpr (SR) v[i].set_pair_rs(k, r.x, r.y, sr_bits(seed, i));
+                collide_pair_cell<REG, FORCE, SP>(m, pop, tau0, kq, nuf, Fx, Fy, Fz, [&](int i, float2 r) {
+                    if constexpr (SR) v[i].set_pair_rs(k, r.x, r.y, bits(i));
                     else v[i].set_pair(k, r.x, r.y);
                 }, drho, ux, uy, uz);
                 if (nodes) {
@@ -211,7 +236,6 @@ __device__ __forceinline__ float row_loop(const StepArgs &a, float (*sacc)[9][32
                     for (int c = 0; c < 2; ++c) {
                         const int j = 2 * k + c, xj = x + 32 * j;
                         if (!has_inlet(j) && !has_outlet(j)) continue;
-                        const float lx = from_left(c ? ux.y : ux.x), ly = from_left(c ? uy.y : uy.x), lz = from_left(c ? uz.y : uz.x);
                         if (!((has_inlet(j) && xj == 0) || (has_outlet(j) && xj == nx - 1))) continue;
                         float g[Q];
 #pragma unroll
@@ -222,7 +246,7 @@ __device__ __forceinline__ float row_loop(const StepArgs &a, float (*sacc)[9][32
 #pragma unroll
                         for (int i = 0; i < Q; ++i) {
                             const unsigned w = v[i].w[k];
-                            if constexpr (SR) v[i].set_pair_rs(k, g[i], g[i], sr_bits(seed, i));
+                            if constexpr (SR) v[i].set_pair_rs(k, g[i], g[i], bits(i));
                             else v[i].set_pair(k, g[i], g[i]);
                             v[i].w[k] = __byte_perm(w, v[i].w[k], c ? 0x7610 : 0x3254);
                         }
@@ -244,7 +268,8 @@ __device__ __forceinline__ float row_loop(const StepArgs &a, float (*sacc)[9][32
                 if (has_inlet(j) || has_outlet(j)) {
                     float ux = 0.f, uy = 0.f, uz = 0.f;
                     if (has_outlet(j)) {
-                        cell_velocity<FORCE>(g, Fx, Fy, Fz, ux, uy, uz);
+                        if (nx & 1) cell_velocity<FORCE, true>(g, Fx, Fy, Fz, ux, uy, uz);
+                        else cell_velocity<FORCE, false>(g, Fx, Fy, Fz, ux, uy, uz);
                         ux = from_left(ux), uy = from_left(uy), uz = from_left(uz);
                     }
                     node_of(g, j, ux, uy, uz);

@@ -1,5 +1,5 @@
 // Host-side launch of one fused step pass (the kernels: step_kernel.cuh and
-// its six instantiation units), the initial-state kernel, the statistics
+// its instantiation units), the initial-state kernel, the statistics
 // reduction of sampling steps and the FP64 mass reduction.
 #include <algorithm>
 

@@ -533,10 +533,12 @@ __device__ __forceinline__ float vec_loop(const StepArgs &a, float (*sacc)[9][BX
     // binary16, regularized collision: pair sums by mixed-precision adds
     constexpr bool MIXED = REG && sizeof(S) == 2;
     // binary16: the lane's cells go through the collision two at a time in
-    // packed FP32 (lbm_pair.cuh) unless one of the warp's lanes holds an inlet or
-    // outlet node in that pair; those pairs and FP32 storage (whose step is bound
-    // by memory either way) go cell by cell.  A warp's chunk is the same in every
-    // kernel and tile, so each cell always takes the same form.
+    // packed FP32 (lbm_pair.cuh) wherever the warp's 32 CPL cells hold no inlet
+    // or outlet node; the warps that do and FP32 storage (whose step is bound by
+    // memory either way) update cell by cell (packing the other pairs of such a
+    // warp as well was slower: its code takes registers from the main path,
+    // 768x128x192 FP16-SR 259 against 237 us per step).  A warp's chunk is the same
+    // in every kernel and tile, so each cell always takes the same form.
     constexpr bool PACKED = sizeof(S) == 2;
     const int nx = a.nx, ny = a.ny, nz = a.nz;
     const int nxy = nx * ny;
@@ -554,10 +556,7 @@ __device__ __forceinline__ float vec_loop(const StepArgs &a, float (*sacc)[9][BX
     // CPL); both are rebuilt here from the values already in registers
     const bool at_inlet = inout && x == 0;
     const bool at_outlet = inout && active && x + CPL == nx;
-    // pairs k of the warp's lanes among which a node is (the first or the last pairs)
-    auto pair_has_node = [&](int k) {
-        return inout && ((k == 0 && x0 == 0) || (k == CPL / 2 - 1 && x0 + BX * CPL >= nx));
-    };
+    const bool node_warp = inout && (x0 == 0 || x0 + BX * CPL >= nx);  // a boundary node among the warp's cells
     // y neighbours of this row (YEDGE rows only)
     bool ym_bb = false, yp_bb = false;
     int ym_off = nx, yp_off = -nx;  // element offset of the source row for c_y = +1 / -1 (subtracted)
@@ -652,80 +651,86 @@ __device__ __forceinline__ float vec_loop(const StepArgs &a, float (*sacc)[9][BX
             }
             sdr += drho;
         };
+        if (PACKED && !node_warp) {
+            // the lane's cells two at a time in packed FP32
 #pragma unroll
-        for (int k = 0; k < CPL / 2; ++k) {
-            const unsigned seed = seed_of(k);
-            if (PACKED && !pair_has_node(k)) {
-                // both cells of the pair in packed FP32
+            for (int k = 0; k < CPL / 2; ++k) {
+                const unsigned seed = seed_of(k);
                 float2 nuf = make_float2(1.0f, 1.0f);
                 if (SP && active) nuf = __ldg(reinterpret_cast<const float2 *>(a.spf + x + 2 * k));
                 auto pop = [&](int i) { return V::pair(v[i], k); };
                 const PairMoments m = pair_moments(pop);
                 float2 drho, ux, uy, uz;
-                collide_pair<REG, FORCE, SP>(m, pop, tau0, kq, nuf, Fx, Fy, Fz, [&](int i, float2 r) {
+                auto put = [&](int i, float2 r) {
                     if constexpr (SR) V::set_pair_rs(v[i], k, r.x, r.y, sr_bits(seed, i));
                     else V::set_pair(v[i], k, r.x, r.y);
-                }, drho, ux, uy, uz);
+                };
+                if constexpr (REG && !FORCE) collide_pair<SP>(m, tau0, kq, nuf, put, drho, ux, uy, uz);
+                else collide_pair_cell<REG, FORCE, SP>(m, pop, tau0, kq, nuf, Fx, Fy, Fz, put, drho, ux, uy, uz);
                 count(2 * k, drho.x, ux.x, uy.x, uz.x);
                 count(2 * k + 1, drho.y, ux.y, uy.y, uz.y);
-                continue;
             }
-            float upx = 0.f, upy = 0.f, upz = 0.f;  // velocity of the pair's first cell
-            float gp[Q];                            // its results
+        } else {
 #pragma unroll
-            for (int j = 2 * k; j < 2 * k + 2; ++j) {
-                float g[Q];
-                // boundary nodes of this cell (inlet x = 0 at j = 0, outlet x = nx-1 at the last j:
-                // rho = 1 and the velocity of the neighbour x = nx-2, the pair's first cell)
-                const bool in = j == 0 && at_inlet, out = j == CPL - 1 && at_outlet;
-                auto rebuild_node = [&](float (&gg)[Q]) {
-                    if (in) inlet_node(a, gg, (size_t)z * ny + y);
-                    if (out) rebuild<-1>(gg, 0.0f, upx, upy, upz);
-                };
-                float drho, ux, uy, uz;
-                const float nuf = SP && active ? __ldg(a.spf + x + j) : 1.0f;
-                if constexpr (MIXED) {
-                    // regularized collision of binary16 pairs: only the pair sums and
-                    // differences enter, formed with one conversion per pair
-                    float s[9], d[9], drho0;
-                    if (in || out) {
+            for (int k = 0; k < CPL / 2; ++k) {
+                const unsigned seed = seed_of(k);
+                float upx = 0.f, upy = 0.f, upz = 0.f;  // velocity of the pair's first cell
+                float gp[Q];                            // its results
 #pragma unroll
-                        for (int i = 0; i < Q; ++i) g[i] = V::cell(v[i], j);
-                        rebuild_node(g);
+                for (int j = 2 * k; j < 2 * k + 2; ++j) {
+                    float g[Q];
+                    // boundary nodes of this cell (inlet x = 0 at j = 0, outlet x = nx-1 at the last j:
+                    // rho = 1 and the velocity of the neighbour x = nx-2, the pair's first cell)
+                    const bool in = j == 0 && at_inlet, out = j == CPL - 1 && at_outlet;
+                    auto rebuild_node = [&](float (&gg)[Q]) {
+                        if (in) inlet_node(a, gg, (size_t)z * ny + y);
+                        if (out) rebuild<-1>(gg, 0.0f, upx, upy, upz);
+                    };
+                    float drho, ux, uy, uz;
+                    const float nuf = SP && active ? __ldg(a.spf + x + j) : 1.0f;
+                    if constexpr (MIXED) {
+                        // regularized collision of binary16 pairs: only the pair sums and
+                        // differences enter, formed with one conversion per pair
+                        float s[9], d[9], drho0;
+                        if (in || out) {
 #pragma unroll
-                        for (int p = 0; p < 9; ++p) {
-                            s[p] = g[2 * p + 1] + g[2 * p + 2];
-                            d[p] = g[2 * p + 1] - g[2 * p + 2];
+                            for (int i = 0; i < Q; ++i) g[i] = V::cell(v[i], j);
+                            rebuild_node(g);
+#pragma unroll
+                            for (int p = 0; p < 9; ++p) {
+                                s[p] = g[2 * p + 1] + g[2 * p + 2];
+                                d[p] = g[2 * p + 1] - g[2 * p + 2];
+                            }
+                            drho0 = g[0] + s[0];
+                        } else {
+#pragma unroll
+                            for (int p = 0; p < 9; ++p) {
+                                const float b = V::cell(v[2 * p + 2], j);
+                                s[p] = V::add_h(v[2 * p + 1], j, b);
+                                d[p] = V::sub_h(v[2 * p + 1], j, b);
+                            }
+                            drho0 = V::add_h(v[0], j, s[0]);
                         }
-                        drho0 = g[0] + s[0];
+                        collide_sd<REG, FORCE, SP>(g, s, d, drho0, tau0, kq, Fx, Fy, Fz, drho, ux, uy, uz, nuf);
                     } else {
 #pragma unroll
-                        for (int p = 0; p < 9; ++p) {
-                            const float b = V::cell(v[2 * p + 2], j);
-                            s[p] = V::add_h(v[2 * p + 1], j, b);
-                            d[p] = V::sub_h(v[2 * p + 1], j, b);
-                        }
-                        drho0 = V::add_h(v[0], j, s[0]);
+                        for (int i = 0; i < Q; ++i) g[i] = V::cell(v[i], j);
+                        if (in || out) rebuild_node(g);
+                        collide<REG, FORCE, SP>(g, tau0, kq, Fx, Fy, Fz, drho, ux, uy, uz, nuf);
                     }
-                    collide_sd<REG, FORCE, SP>(g, s, d, drho0, tau0, kq, Fx, Fy, Fz, drho, ux, uy, uz, nuf);
-                } else {
+                    upx = ux;
+                    upy = uy;
+                    upz = uz;
+                    // the first cell waits in FP32; the second completes the pair, which
+                    // replaces the pair's (already read) inputs
 #pragma unroll
-                    for (int i = 0; i < Q; ++i) g[i] = V::cell(v[i], j);
-                    if (in || out) rebuild_node(g);
-                    collide<REG, FORCE, SP>(g, tau0, kq, Fx, Fy, Fz, drho, ux, uy, uz, nuf);
+                    for (int i = 0; i < Q; ++i) {
+                        if (j == 2 * k) gp[i] = g[i];
+                        else if constexpr (SR) V::set_pair_rs(v[i], k, gp[i], g[i], sr_bits(seed, i));
+                        else V::set_pair(v[i], k, gp[i], g[i]);
+                    }
+                    count(j, drho, ux, uy, uz);
                 }
-                upx = ux;
-                upy = uy;
-                upz = uz;
-                // the first cell waits in FP32; the second completes the pair, which
-                // replaces the pair's (already read) inputs
-#pragma unroll
-                for (int i = 0; i < Q; ++i) {
-                    if (j == 2 * k) gp[i] = g[i];
-                    else if constexpr (SR) V::set_pair_rs(v[i], k, gp[i], g[i], sr_bits(seed, i));
-                    else V::set_pair(v[i], k, gp[i], g[i]);
-                }
-                count(j, drho, ux, uy, uz);
             }
         }
         // (in place, even steps: the quads go through shuffles of the whole warp)
