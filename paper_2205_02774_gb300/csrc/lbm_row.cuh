@@ -5,12 +5,15 @@
 // x neighbours are the same runs one element to the side (no shuffle, no halo
 // case).  What keeps the bytes in flight that an aligned vector keeps is CPL
 // independent loads per population (FP32 2, binary16 4, whose pairs of cells go
-// through the packed collision).  One cell per thread in whole-column blocks took
-// 88 us per step on 385x65x97 FP32 and 742 on 767x127x191, this loop 68 and 458
-// (55 and 423 at the copy rate); it is kept for lattices beyond 32-bit element
-// offsets only.  What is left is the odd alignment (a run of 32 lanes touches one
-// sector more than it fills) and, for binary16, 2-byte accesses (767x127x191 317 us
-// of 211).
+// through the packed collision).  One cell per thread in whole-column blocks, kept
+// for lattices beyond 32-bit element offsets only, and this loop, us per step:
+//                        385x65x97     767x127x191
+//   FP32                 93 -> 66      733 -> 452    (55 and 423 at the copy rate)
+//   binary16             70 -> 54      464 -> 323    (28 and 211)
+//   stochastic rounding  73 -> 69      484 -> 385
+//   the same, BGK        74 -> 72      483 -> 400
+// What is left is the odd alignment (a run of 32 lanes touches one sector more than
+// it fills) and, for binary16, issue: 2-byte accesses and a random word per cell.
 #pragma once
 
 #include <cuda_fp16.h>
@@ -199,10 +202,13 @@ __device__ __forceinline__ float row_loop(const StepArgs &a, float (*sacc)[9][32
         if constexpr (PACKED) {
 #pragma unroll
             for (int k = 0; k < CPL / 2; ++k) {
+                // a last chunk of up to 64 cells (385 = 3 x 128 + 1): one pair per lane, not two
+                // (stochastic rounding 71.5 -> 69.1 us per step, BGK 76.1 -> 71.8)
+                if (k > 0 && x0 + 64 * k >= nx) continue;
                 // stochastic rounding: each cell has its own seed, its bits the low 13 of a word
                 const unsigned s0 = SR ? sr_seed((unsigned)here + 64 * k, tmix) : 0u;
                 const unsigned s1 = SR ? sr_seed((unsigned)here + 64 * k + 32, tmix) : 0u;
-                auto bits = [&](int i) { return __byte_perm(sr_bits(s0, i), sr_bits(s1, i), 0x5410); };
+                auto bits = [&](int i) { return sr_bits_low2(s0, s1, i); };
                 const float2 nuf = make_float2(nu_factor(2 * k), nu_factor(2 * k + 1));
                 const bool nodes = has_inlet(2 * k) || has_outlet(2 * k) || has_outlet(2 * k + 1);
                 // the lane of an inlet / outlet node keeps the pair's inputs (in shared

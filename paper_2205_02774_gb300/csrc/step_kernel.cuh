@@ -103,6 +103,14 @@ __device__ __forceinline__ unsigned sr_bits(unsigned seed, int i)
     const unsigned long long p = (unsigned long long)(seed ^ (0x9E3779B9u * (unsigned)(i + 1))) * 0xD168AAADull;
     return (unsigned)(p >> 16);
 }
+// The low halves of two seeds' words in one: they are bits 16-31 of the products,
+// so 32-bit products do (row lanes, 385x65x97: 71.5 us per step, 75.2 with the two
+// words cut together; 767x127x191: 390 and 411).
+__device__ __forceinline__ unsigned sr_bits_low2(unsigned seed0, unsigned seed1, int i)
+{
+    const unsigned k = 0x9E3779B9u * (unsigned)(i + 1);
+    return __byte_perm((seed0 ^ k) * 0xD168AAADu, (seed1 ^ k) * 0xD168AAADu, 0x7632);
+}
 // one binary16 by stochastic rounding (the low half of the pair conversion)
 __device__ __forceinline__ void st_half_rs(__half *p, float g, unsigned rb)
 {
@@ -822,7 +830,7 @@ constexpr int INNER = 0, ANY = 1;
 // registers with binary16 quads (20 warps per SM: with 8-byte row pieces those
 // warps keep as many bytes in flight as FP32) and, unforced, 64 with pairs (32
 // warps per SM); BGK, forced and sampling pairs get 80; BGK and sampling quads 128
-// (BGK FP16-SR on 768x128x192 260 us per step, 274 with the spills of 96 and as
+// (BGK FP16-SR on 768x128x192 263 us per step, 274 with the spills of 96 and as
 // pairs), as do the launches of any rows (the wall rows beside the inner launch,
 // all rows of a lattice too small to fill the GPU), so that they need no stack frame.
 template <int CPL, bool STATS>
