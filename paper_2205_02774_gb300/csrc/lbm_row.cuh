@@ -182,7 +182,7 @@ __device__ __forceinline__ float row_loop(const StepArgs &a, float (*sacc)[9][32
         auto count = [&](int j, float drho, float ux, float uy, float uz) {
             if (!on(j)) return;
             if (STATS) {
-                float *sp = &sacc[wi][0][32 * j + lane];
+                float *sp = &sacc[wi][0][stat_slot<ROW, CPL>(lane, j)];
                 constexpr int L = 32 * CPL;
                 sp[0 * L] += ux; sp[1 * L] += uy; sp[2 * L] += uz;
                 sp[3 * L] = __fmaf_rn(ux, ux, sp[3 * L]); sp[4 * L] = __fmaf_rn(uy, uy, sp[4 * L]);

@@ -51,6 +51,15 @@ constexpr int PULL = 0, AA_SHIFT = 1, AA_LOCAL = 2;
 // two lattices as PULL, lanes 32 cells apart (lbm_row.cuh)
 constexpr int ROW = 3;
 
+// Slot of the lane's cell j in the per-thread statistics sums, by cell of the warp's
+// chunk.  A lane clears the slots that it alone adds to; the block's barrier comes
+// only after the plane loop.
+template <int MODE, int CPL>
+__host__ __device__ constexpr int stat_slot(int lane, int j)
+{
+    return MODE == ROW ? 32 * j + lane : CPL * lane + j;
+}
+
 // the place of this step's plane in StepArgs::ubc; the step index is read again
 // (an L1 hit, by the lanes that hold an inlet node) rather than kept in a
 // register over the plane loop, which several instances would spill for
@@ -650,7 +659,7 @@ __device__ __forceinline__ float vec_loop(const StepArgs &a, float (*sacc)[9][BX
                 // explicit fused multiply-adds: every kernel instance rounds the sums
                 // alike (the compiler would otherwise fuse them or not depending on
                 // how it shares the products with the collision)
-                float *sp = &sacc[wi][0][CPL * lane + j];
+                float *sp = &sacc[wi][0][stat_slot<MODE, CPL>(lane, j)];
                 constexpr int L = BX * CPL;
                 sp[0 * L] += ux; sp[1 * L] += uy; sp[2 * L] += uz;
                 sp[3 * L] = __fmaf_rn(ux, ux, sp[3 * L]); sp[4 * L] = __fmaf_rn(uy, uy, sp[4 * L]);
@@ -870,7 +879,7 @@ __global__ void __launch_bounds__(BX *block_warps<CPL, STATS>(), warps_per_sm<CP
 #pragma unroll
         for (int q = 0; q < 9; ++q)
 #pragma unroll
-            for (int j = 0; j < CPL; ++j) sacc[wi][q][CPL * lane + j] = 0.f;
+            for (int j = 0; j < CPL; ++j) sacc[wi][q][stat_slot<MODE, CPL>(lane, j)] = 0.f;
     }
     float sdr;
     const bool edge = ROWS == ANY && (y == 0 || y == ny - 1);
