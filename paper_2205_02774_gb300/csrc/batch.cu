@@ -363,8 +363,6 @@ int stg_batch_step(stg_batch *b, int64_t n)
         if (rc) return bfail(b, rc, "member " + std::to_string(d) + ": " + h->err);
     }
     if (b->m.empty() || n == 0) return STG_OK;
-    std::vector<int64_t> t_before(b->m.size());
-    for (size_t d = 0; d < b->m.size(); ++d) t_before[d] = b->m[d]->t;
     int rc = order_after_members(b);
     if (rc) return rc;
     while (n >= b->B) {
@@ -399,7 +397,7 @@ int stg_batch_step(stg_batch *b, int64_t n)
     rc = order_members_after(b);
     if (rc) return rc;
     for (size_t d = 0; d < b->m.size(); ++d) {
-        rc = queue_check_readback(b->m[d], t_before[d]);
+        rc = queue_check_readback(b->m[d]);
         if (rc) return bfail(b, rc, "member " + std::to_string(d) + ": " + b->m[d]->err);
     }
     return STG_OK;

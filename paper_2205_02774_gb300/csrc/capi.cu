@@ -673,14 +673,15 @@ namespace {
 namespace stg {
 namespace host {
 
-int queue_check_readback(stg_lbm *h, int64_t t_before)
+int queue_check_readback(stg_lbm *h)
 {
-    // only when a check step has run: the result of an earlier one is on its way already
-    if (h->d.check_every > 0 && h->t / h->d.check_every > t_before / h->d.check_every) {
+    // only when a check step has run since the last read-back was queued
+    if (h->d.check_every > 0 && h->t / h->d.check_every > h->t_read / h->d.check_every) {
         CK(cudaMemcpyAsync(h->h_pinned, h->mass_out, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
         CK(cudaEventRecord(h->ev_check, h->stream));
         h->check_pending = true;
     }
+    h->t_read = h->t;
     return STG_OK;
 }
 
@@ -769,6 +770,7 @@ int reset_counters(stg_lbm *h, int64_t step)
     }
     CK(cudaStreamSynchronize(h->stream));
     h->t = step;
+    h->t_read = step;
     h->t0_stats = step;
     h->check_pending = false;
     h->sticky = STG_OK;
@@ -1023,7 +1025,6 @@ int stg_lbm_step(stg_lbm *h, int64_t n)
     int rc = poll_check(h);
     if (rc) return rc;
     if (h->sticky) return fail(h, h->sticky, "an earlier check failed; reset the state first");
-    const int64_t t_before = h->t;
     const int per = h->d.stats_every;
     while (n > 0) {
         cudaGraphExec_t g;
@@ -1040,7 +1041,7 @@ int stg_lbm_step(stg_lbm *h, int64_t n)
         h->t += k;
         n -= k;
     }
-    return queue_check_readback(h, t_before);
+    return queue_check_readback(h);
 }
 
 int stg_lbm_step_timed(stg_lbm *h, int64_t n, double *ms_step, double *ms_inlet)
@@ -1065,6 +1066,7 @@ int stg_lbm_step_timed(stg_lbm *h, int64_t n, double *ms_step, double *ms_inlet)
         if (e != cudaSuccess) rc = cuda_fail(h, e, "timed step launch");
         else h->t += 1;
     }
+    if (rc == STG_OK) rc = queue_check_readback(h);
     if (rc == STG_OK) rc = wait_stream(h);
     double sum_s = 0.0, sum_i = 0.0;
     if (rc == STG_OK) {
@@ -1390,7 +1392,6 @@ int stg_lbm_step_probed(stg_lbm *h, int64_t n, float *u_host)
         h->probe_cap = need;
     }
     // where the call's samples go (the words are free again: the call waits for its work)
-    const int64_t t_before = h->t;
     struct {
         long long t;
         float *out;
@@ -1412,7 +1413,7 @@ int stg_lbm_step_probed(stg_lbm *h, int64_t n, float *u_host)
         s += 1;
         CK(enqueue_probes(h, h->t, h->stream));
     }
-    rc = queue_check_readback(h, t_before);
+    rc = queue_check_readback(h);
     if (rc) return rc;
     CK(cudaMemcpyAsync(u_host, h->probe_buf, sizeof(float) * need, cudaMemcpyDeviceToHost, h->stream));
     return wait_stream(h);

@@ -55,6 +55,7 @@ struct stg_lbm {
     cudaEvent_t ev_pfork = nullptr, ev_pjoin[2] = {nullptr, nullptr};  // probes beside the next step
     bool check_pending = false;
     int64_t t = 0, t0_stats = 0;
+    int64_t t_read = 0;  // the read-backs of the mass checks before this step index are queued
     double mass0 = 0.0;
     int sticky = STG_OK;
     std::string err;
@@ -94,9 +95,9 @@ cudaError_t enqueue_steps(stg_lbm *h, int64_t t, int n, bool probed = false);
 bool is_stats_step(const stg_lbm *h, int64_t t);
 // evaluate the last completed mass check (non-blocking)
 int poll_check(stg_lbm *h);
-// after the steps that took h from t_before to h->t were enqueued on
-// h->stream: queue the read-back of the last mass check, if one ran
-int queue_check_readback(stg_lbm *h, int64_t t_before);
+// after steps were enqueued on h->stream: queue the read-back of the last mass
+// check, if one ran since the last call
+int queue_check_readback(stg_lbm *h);
 // wait for h->stream (bounded by the handle's timeout)
 int wait_stream(stg_lbm *h);
 // one plain (non-sampling) step pass from the current state with `tile`, on
