@@ -592,15 +592,17 @@ int capture_all(stg_lbm *h)
     int rc = STG_OK;
     const int64_t shared = h->in_flight;
     h->in_flight = 0;  // these graphs run the lattice alone
-    // one full cycle of step indices: parities and sampling flags that never meet
-    // (with an even sampling period, half of them) need no graph
-    const int k = std::max(h->d.stats_every, 1);
-    for (int64_t t = 0; t < 2 * (int64_t)k && rc == STG_OK; ++t) {
+    // the first step of each parity and of each parity's samples (every k-th step
+    // samples, the first of them step k - 1); parities and sampling flags that never
+    // meet (with an even sampling period, half of them) need no graph
+    const int64_t k = std::max(h->d.stats_every, 1);
+    for (int64_t t : {int64_t(0), int64_t(1), k - 1, 2 * k - 1}) {
         cudaGraphExec_t &g = h->g_single[t & 1][is_stats_step(h, t) ? 1 : 0];
-        if (!g) rc = capture(h, t, 1, &g);
-        if (rc == STG_OK && h->block_steps > 0 && t % k == 0 && !h->g_block[t & 1])
-            rc = capture(h, t, h->block_steps, &h->g_block[t & 1]);
+        if (rc == STG_OK && !g) rc = capture(h, t, 1, &g);
     }
+    for (int64_t t : {int64_t(0), k})
+        if (rc == STG_OK && h->block_steps > 0 && !h->g_block[t & 1])
+            rc = capture(h, t, h->block_steps, &h->g_block[t & 1]);
     h->in_flight = shared;
     if (rc == STG_OK) rc = capture_probed(h);
     return rc;
