@@ -49,8 +49,8 @@ __global__ void __launch_bounds__(INLET_J * INLET_WARPS, 2) stg_inlet_kernel(con
     const int lane = threadIdx.x, w = threadIdx.y;
     const int tid = w * INLET_J + lane;
     const int ny = a.ny, nz = a.nz, N = a.N, T = a.planes;
-    const int j0 = blockIdx.x * INLET_J;
-    const int k0 = blockIdx.y * kb;   // the block's span nodes k0 .. k0 + kb - 1; item q = (k0 + q / T, step q % T)
+    const int j0 = blockIdx.y * INLET_J;
+    const int k0 = blockIdx.x * kb;   // the block's span nodes k0 .. k0 + kb - 1; item q = (k0 + q / T, step q % T)
     const int items = kb * T;         // <= ITEMS
     const float af = a.a_filter, bf = 1.0f - a.a_filter;
     const size_t plane = (size_t)ny * nz;
@@ -174,8 +174,8 @@ cudaError_t launch_inlet(const InletArgs &a, cudaStream_t s)
     if (a.planes < 1 || a.planes > INLET_MAX_PLANES) return cudaErrorInvalidValue;
     const int ipw = a.planes > INLET_WARPS ? 4 : 1;
     const int kb = ipw * INLET_WARPS / a.planes;
-    const dim3 grid((a.ny + INLET_J - 1) / INLET_J, (a.nz + kb - 1) / kb);
-    if (grid.y > 65535u) return cudaErrorInvalidConfiguration;
+    // span nodes along x: nz may be longer than the 65535 blocks of the other axes (ny may not)
+    const dim3 grid((a.nz + kb - 1) / kb, (a.ny + INLET_J - 1) / INLET_J);
     const dim3 block(INLET_J, INLET_WARPS);
     if (ipw == 4) stg_inlet_kernel<4><<<grid, block, 0, s>>>(a, kb);
     else stg_inlet_kernel<1><<<grid, block, 0, s>>>(a, kb);
