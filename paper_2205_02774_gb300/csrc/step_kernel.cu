@@ -50,7 +50,7 @@ int stat_group(int nx, int ny, int nz)
     const long long rows = (long long)((nx + 2 * BX - 1) / (2 * BX)) * ny;
     int g = 32;
     while (g > STAT_WARPS && rows * ((nz + g - 1) / g) * STAT_WARPS < 152LL * 32 * 3 / 2 && nz / (g / 2) < 65535) g /= 2;
-    return g;
+    return std::max(g, (nz + 65534) / 65535);  // a launch holds 65535 runs
 }
 
 // FP32 lattices with fewer than 4 cells per resident lane (32 warps per SM): one

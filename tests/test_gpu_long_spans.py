@@ -3,9 +3,9 @@ nz that the lattice's sizes allow, more blocks along z than a grid's 65 535 rows
 import numpy as np
 import pytest
 
-from workloads import case
+from workloads import case, perturbed_equilibrium_field
 
-from gpu_helpers import require_cuda, pair
+from gpu_helpers import require_cuda, pair, max_rel, normwise
 
 pytestmark = pytest.mark.gpu
 
@@ -26,4 +26,22 @@ def test_inlet_planes(nz):
     orc.step(26)
     u, u_or = gpu.inlet(), orc.inlet()
     assert np.abs(u - u_or).max() <= 1e-5 * np.abs(u_or).max()
+    gpu.close()
+
+
+@pytest.mark.parametrize("nx", [1, 4])
+def test_sampling_runs(nx):
+    nz = 65535 * 32 + 3
+    c = SMALL.with_(nx=nx, ny=1, nz=nz, bc_x="periodic", bc_y="periodic", stats_every=1)
+    gpu, orc = pair(c)
+    st = gpu.encode(perturbed_equilibrium_field(nx, 1, nz, seed=nx))
+    gpu.set_state(st, 0)
+    orc.set_pops(gpu.decode(st))
+    gpu.step(1)
+    orc.step(1)
+    assert max_rel(gpu.populations(), orc.pops()) < 1e-5
+    s = gpu.stats()
+    m, r, n = orc.stats()
+    assert s["n_samples"] == n == 1
+    assert normwise(s["mean_sum"], m) < 1e-4 and normwise(s["rey_sum"], r) < 1e-4
     gpu.close()
