@@ -353,10 +353,13 @@ int stat_runs(int nx, int ny, int nz)
 
 size_t plane_floats(const stg_lbm *h) { return 3 * (size_t)h->d.ny * h->d.nz; }
 
+// inlet planes that a lattice keeps: without an inlet one, which stays zero
+int ubc_planes(const stg_domain &d) { return d.bc_x == STG_BC_X_INLET_OUTLET ? stg::INLET_RING : 1; }
+
 // inlet plane of step t
 float *ubc_plane(const stg_lbm *h, int64_t t)
 {
-    return h->ubc + (size_t)(t & (stg::INLET_RING - 1)) * plane_floats(h);
+    return h->ubc + (size_t)(t & (ubc_planes(h->d) - 1)) * plane_floats(h);
 }
 
 // where the populations of the current state live (for probes and block reads)
@@ -920,7 +923,7 @@ int stg_lbm_create(const stg_domain *domain, const stg_rans_profile *rans, const
     h->aa = domain->streaming == STG_STREAM_AA;
     h->lat[0] = dalloc(h, 19 * h->P * h->elem);
     h->lat[1] = h->aa ? h->lat[0] : dalloc(h, 19 * h->P * h->elem);  // in place: one lattice
-    h->ubc = (float *)dalloc(h, sizeof(float) * stg::INLET_RING * plane_floats(h));
+    h->ubc = (float *)dalloc(h, sizeof(float) * ubc_planes(*domain) * plane_floats(h));
     h->uf = (float *)dalloc(h, sizeof(float) * 3 * (size_t)ny * nz);
     h->ctl = (StepCtl *)dalloc(h, sizeof(StepCtl));
     h->stat_mean = (double *)dalloc(h, sizeof(double) * 3 * (size_t)nx * ny);
@@ -961,7 +964,7 @@ int stg_lbm_create(const stg_domain *domain, const stg_rans_profile *rans, const
     e = cudaMemsetAsync(h->mass_counter, 0, sizeof(unsigned) * mass_counters(nx, ny, nz), h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->m_counter, 0, sizeof(unsigned) * 4, h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->mass_out, 0, sizeof(double) * 2, h->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->ubc, 0, sizeof(float) * stg::INLET_RING * plane_floats(h), h->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(h->ubc, 0, sizeof(float) * ubc_planes(*domain) * plane_floats(h), h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->uf, 0, sizeof(float) * 3 * (size_t)ny * nz, h->stream);
     if (e != cudaSuccess) {
         cuda_fail(h, e, "cudaMemsetAsync");
@@ -1001,7 +1004,7 @@ int stg_lbm_estimate_bytes(const stg_domain *d, const stg_params *p, int64_t *by
     const double nx = d->nx, ny = d->ny, nz = d->nz, P = nx * ny * nz;
     const double elem = d->storage == STG_FP32 ? 4.0 : 2.0;
     const double lattices = d->streaming == STG_STREAM_AA ? 1.0 : 2.0;
-    double b = lattices * r(19 * P * elem) + r(12.0 * stg::INLET_RING * ny * nz) + r(12 * ny * nz) + r(sizeof(StepCtl)) + r(24 * nx * ny) + r(48 * nx * ny) +
+    double b = lattices * r(19 * P * elem) + r(12.0 * ubc_planes(*d) * ny * nz) + r(12 * ny * nz) + r(sizeof(StepCtl)) + r(24 * nx * ny) + r(48 * nx * ny) +
                r(8.0 * mass_slots(d->nx, d->ny, d->nz)) + r(4.0 * mass_counters(d->nx, d->ny, d->nz)) + 3 * r(16) +
                r(8.0 * stg::mass_grid_blocks());
     if (d->sponge_len > 0.0) b += r(4 * nx);

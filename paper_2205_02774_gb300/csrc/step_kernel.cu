@@ -33,11 +33,13 @@ bool launch_f32_reg(const StepArgs &, bool, cudaStream_t, cudaStream_t),
     launch_f16sr_reg_row(const StepArgs &, bool, cudaStream_t, cudaStream_t),
     launch_f16sr_bgk_row(const StepArgs &, bool, cudaStream_t, cudaStream_t);
 
+// One plane and 32 cells per item, at most the 65535 runs of a launch per row; lattices
+// beyond 32-bit element offsets take one cell per thread in whole columns.
 int step_grid_blocks(int nx, int ny, int nz)
 {
-    const long long vec = (long long)((nx + BX - 1) / BX) * ny * nz;  // one plane and 32 cells per item
     const long long col = (long long)((nx + BX - 1) / BX) * ny;
-    return (int)((vec > col ? vec : col) + 2LL * ny + 64);
+    const long long runs = 19.0 * nx * ny * nz < 4294967296.0 ? std::min(nz, 65535) : 1;
+    return (int)(col * runs + 2LL * ny + 64);
 }
 
 // The longer a run, the less scratch a sampling step writes and reads (36 B each
