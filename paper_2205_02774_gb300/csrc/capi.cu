@@ -1370,9 +1370,14 @@ int stg_lbm_set_probes(stg_lbm *h, int32_t n, const int32_t *xyz)
     int rc = wait_stream(h);
     if (rc) return rc;
     if (n > h->n_probes || !h->probe_xyz) {
-        h->probe_xyz = (int *)dalloc(h, sizeof(int) * 3 * (size_t)std::max(n, 1));
-        if (!h->probe_xyz) return fail(h, STG_ERR_NOMEM, "probe table");
+        int *table = (int *)dalloc(h, sizeof(int) * 3 * (size_t)std::max(n, 1));
+        if (!table) return fail(h, STG_ERR_NOMEM, "probe table");  // the earlier probes stay
+        h->probe_xyz = table;
     }
+    // until the new probes are in place there are none: no graph and no step of an
+    // earlier set runs against the new table
+    h->n_probes = 0;
+    capture_probed(h);
     if (n > 0) CK(cudaMemcpy(h->probe_xyz, xyz, sizeof(int) * 3 * (size_t)n, cudaMemcpyHostToDevice));
     h->n_probes = n;
     return capture_probed(h);
