@@ -149,8 +149,8 @@ class Channel:
         return A.stg_lbm_autotune(self.h, trial_passes)
 
     def set_probes(self, xyz):
-        self._n_probes = int(np.asarray(xyz).reshape(-1, 3).shape[0])
         A.stg_lbm_set_probes(self.h, xyz)
+        self._n_probes = int(np.asarray(xyz).reshape(-1, 3).shape[0])  # (a refused set leaves the earlier one)
 
     def step_probed(self, n):
         """n steps; returns the probe velocities after each, shape (n, n_probes, 3)."""
