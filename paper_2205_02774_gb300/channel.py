@@ -96,6 +96,8 @@ class Channel:
     ``profile`` needs attributes y_c, U, k, eps, R (n x 6), U_bulk, nu_phys,
     h_phys (a RANS interface profile in physical units)."""
 
+    _n_probes = 0
+
     def __init__(self, nx, ny, nz, *, profile=None, tau0=0.52, c_smag=0.01, force=(0.0, 0.0, 0.0),
                  storage="fp32", collision="regularized", bc_x="stg", bc_y="walls", stats_every=0,
                  check_every=0, mass_tol=0.0, n_modes=100, C_l=3.0, alpha=0.01, t_filter=0.0,
