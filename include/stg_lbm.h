@@ -260,17 +260,20 @@ int stg_lbm_device_state(stg_lbm *h, void **pops, float **inlet_u);
 int stg_lbm_info(const stg_lbm *h, stg_info *out);
 
 /* Launch tile of the plain (non-sampling) steps of the vector step kernels
- * (lattices with even nx; other lattices ignore it).  The paper fixes no
+ * (lattices with even nx >= 4; other lattices ignore it).  The paper fixes no
  * kernel decomposition: the tile changes only how the lattice is cut into
  * thread blocks, never the arithmetic of a cell, so every tile gives
  * bit-identical populations and statistics (the FP64 mass of a check can
  * differ in its last bits, its block partials being summed in another order).
- *   interior_layout  0 or 1 (both stand for the same layout: one warp per x chunk of 64
- *                    cells, 128 for binary16 regularized unforced lattices with nx a
- *                    multiple of 4)
- *   interior_zc      z planes per warp of the rows 1..ny-2 at most (0: the whole z column,
- *                    else >= 4); the launches take fewer where that leaves warps without work
- *   wall_zc          the same for the wall rows y = 0, ny-1 (0 or >= 4)
+ *   interior_layout  1: a warp walks a whole z chunk; 0: 8 warps share it.  A warp's row
+ *                    piece is 32 cells (FP32 lattices of fewer than 622592 cells), 64, or
+ *                    128 (binary16, nx a multiple of 4)
+ *   interior_zc      z planes per chunk of the rows 1..ny-2, or of all rows on lattices
+ *                    small enough for one launch (0: the whole z column, else >= 4)
+ *   wall_zc          z planes per chunk of the wall rows y = 0, ny-1, which 8 warps
+ *                    share (0 or >= 4)
+ * With the default chunks the launches choose the planes per warp by the lattice's
+ * size: {1, 8, x} for the inner rows, 24 for the wall rows.
  * Default {1, 8, 24}. */
 typedef struct {
     int32_t interior_layout;
@@ -297,7 +300,9 @@ int stg_lbm_step_probed(stg_lbm *h, int64_t n, float *u_host);
 
 /* Autotuner: time every candidate tile on this lattice (`trial_passes` >= 1
  * plain step passes each, CUDA events on the handle's stream, after one
- * warm-up pass), keep the fastest and store it in *chosen (may be NULL).
+ * warm-up pass; tiles that stand for the same launches once), keep the fastest,
+ * or the default tile unless another is faster by more than 1 %, and store it in
+ * *chosen (may be NULL).
  * The trial passes recompute the next state from the current one without
  * advancing the step counter, the inlet filter or the statistics, so tuning
  * leaves the simulation's results unchanged.  An in-place lattice's trial
@@ -359,7 +364,7 @@ int stg_batch_step(stg_batch *b, int64_t n);
 int stg_batch_sync(stg_batch *b);
 /* Autotuner for the batch: every candidate tile is timed over `trial_passes`
  * concurrent plain passes of all members (no state advance, as in
- * stg_lbm_autotune); the fastest is set on every member. */
+ * stg_lbm_autotune); the one chosen as there is set on every member. */
 int stg_batch_autotune(stg_batch *b, int32_t trial_passes, stg_tile *chosen);
 /* Release the members (they stay alive) and the batch (NULL-safe). */
 void stg_batch_destroy(stg_batch *b);

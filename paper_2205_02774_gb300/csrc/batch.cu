@@ -429,8 +429,11 @@ int stg_batch_autotune(stg_batch *b, int32_t trial_passes, stg_tile *chosen)
         if (rc) return bfail(b, rc, "member " + std::to_string(d) + ": " + b->m[d]->err);
     }
     stg_tile best = b->m[0]->tile;
-    float best_ms = -1.f;
+    float best_ms = 0.f, own_ms = 0.f;
     for (int c = 0; c < ncand; ++c) {
+        bool same = c > 0;  // the same launches as the members' own rules
+        for (stg_lbm *h : b->m) same = same && tile_inner_run(h, cand[c]) == tile_inner_run(h, cand[0]);
+        if (same) continue;
         // all members' plain passes from their current states, concurrently
         // (no state advance; see stg_lbm_autotune)
         for (int k = 0; k <= trial_passes; ++k) {
@@ -447,10 +450,11 @@ int stg_batch_autotune(stg_batch *b, int32_t trial_passes, stg_tile *chosen)
         BCK(cudaEventSynchronize(b->e1));
         float ms = 0.f;
         BCK(cudaEventElapsedTime(&ms, b->e0, b->e1));
-        if (best_ms < 0.f || ms < best_ms) {
+        if (better_tile(c, ms, best_ms, own_ms)) {
             best_ms = ms;
             best = cand[c];
         }
+        if (c == 0) own_ms = ms;
     }
     rc = order_members_after(b);
     if (rc) return rc;

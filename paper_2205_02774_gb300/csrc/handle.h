@@ -115,6 +115,11 @@ int restore_trial_state(stg_lbm *h, const std::vector<unsigned char> &pops, cons
 int apply_tile(stg_lbm *h, const stg_tile &tile);
 // the autotuner's candidate tiles
 const stg_tile *tile_candidates(int *n);
+// planes per warp of the inner rows with `tile`
+int tile_inner_run(stg_lbm *h, const stg_tile &tile);
+// whether candidate c, the first of them the lattice's own rule, replaces the best so far:
+// the own rule stays unless another is faster by more than the noise of such a trial
+bool better_tile(int c, float ms, float best_ms, float own_ms);
 // take h out of its batch (batch.cu)
 void batch_detach(stg_lbm *h);
 

@@ -40,7 +40,8 @@ struct StepArgs {
     int il, ir;             // 32-wide x chunks [il, ir) of rows 1..ny-2 belong to the interior kernel
     int interior;           // interior kernel: 0 best available, 1 one cell per thread, 2 cell pairs
     int aa;                 // 1: one lattice updated in place (AA pattern; src == dst), 0: two lattices
-    // z planes per run of the plain (non-sampling) vector launches at most, inner / wall rows (0: the whole z column)
+    // z planes per run of the plain (non-sampling) vector launches, inner / wall rows: the
+    // set tile's, 0 by the lattice's size (run_planes); in a launch its own
     int tile_zc, tile_wall_zc;
     int row_step;           // vector launches of the rows 0, row_step, ...
     int stat_group;         // z planes per run of the sampling vector launches
@@ -113,7 +114,7 @@ inline bool vector_fits(const StepArgs &a)
 // Whether a pass of the vector kernels (cpl cells per lane) is one launch of all
 // rows, and the z planes per run of its launches (step_kernel.cu).
 bool one_launch(const StepArgs &a, int cpl);
-int run_planes(const StepArgs &a, int cpl, int tile_zc, int elem, bool walls);
+int run_planes(const StepArgs &a, int cpl, int elem, bool walls);
 // cells per lane of the vector kernels, and whether they lie 32 apart
 int lane_cells(const StepArgs &a, int storage);
 bool row_lanes(const StepArgs &a, int storage);
@@ -139,8 +140,9 @@ cudaError_t launch_probe(const void *src, int storage, const LatticeView &lv, in
 cudaError_t launch_gather_block(const void *src, int storage, const LatticeView &lv, int x0, int y0, int z0, int bx,
                                 int by, int bz, void *out, cudaStream_t s);
 
-// shortest z chunk that set_tile accepts
-constexpr int MIN_ZC = 4;
+// Tiles: shortest z chunk that set_tile accepts; the default chunks (layout 1), which
+// leave the runs to run_planes; warps that share a chunk of layout 0 or of the wall rows.
+constexpr int MIN_ZC = 4, DEFAULT_ZC = 8, DEFAULT_WALL_ZC = 24, TILE_WARPS = 8;
 // z planes per run on sampling steps of the vector kernels, walked by STAT_WARPS
 // warps: a function of the lattice alone, so the statistics do not depend on the
 // launch tile

@@ -104,15 +104,17 @@ bool one_launch(const StepArgs &a, int cpl)
 // The wall rows, beside the inner launch, are spread over as many warps as their
 // latency needs: binary16 1, FP32 4 (768x128x192: FP16 226, 228, 230 us with
 // 1, 2, 4, and 236 with 24; FP32 420, 420, 418), and 4 among the members of a batch.
-int run_planes(const StepArgs &a, int cpl, int tile_zc, int elem, bool walls)
+// A tile that was set sets the runs instead.
+int run_planes(const StepArgs &a, int cpl, int elem, bool walls)
 {
-    const int most = tile_zc > 0 ? tile_zc : a.nz;
     const int least = (a.nz + 65534) / 65535;  // a launch holds 65535 runs
-    if (walls) return std::max(least, std::min(most, elem == 4 || a.in_flight > a.P ? 4 : 1));
+    const int tile = walls ? a.tile_wall_zc : a.tile_zc;
+    if (tile > 0) return std::max(least, std::min(tile, a.nz));
+    if (walls) return std::max(least, std::min(a.nz, elem == 4 || a.in_flight > a.P ? 4 : 1));
     const long long per_warp = items_of(a, cpl) / (152 * (elem == 4 ? 32 : 20));
     int zc = 1;
     while (zc < (elem == 4 ? 2 : 8) && per_warp >= 5 * zc) zc *= 2;
-    return std::max(least, std::min(zc, most));
+    return std::max(least, std::min(zc, a.nz));
 }
 
 // Adds the z-group sums of a sampling step to the FP64 statistics, group by

@@ -984,8 +984,8 @@ static void launch_vec(StepArgs a, bool stats, cudaStream_t s, cudaStream_t side
         if ((chunks + k - 1) / k * k < (chunks + nw - 1) / nw * nw) nw = k;
     const bool one = one_launch(a, CPL);
     StepArgs w = a;
-    a.tile_zc = stats ? a.stat_group : run_planes(a, CPL, a.tile_zc, sizeof(S), false);
-    w.tile_zc = stats ? a.stat_group : run_planes(a, CPL, a.tile_wall_zc, sizeof(S), true);
+    a.tile_zc = stats ? a.stat_group : run_planes(a, CPL, sizeof(S), false);
+    w.tile_zc = stats ? a.stat_group : run_planes(w, CPL, sizeof(S), true);
     if (stats) nw = STAT_WARPS;
     auto grid_of = [&](int rows, int zc) {
         return dim3(stats ? chunks : (chunks + nw - 1) / nw, rows, (a.nz + zc - 1) / zc);
