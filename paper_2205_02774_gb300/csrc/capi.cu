@@ -4,7 +4,6 @@
 #include <algorithm>
 #include <chrono>
 #include <cmath>
-#include <cstddef>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -480,19 +479,20 @@ namespace {
 namespace stg {
 namespace host {
 
+// samples of the probes after t steps, into out or the call's series
+cudaError_t enqueue_probes(stg_lbm *h, int64_t t, float *out, cudaStream_t s)
+{
+    stg::LatticeView v = lattice_view(h);
+    v.t = t;
+    return stg::launch_probe(h->lat[t & 1], h->d.storage, v, h->n_probes, h->probe_xyz, (float)h->d.force[0],
+                             (float)h->d.force[1], (float)h->d.force[2], h->ctl, out, s);
+}
+
 // The inlet planes are computed beside the passes on a branch of their own, a few
 // for the next steps first (they are due when the first pass ends) and the rest of
 // the block, INLET_MAX_PLANES at a time, beside the passes that read those.  One
 // launch per step instead took 10 to 19 us each on lattices whose pass takes 4 to
 // 60, ahead of the pass or of its wall rows.
-cudaError_t enqueue_probes(stg_lbm *h, int64_t t, cudaStream_t s)
-{
-    stg::LatticeView v = lattice_view(h);
-    v.t = t;
-    return stg::launch_probe(h->lat[t & 1], h->d.storage, v, h->n_probes, h->probe_xyz, (float)h->d.force[0],
-                             (float)h->d.force[1], (float)h->d.force[2], h->ctl, s);
-}
-
 cudaError_t enqueue_steps(stg_lbm *h, int64_t t, int n, bool probed)
 {
     constexpr int FIRST = 4;
@@ -526,12 +526,12 @@ cudaError_t enqueue_steps(stg_lbm *h, int64_t t, int n, bool probed)
                                  h->stream, h->side, h->ev_fork, h->ev_join);
         if (!probed || e != cudaSuccess) continue;
         if (h->aa) {
-            e = enqueue_probes(h, t + s + 1, h->stream);
+            e = enqueue_probes(h, t + s + 1, nullptr, h->stream);
             continue;
         }
         e = cudaEventRecord(h->ev_pfork, h->stream);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(h->side, h->ev_pfork, 0);
-        if (e == cudaSuccess) e = enqueue_probes(h, t + s + 1, h->side);
+        if (e == cudaSuccess) e = enqueue_probes(h, t + s + 1, nullptr, h->side);
         if (e == cudaSuccess) e = cudaEventRecord(h->ev_pjoin[s & 1], h->side);
     }
     for (int s = std::max(0, n - 2); s < n && probed && !h->aa && e == cudaSuccess; ++s)
@@ -1412,18 +1412,14 @@ int stg_lbm_step_probed(stg_lbm *h, int64_t n, float *u_host)
         }
         h->probe_cap = need;
     }
-    // where the call's samples go (the words are free again: the call waits for its work)
-    struct {
-        long long t;
-        float *out;
-    } series{h->t, h->probe_buf};
-    static_assert(sizeof series == 2 * sizeof(double) && offsetof(StepCtl, probe_out) == offsetof(StepCtl, t_probe) + 8, "layout");
-    std::memcpy(h->h_pinned + 2, &series, sizeof series);
-    CK(cudaMemcpyAsync(&h->ctl->t_probe, h->h_pinned + 2, sizeof series, cudaMemcpyHostToDevice, h->stream));
+    const int64_t t0 = h->t;
     const int per = h->d.stats_every;
+    bool series = false;  // whether the device knows where the call's samples go
     for (int64_t s = 0; s < n;) {
         cudaGraphExec_t g = h->g_probed[h->t & 1];
         if (g && n - s >= h->block_steps && (per <= 0 || h->t % per == 0)) {
+            if (!series) CK(stg::launch_probe_series(h->ctl, t0, h->probe_buf, h->stream));
+            series = true;
             CK(cudaGraphLaunch(g, h->stream));
             h->t += h->block_steps;
             s += h->block_steps;
@@ -1431,8 +1427,8 @@ int stg_lbm_step_probed(stg_lbm *h, int64_t n, float *u_host)
         }
         CK(cudaGraphLaunch(h->g_single[h->t & 1][is_stats_step(h, h->t) ? 1 : 0], h->stream));
         h->t += 1;
+        CK(enqueue_probes(h, h->t, h->probe_buf + (size_t)s * h->n_probes * 3, h->stream));
         s += 1;
-        CK(enqueue_probes(h, h->t, h->stream));
     }
     rc = queue_check_readback(h);
     if (rc) return rc;

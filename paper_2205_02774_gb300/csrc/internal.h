@@ -15,7 +15,7 @@ struct StepCtl {
     long long t[2];
     long long t0_filter;  // step at which the temporal filter restarts
     long long t_block;    // step at which the current block of steps began
-    long long t_probe;    // probed steps: step index before the first one of the call
+    long long t_probe;    // probed blocks: step index before the first one of the call
     float *probe_out;     // and its samples [steps][3 n]
     unsigned long long err; // error bits set by kernels (none of the current kernels sets one)
 };
@@ -133,9 +133,11 @@ struct LatticeView {
     long long t;
 };
 // velocity of n cells (xyz: device int triples) of the lattice stored after lv.t
-// steps, into the place of that step in ctl->probe_out
+// steps, into out or (NULL) the place of that step in the series of ctl, which
+// launch_probe_series sets for the steps from t on
 cudaError_t launch_probe(const void *src, int storage, const LatticeView &lv, int n, const int *xyz, float Fx,
-                         float Fy, float Fz, const StepCtl *ctl, cudaStream_t s);
+                         float Fy, float Fz, const StepCtl *ctl, float *out, cudaStream_t s);
+cudaError_t launch_probe_series(StepCtl *ctl, long long t, float *out, cudaStream_t s);
 // canonical sub-block [19][bz][by][bx] of a stored lattice into device memory `out`
 cudaError_t launch_gather_block(const void *src, int storage, const LatticeView &lv, int x0, int y0, int z0, int bx,
                                 int by, int bz, void *out, cudaStream_t s);

@@ -25,15 +25,16 @@ __device__ __forceinline__ size_t pop_index(const LatticeView &v, int i, int x, 
     return aa_slot(i, x, y, z, v.t, v.nx, v.ny, v.nz, v.bc_x, v.bc_y);
 }
 
-// The samples of step t (ctl->t after it) go to place t - 1 - ctl->t_probe of the
-// series ctl->probe_out: the graphs of probed steps are replayed for any call.
+// The samples go to `out`, or, where that is NULL, those of step t (ctl->t after it) to
+// place t - 1 - ctl->t_probe of the series ctl->probe_out: the graphs of probed steps
+// are replayed for any call.
 template <typename S>
 __global__ void probe_kernel(const S *src, LatticeView lv, int n, const int *xyz, float Fx, float Fy, float Fz,
-                             const StepCtl *ctl)
+                             const StepCtl *ctl, float *out)
 {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
-    float *out = ctl->probe_out + (size_t)(ctl->t[lv.t & 1] - 1 - ctl->t_probe) * 3 * n;
+    if (!out) out = ctl->probe_out + (size_t)(ctl->t[lv.t & 1] - 1 - ctl->t_probe) * 3 * n;
     const int x = xyz[3 * k + 0], y = xyz[3 * k + 1], z = xyz[3 * k + 2];
     float r = 0.f, jx = 0.f, jy = 0.f, jz = 0.f;
 #pragma unroll
@@ -50,15 +51,29 @@ __global__ void probe_kernel(const S *src, LatticeView lv, int n, const int *xyz
     out[3 * k + 2] = (jz - 0.5f * Fz) * ir;
 }
 
+// The place of a call's series as kernel parameters, which are the launch's own: from
+// pinned host words the copy could read what a later call has written there.
+__global__ void probe_series_kernel(StepCtl *ctl, long long t, float *out)
+{
+    ctl->t_probe = t;
+    ctl->probe_out = out;
+}
+
+cudaError_t launch_probe_series(StepCtl *ctl, long long t, float *out, cudaStream_t s)
+{
+    probe_series_kernel<<<1, 1, 0, s>>>(ctl, t, out);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_probe(const void *src, int storage, const LatticeView &lv, int n, const int *xyz, float Fx,
-                         float Fy, float Fz, const StepCtl *ctl, cudaStream_t s)
+                         float Fy, float Fz, const StepCtl *ctl, float *out, cudaStream_t s)
 {
     if (n <= 0) return cudaSuccess;
     const int T = 128, B = (n + T - 1) / T;
     if (storage == 0)
-        probe_kernel<float><<<B, T, 0, s>>>(static_cast<const float *>(src), lv, n, xyz, Fx, Fy, Fz, ctl);
+        probe_kernel<float><<<B, T, 0, s>>>(static_cast<const float *>(src), lv, n, xyz, Fx, Fy, Fz, ctl, out);
     else
-        probe_kernel<__half><<<B, T, 0, s>>>(static_cast<const __half *>(src), lv, n, xyz, Fx, Fy, Fz, ctl);
+        probe_kernel<__half><<<B, T, 0, s>>>(static_cast<const __half *>(src), lv, n, xyz, Fx, Fy, Fz, ctl, out);
     return cudaGetLastError();
 }
 
