@@ -64,6 +64,7 @@ struct stg_lbm {
     cudaGraphExec_t g_single[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
     cudaGraphExec_t g_block[2] = {nullptr, nullptr};
     cudaGraphExec_t g_probed[2] = {nullptr, nullptr};  // blocks with the probes sampled after every step
+    int64_t probed_steps = 0;                          // steps asked for with the present probes and tile
     int block_steps = 16;
     stg_info info{};
     double timeout_s = 900.0;
