@@ -335,8 +335,9 @@ int stg_lbm_estimate_bytes(const stg_domain *domain, const stg_params *stg, int6
  * fill the GPU together and no member waits for another between steps.  B is
  * the smallest multiple of 2 and of every member's sampling period that is at
  * least 16 (members whose periods have no common multiple <= 256 are
- * refused).  A member runs exactly the kernels and arguments it runs alone:
- * its populations and statistics are bit-identical to a solo run.  Members
+ * refused).  A member's launches may be cut otherwise than alone (by the cells
+ * that share the GPU), with the same operations per cell: its populations and
+ * statistics are bit-identical to a solo run.  Members
  * keep their own state, statistics and mass checks; stg_lbm_stats,
  * get_state, get_inlet, device_state and info work on a member as usual and
  * are ordered after the batch's work; stg_lbm_step, step_timed, set_state,

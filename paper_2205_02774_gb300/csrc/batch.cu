@@ -4,8 +4,9 @@
 // steps (inlet kernel, then the step pass with its forked boundary branch) as
 // its own branch between one fork and one join, so the members' kernels
 // overlap on the GPU and no member waits for another between steps; a block is
-// one graph launch.  A member runs exactly the kernels and arguments it runs
-// alone, so its populations and statistics are bit-identical to a solo run.
+// one graph launch.  A member's cells go through the same operations as alone, so
+// its populations and statistics are bit-identical to a solo run; how its passes
+// are cut (lanes, launches, runs) follows the cells of all members together.
 // While members come and go, each member's own graph of B steps is launched
 // on its branch instead (no capture of the whole batch per change); the
 // combined graph is captured once the membership has been stable for a few
