@@ -113,7 +113,11 @@ def _launches_enqueued(c, t0, steps, batch=False):
         period = k * (1 if k % 2 == 0 else 2) * -(-16 // (k * (1 if k % 2 == 0 else 2)))
     row = c.streaming == "pull" and (c.nx % 2 != 0 or c.nx < 4)
     small = c.streaming == "pull" and c.storage == "fp32" and c.cells < 4 * 152 * 32 * 32 and not batch
-    cpl = (4 if row or (c.nx % 4 == 0 and c.nx >= 8) else 2) if c.storage != "fp32" else (1 if small else 2)
+    bgk_pairs = c.collision == "bgk" and not row and (
+        c.streaming == "aa" or (c.nx <= (720 if c.storage == "fp16sr" else 580) if c.bc_x == "stg" else
+                                c.storage != "fp16sr" or 2 * -(-c.nx // 128) != -(-c.nx // 64)))
+    quads = row or (c.nx % 4 == 0 and c.nx >= 8 and not bgk_pairs)
+    cpl = (4 if quads else 2) if c.storage != "fp32" else (1 if small else 2)
     items = -(-c.nx // (32 * cpl)) * c.ny * c.nz
     passes = 1 if c.ny < 3 or (not batch and 2 * items < 152 * 16 * (3 if cpl == 4 else 8)) else 2
     inlet = c.bc_x == "stg"

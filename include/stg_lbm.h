@@ -267,7 +267,7 @@ int stg_lbm_info(const stg_lbm *h, stg_info *out);
  * differ in its last bits, its block partials being summed in another order).
  *   interior_layout  1: a warp walks a whole z chunk; 0: 8 warps share it.  A warp's row
  *                    piece is 32 cells (FP32 lattices of fewer than 622592 cells), 64, or
- *                    128 (binary16, nx a multiple of 4)
+ *                    128 (binary16 with nx a multiple of 4; some BGK lattices keep 64)
  *   interior_zc      z planes per chunk of the rows 1..ny-2, or of all rows on lattices
  *                    small enough for one launch (0: the whole z column, else >= 4)
  *   wall_zc          z planes per chunk of the wall rows y = 0, ny-1, which 8 warps

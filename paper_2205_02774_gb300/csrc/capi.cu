@@ -409,6 +409,8 @@ stg::StepArgs step_args(const stg_lbm *h, int parity)
     a.in_flight = std::max<int64_t>(h->in_flight, (int64_t)h->P);
     a.bc_x = h->d.bc_x;
     a.bc_y = h->d.bc_y;
+    a.storage = h->d.storage;
+    a.collision = h->d.collision;
     a.tau0 = (float)h->d.tau0;
     a.kq = (float)(18.0 * std::sqrt(2.0) * h->d.c_smag);
     a.Fx = (float)h->d.force[0];
@@ -522,8 +524,8 @@ cudaError_t enqueue_steps(stg_lbm *h, int64_t t, int n, bool probed)
         // reads the same lattice, and before the one after, which writes it
         if (e == cudaSuccess && probed && s >= 2 && !h->aa) e = cudaStreamWaitEvent(h->stream, h->ev_pjoin[s & 1], 0);
         if (e == cudaSuccess)
-            e = stg::launch_step(step_args(h, (int)((t + s) & 1)), h->d.storage, h->d.collision, is_stats_step(h, t + s),
-                                 h->stream, h->side, h->ev_fork, h->ev_join);
+            e = stg::launch_step(step_args(h, (int)((t + s) & 1)), is_stats_step(h, t + s), h->stream, h->side,
+                                 h->ev_fork, h->ev_join);
         if (!probed || e != cudaSuccess) continue;
         if (h->aa) {
             e = enqueue_probes(h, t + s + 1, nullptr, h->stream);
@@ -1080,8 +1082,7 @@ int stg_lbm_step_timed(stg_lbm *h, int64_t n, double *ms_step, double *ms_inlet)
         if (e == cudaSuccess && h->inout) e = stg::launch_inlet(inlet_args(h, parity), h->stream);
         if (e == cudaSuccess) e = cudaEventRecord(ev[3 * s + 1], h->stream);
         if (e == cudaSuccess)
-            e = stg::launch_step(step_args(h, parity), h->d.storage, h->d.collision, is_stats_step(h, h->t),
-                                 h->stream, h->side, h->ev_fork, h->ev_join);
+            e = stg::launch_step(step_args(h, parity), is_stats_step(h, h->t), h->stream, h->side, h->ev_fork, h->ev_join);
         if (e == cudaSuccess) e = cudaEventRecord(ev[3 * s + 2], h->stream);
         if (e != cudaSuccess) rc = cuda_fail(h, e, "timed step launch");
         else h->t += 1;
@@ -1465,7 +1466,7 @@ cudaError_t trial_pass(stg_lbm *h, const stg_tile &tile, cudaStream_t s, int k)
     stg::StepArgs a = step_args(h, parity);
     h->tile = keep;
     a.stats_every = 0;  // the edge kernel samples on its own otherwise
-    return stg::launch_step(a, h->d.storage, h->d.collision, false, s, h->side, h->ev_fork, h->ev_join);
+    return stg::launch_step(a, false, s, h->side, h->ev_fork, h->ev_join);
 }
 
 int save_trial_state(stg_lbm *h, std::vector<unsigned char> &pops, stg::StepCtl &ctl)
@@ -1520,7 +1521,7 @@ int tile_inner_run(stg_lbm *h, const stg_tile &tile)
     h->tile = tile;
     const stg::StepArgs a = step_args(h, 0);
     h->tile = keep;
-    return stg::run_planes(a, stg::lane_cells(a, h->d.storage), (int)h->elem, false);
+    return stg::run_planes(a, stg::lane_cells(a), (int)h->elem, false);
 }
 
 bool better_tile(int c, float ms, float best_ms, float own_ms)

@@ -51,6 +51,7 @@ struct StepArgs {
     unsigned P;           // cells per population plane (nx*ny*nz)
     long long in_flight;  // cells of all lattices advanced together (a batch's members; else P)
     int bc_x, bc_y;       // STG_BC_X_*, STG_BC_Y_*
+    int storage, collision;  // stg_domain's
     float tau0, kq;       // kq = 18 sqrt(2) C  (eq. tau_eff)
     float Fx, Fy, Fz;
     int has_force;
@@ -98,13 +99,12 @@ struct MassArgs {
 // launchers (return the launch status)
 // `stats` must be true exactly on sampling steps ((t + 1) % stats_every == 0);
 // the host tracks t and decides.
-cudaError_t launch_step(const StepArgs &a, int storage, int collision, bool stats,
-                        cudaStream_t s, cudaStream_t side, cudaEvent_t fork, cudaEvent_t join);
-// binary16 lattices take quads (four cells per lane)
-// when the rows split into whole quads
+cudaError_t launch_step(const StepArgs &a, bool stats, cudaStream_t s, cudaStream_t side, cudaEvent_t fork,
+                        cudaEvent_t join);
+// whether the rows split into whole quads (four cells per lane, binary16)
 inline bool quads_fit(int nx) { return nx % 4 == 0 && nx >= 8; }
-// Lattices of the vector kernels (the others take one cell per thread): rows of
-// whole pairs and 32-bit element offsets.  The in-place scheme exists for them
+// Lattices of aligned vectors (the others take lanes 32 cells apart, or one cell per
+// thread): rows of whole pairs and 32-bit element offsets.  The in-place scheme exists for them
 // only (the host checks its conditions), so it ignores the interior override.
 inline bool vector_fits(const StepArgs &a)
 {
@@ -116,8 +116,8 @@ inline bool vector_fits(const StepArgs &a)
 bool one_launch(const StepArgs &a, int cpl);
 int run_planes(const StepArgs &a, int cpl, int elem, bool walls);
 // cells per lane of the vector kernels, and whether they lie 32 apart
-int lane_cells(const StepArgs &a, int storage);
-bool row_lanes(const StepArgs &a, int storage);
+int lane_cells(const StepArgs &a);
+bool row_lanes(const StepArgs &a);
 cudaError_t launch_inlet(const InletArgs &a, cudaStream_t s);
 // FP64 Cholesky factor of the lattice-unit Reynolds stress per inlet node (setup)
 cudaError_t launch_setup_nodes(int ny, const double *R6, float *a6, cudaStream_t s);

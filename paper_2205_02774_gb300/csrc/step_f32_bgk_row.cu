@@ -7,7 +7,7 @@ namespace stg {
 
 bool launch_f32_bgk_row(const StepArgs &a, bool stats, cudaStream_t s, cudaStream_t side)
 {
-    if (lane_cells(a, 0) == 1) return launch_row<float, 1, false>(a, stats, s, side);
+    if (lane_cells(a) == 1) return launch_row<float, 1, false>(a, stats, s, side);
     return launch_row<float, 2, false>(a, stats, s, side);
 }
 

@@ -64,16 +64,35 @@ static bool small_row(const StepArgs &a)
     return std::max<long long>(a.P, a.in_flight) < 4LL * 152 * 32 * 32;
 }
 
-bool row_lanes(const StepArgs &a, int storage)
+bool row_lanes(const StepArgs &a)
 {
     if (a.aa || a.interior != 0 || 19.0 * a.P >= 4294967296.0) return false;
-    return a.nx % 2 != 0 || a.nx < 4 || (storage == 0 && small_row(a));
+    return a.nx % 2 != 0 || a.nx < 4 || (a.storage == 0 && small_row(a));
 }
 
-int lane_cells(const StepArgs &a, int storage)
+// Binary16 BGK lattices whose rows split into quads take pairs all the same where the
+// quads' wider chunks (128 cells, 16 warps per SM) lose more than their accesses gain:
+// at an inlet and an outlet, where the chunks with a node go cell by cell, up to the
+// length where the others outweigh them (round to nearest 580 cells, stochastic
+// rounding 720: us per step with quads and pairs, 160^3 91.0 and 73.9, 200^3 147 and
+// 136, 520x128x128 135.5 and 129.1, 640x128x128 144.5 and 148.4; stochastic rounding
+// 160^3 95.6 and 79.2, 700x128x128 183 and 173, 768x128x192 260 and 267); in a periodic
+// box with round to nearest (160^3 85.7 and 68.5, 768x128x128 184.6 and 181.8) and, with
+// stochastic rounding, where pairs also fill their chunks better (320x160x160 142.5 and
+// 133.3, 768x128x128 191 and 207); in place (768x160x160 SR 329 and 318).
+static bool bgk_pairs(const StepArgs &a)
 {
-    if (row_lanes(a, storage)) return storage != 0 ? 4 : (small_row(a) ? 1 : 2);
-    return storage != 0 && quads_fit(a.nx) && vector_fits(a) ? 4 : 2;
+    const bool sr = a.storage == 2;
+    if (a.aa) return true;
+    if (a.bc_x != 0) return !sr || 2 * ((a.nx + 127) / 128) != (a.nx + 63) / 64;
+    return a.nx <= (sr ? 720 : 580);
+}
+
+int lane_cells(const StepArgs &a)
+{
+    if (row_lanes(a)) return a.storage != 0 ? 4 : (small_row(a) ? 1 : 2);
+    const bool quads = a.storage != 0 && quads_fit(a.nx) && vector_fits(a) && !(a.collision != 0 && bgk_pairs(a));
+    return quads ? 4 : 2;
 }
 
 // Items: one x chunk (32 cpl cells) of one row and plane each, of all lattices
@@ -145,12 +164,12 @@ __global__ void stats_reduce_kernel(const float *part, int groups, size_t m, dou
 // One fused step pass.  The wall rows (or the edge kernel of the one-cell-per-
 // thread path) run on the forked branch `side` beside the inner rows (they write
 // disjoint slots); `s` waits for both.  A pass of one launch needs no branch.
-cudaError_t launch_step(const StepArgs &a, int storage, int collision, bool stats,
-                        cudaStream_t s, cudaStream_t side, cudaEvent_t fork, cudaEvent_t join)
+cudaError_t launch_step(const StepArgs &a, bool stats, cudaStream_t s, cudaStream_t side, cudaEvent_t fork,
+                        cudaEvent_t join)
 {
     cudaError_t e = cudaSuccess;
-    const int cpl = lane_cells(a, storage);
-    const bool one = (vector_fits(a) || row_lanes(a, storage)) && one_launch(a, cpl);
+    const int cpl = lane_cells(a);
+    const bool one = (vector_fits(a) || row_lanes(a)) && one_launch(a, cpl);
     const bool forked = !one && side != nullptr && fork != nullptr && join != nullptr;
     if (forked) {
         if ((e = cudaEventRecord(fork, s)) != cudaSuccess) return e;
@@ -163,7 +182,7 @@ cudaError_t launch_step(const StepArgs &a, int storage, int collision, bool stat
         {{launch_f16_reg, launch_f16_reg_quad, launch_f16_reg_row}, {launch_f16_bgk, launch_f16_bgk_quad, launch_f16_bgk_row}},
         {{launch_f16sr_reg, launch_f16sr_reg_quad, launch_f16sr_reg_row},
          {launch_f16sr_bgk, launch_f16sr_bgk_quad, launch_f16sr_bgk_row}}};
-    const bool reduce = passes[storage][collision][row_lanes(a, storage) ? 2 : (cpl == 4 ? 1 : 0)](a, stats, s, es);
+    const bool reduce = passes[a.storage][a.collision][row_lanes(a) ? 2 : (cpl == 4 ? 1 : 0)](a, stats, s, es);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (forked) {
         if ((e = cudaEventRecord(join, side)) != cudaSuccess) return e;
