@@ -1521,7 +1521,7 @@ int tile_inner_run(stg_lbm *h, const stg_tile &tile)
     h->tile = tile;
     const stg::StepArgs a = step_args(h, 0);
     h->tile = keep;
-    return stg::run_planes(a, stg::lane_cells(a), (int)h->elem, false);
+    return stg::run_planes(a, stg::lane_cells(a), false);
 }
 
 bool better_tile(int c, float ms, float best_ms, float own_ms)

@@ -114,7 +114,9 @@ inline bool vector_fits(const StepArgs &a)
 // Whether a pass of the vector kernels (cpl cells per lane) is one launch of all
 // rows, and the z planes per run of its launches (step_kernel.cu).
 bool one_launch(const StepArgs &a, int cpl);
-int run_planes(const StepArgs &a, int cpl, int elem, bool walls);
+int run_planes(const StepArgs &a, int cpl, bool walls);
+// warps of a block of such a launch, `most` of them at most
+int block_chunks(const StepArgs &a, int cpl, int chunks, int most);
 // cells per lane of the vector kernels, and whether they lie 32 apart
 int lane_cells(const StepArgs &a);
 bool row_lanes(const StepArgs &a);

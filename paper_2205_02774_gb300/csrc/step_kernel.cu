@@ -55,6 +55,9 @@ int stat_group(int nx, int ny, int nz)
     return std::max(g, (nz + 65534) / 65535);  // a launch holds 65535 runs
 }
 
+// the regularized collision without a force, whose kernels have the most warps per SM
+static bool lean(const StepArgs &a) { return a.collision == 0 && !a.has_force; }
+
 // FP32 lattices with fewer than 4 cells per resident lane (32 warps per SM): one
 // cell per lane halves the serial work of a warp (64x32x32 5.3 against 6.2 us per
 // step, 144x24x36 7.0 against 8.1, 240x40x60 15.4 against 18.2, 241x41x61 16.9
@@ -116,24 +119,44 @@ bool one_launch(const StepArgs &a, int cpl)
 
 // A run of several planes costs one block start instead of several, but a pass
 // ends with its last runs, and a short pass needs every warp from the start: so
-// runs grow with the number of items per resident warp.  FP32 (256 B per row piece)
-// is fastest with runs of 1 or 2 (768x128x192: 415, 418, 425 us with 2, 4, 8;
-// 1536x256x384: 3.27, 3.29, 3.31, 3.34 ms with 1, 2, 4, 8), binary16 with 4 or 8
-// (1536x256x384: 1.82, 1.76, 1.72, 1.72 ms with 1, 2, 4, 8; 384x64x96: 2).
+// runs grow with the number of items per resident warp, up to what the form takes:
+//  FP32 (256 B per row piece) 2 (768x128x192: 415, 418, 425 us with 2, 4, 8;
+//    1536x256x384: 3.27, 3.29, 3.31, 3.34 ms with 1, 2, 4, 8);
+//  binary16 quads 8 (1536x256x384: 1.82, 1.76, 1.72, 1.72 ms with 1, 2, 4, 8;
+//    384x64x96: 2);
+//  binary16 pairs (128 B) 2, with BGK or a force 4 (250x125x125 61.8, 64.9, 69.1 us with
+//    2, 4, 8, 770x128x192 282, 293, 305; BGK 200^3 142, 136, 142);
+//  binary16 lanes 32 cells apart 2 (767x127x191: 302, 308, 321 us with 2, 4, 8, 63x300x300
+//    174, 179, 184).
 // The wall rows, beside the inner launch, are spread over as many warps as their
 // latency needs: binary16 1, FP32 4 (768x128x192: FP16 226, 228, 230 us with
 // 1, 2, 4, and 236 with 24; FP32 420, 420, 418), and 4 among the members of a batch.
 // A tile that was set sets the runs instead.
-int run_planes(const StepArgs &a, int cpl, int elem, bool walls)
+int run_planes(const StepArgs &a, int cpl, bool walls)
 {
     const int least = (a.nz + 65534) / 65535;  // a launch holds 65535 runs
     const int tile = walls ? a.tile_wall_zc : a.tile_zc;
     if (tile > 0) return std::max(least, std::min(tile, a.nz));
-    if (walls) return std::max(least, std::min(a.nz, elem == 4 || a.in_flight > a.P ? 4 : 1));
-    const long long per_warp = items_of(a, cpl) / (152 * (elem == 4 ? 32 : 20));
+    const bool fp32 = a.storage == 0;
+    if (walls) return std::max(least, std::min(a.nz, fp32 || a.in_flight > a.P ? 4 : 1));
+    int most = 2;
+    if (!fp32 && !row_lanes(a)) most = cpl == 4 ? 8 : (lean(a) ? 2 : 4);
+    const long long per_warp = items_of(a, cpl) / (152 * (fp32 ? 32 : 20));
     int zc = 1;
-    while (zc < (elem == 4 ? 2 : 8) && per_warp >= 5 * zc) zc *= 2;
+    while (zc < most && per_warp >= 5 * zc) zc *= 2;
     return std::max(least, std::min(zc, a.nz));
+}
+
+// Warps (x chunks) of a block: as many as leave the fewest idle; one where a block of
+// several waits for the slowest of chunks that differ: stochastic rounding in pairs
+// (210^3 155.8 us per step with one, 157.3 with four, 250x125x125 66.3 and 67.1).
+int block_chunks(const StepArgs &a, int cpl, int chunks, int most)
+{
+    if (a.storage == 2 && cpl == 2) return 1;
+    int nw = most;
+    for (int k = nw - 1; k > 0; --k)
+        if ((chunks + k - 1) / k * k < (chunks + nw - 1) / nw * nw) nw = k;
+    return nw;
 }
 
 // Adds the z-group sums of a sampling step to the FP64 statistics, group by

@@ -978,14 +978,11 @@ template <typename S, int CPL, bool REG, bool FORCE, bool SP, int MODE, bool SR>
 static void launch_vec(StepArgs a, bool stats, cudaStream_t s, cudaStream_t side)
 {
     const int chunks = (a.nx + BX * CPL - 1) / (BX * CPL);  // (a row's shift adds none)
-    int nw = block_warps<CPL, false>();
-    // chunks per block: as many as leave the fewest warps idle
-    for (int k = nw - 1; k > 0; --k)
-        if ((chunks + k - 1) / k * k < (chunks + nw - 1) / nw * nw) nw = k;
+    int nw = block_chunks(a, CPL, chunks, block_warps<CPL, false>());
     const bool one = one_launch(a, CPL);
     StepArgs w = a;
-    a.tile_zc = stats ? a.stat_group : run_planes(a, CPL, sizeof(S), false);
-    w.tile_zc = stats ? a.stat_group : run_planes(w, CPL, sizeof(S), true);
+    a.tile_zc = stats ? a.stat_group : run_planes(a, CPL, false);
+    w.tile_zc = stats ? a.stat_group : run_planes(w, CPL, true);
     if (stats) nw = STAT_WARPS;
     auto grid_of = [&](int rows, int zc) {
         return dim3(stats ? chunks : (chunks + nw - 1) / nw, rows, (a.nz + zc - 1) / zc);
