@@ -111,7 +111,8 @@ def _launches_enqueued(c, t0, steps, batch=False):
     period = k * -(-16 // k) if c.stats_every > 0 else 16
     if batch:
         period = k * (1 if k % 2 == 0 else 2) * -(-16 // (k * (1 if k % 2 == 0 else 2)))
-    row = c.streaming == "pull" and (c.nx % 2 != 0 or c.nx < 4)
+    narrow = c.storage != "fp32" and c.nx < 32 and c.ny * c.nz >= 152 * 20 * (19 if c.storage == "fp16sr" else 24)
+    row = c.streaming == "pull" and (c.nx % 2 != 0 or c.nx < 4) and not narrow
     small = c.streaming == "pull" and c.storage == "fp32" and c.cells < 4 * 152 * 32 * 32 and not batch
     bgk_pairs = c.collision == "bgk" and not row and (
         c.streaming == "aa" or (c.nx <= (720 if c.storage == "fp16sr" else 580) if c.bc_x == "stg" else
@@ -119,7 +120,8 @@ def _launches_enqueued(c, t0, steps, batch=False):
     quads = row or (c.nx % 4 == 0 and c.nx >= 8 and not bgk_pairs)
     cpl = (4 if quads else 2) if c.storage != "fp32" else (1 if small else 2)
     items = -(-c.nx // (32 * cpl)) * c.ny * c.nz
-    passes = 1 if c.ny < 3 or (not batch and 2 * items < 152 * 16 * (3 if cpl == 4 else 8)) else 2
+    scalar = c.streaming == "pull" and (c.nx % 2 != 0 or c.nx < 4) and not row  # a pass of its own kernels, no reduction
+    passes = 1 if not scalar and (c.ny < 3 or (not batch and 2 * items < 152 * 16 * (3 if cpl == 4 else 8))) else 2
     inlet = c.bc_x == "stg"
     n, t, left = 0, t0, steps
     while left > 0:
@@ -128,7 +130,7 @@ def _launches_enqueued(c, t0, steps, batch=False):
         n += b * passes + (inlet and 1 + max(0, -(-(b - 4) // 16)))
         t += b
         left -= b
-    if c.stats_every > 0:
+    if c.stats_every > 0 and not scalar:
         n += (t0 + steps) // c.stats_every - t0 // c.stats_every
     return n
 

@@ -67,9 +67,19 @@ static bool small_row(const StepArgs &a)
     return std::max<long long>(a.P, a.in_flight) < 4LL * 152 * 32 * 32;
 }
 
+// Rows of fewer than 32 cells in binary16: a lane's other three cells lie outside the
+// row, and once such rows fill the GPU one cell per thread is the faster form (from 24
+// rows x planes per resident warp on, with stochastic rounding 19: 5x300x300 132 against
+// 145 us per step, 141 against 171; 31x260x260 126 against 114, 133 against 139).
+static bool narrow_rows(const StepArgs &a)
+{
+    return a.storage != 0 && a.nx < 32 && (long long)a.ny * a.nz >= 152LL * 20 * (a.storage == 2 ? 19 : 24);
+}
+
 bool row_lanes(const StepArgs &a)
 {
     if (a.aa || a.interior != 0 || 19.0 * a.P >= 4294967296.0) return false;
+    if (narrow_rows(a)) return false;
     return a.nx % 2 != 0 || a.nx < 4 || (a.storage == 0 && small_row(a));
 }
 

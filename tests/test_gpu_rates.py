@@ -52,3 +52,11 @@ def test_bgk_of_binary16_on_ragged_rows(n):
 def test_runs_of_binary16_pairs(dims):
     kw = dict(nx=dims[0], ny=dims[1], nz=dims[2], storage="fp16s")
     assert _us(**kw) < 0.97 * _us(tile=(1, 9, 24), **kw)
+
+
+# four cells per lane of which one is in the row: 1.30 times the time of one cell per thread
+def test_narrow_rows_of_binary16(monkeypatch):
+    kw = dict(nx=5, ny=300, nz=300, storage="fp16sr")
+    own = _us(**kw)
+    monkeypatch.setenv("STG_LBM_INTERIOR", "scalar")
+    assert own < 1.1 * _us(**kw)

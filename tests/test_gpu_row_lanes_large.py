@@ -57,3 +57,11 @@ def test_step_and_statistics(dims, storage, kw):
     assert normwise(s["mean_sum"], m) < tol and normwise(s["rey_sum"], r) < tol
     assert abs(s["mass"] - orc.pops().sum()) <= (1e-6 if storage == "fp32" else 1e-4) * nx * ny * nz
     gpu.close()
+
+
+# rows of fewer than 32 cells change to one cell per thread at 57 760 (stochastic rounding) and
+# 72 960 rows x planes
+@pytest.mark.parametrize("dims", [(31, 190, 303), (31, 190, 305), (3, 190, 305), (5, 240, 303), (5, 240, 305)])
+@pytest.mark.parametrize("storage", ["fp16s", "fp16sr"])
+def test_narrow_rows(dims, storage):
+    test_step_and_statistics(dims, storage, dict(collision="bgk"))
