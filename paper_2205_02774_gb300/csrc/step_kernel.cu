@@ -57,6 +57,12 @@ int stat_group(int nx, int ny, int nz)
 
 // the regularized collision without a force, whose kernels have the most warps per SM
 static bool lean(const StepArgs &a) { return a.collision == 0 && !a.has_force; }
+// FP32 pairs, BGK or a force (24 warps per SM), the last chunk of a row up to three
+// quarters full
+static bool ragged_fp32(const StepArgs &a)
+{
+    return a.storage == 0 && !lean(a) && !row_lanes(a) && a.nx % 64 != 0 && a.nx % 64 <= 48;
+}
 
 // FP32 lattices with fewer than 4 cells per resident lane (32 warps per SM): one
 // cell per lane halves the serial work of a warp (64x32x32 5.3 against 6.2 us per
@@ -131,7 +137,9 @@ bool one_launch(const StepArgs &a, int cpl)
 // ends with its last runs, and a short pass needs every warp from the start: so
 // runs grow with the number of items per resident warp, up to what the form takes:
 //  FP32 (256 B per row piece) 2 (768x128x192: 415, 418, 425 us with 2, 4, 8;
-//    1536x256x384: 3.27, 3.29, 3.31, 3.34 ms with 1, 2, 4, 8);
+//    1536x256x384: 3.27, 3.29, 3.31, 3.34 ms with 1, 2, 4, 8), with BGK or a force and
+//    a ragged last chunk 4 (200^3 228, 218, 216 us with 2, 4, 8; full rows stay at 2:
+//    320x160x160 193, 193, 197, 256x128x128 97.6, 98.4, 106.7);
 //  binary16 quads 8 (1536x256x384: 1.82, 1.76, 1.72, 1.72 ms with 1, 2, 4, 8;
 //    384x64x96: 2);
 //  binary16 pairs (128 B) 2, with BGK or a force 4 (250x125x125 61.8, 64.9, 69.1 us with
@@ -149,7 +157,7 @@ int run_planes(const StepArgs &a, int cpl, bool walls)
     if (tile > 0) return std::max(least, std::min(tile, a.nz));
     const bool fp32 = a.storage == 0;
     if (walls) return std::max(least, std::min(a.nz, fp32 || a.in_flight > a.P ? 4 : 1));
-    int most = 2;
+    int most = ragged_fp32(a) ? 4 : 2;
     if (!fp32 && !row_lanes(a)) most = cpl == 4 ? 8 : (lean(a) ? 2 : 4);
     const long long per_warp = items_of(a, cpl) / (152 * (fp32 ? 32 : 20));
     int zc = 1;
@@ -159,10 +167,11 @@ int run_planes(const StepArgs &a, int cpl, bool walls)
 
 // Warps (x chunks) of a block: as many as leave the fewest idle; one where a block of
 // several waits for the slowest of chunks that differ: stochastic rounding in pairs
-// (210^3 155.8 us per step with one, 157.3 with four, 250x125x125 66.3 and 67.1).
+// (210^3 155.8 us per step with one, 157.3 with four, 250x125x125 66.3 and 67.1), and
+// ragged FP32 rows (200^3 BGK 209.6 and 217.0, 210^3 249.6 and 256.3).
 int block_chunks(const StepArgs &a, int cpl, int chunks, int most)
 {
-    if (a.storage == 2 && cpl == 2) return 1;
+    if ((a.storage == 2 && cpl == 2) || ragged_fp32(a)) return 1;
     int nw = most;
     for (int k = nw - 1; k > 0; --k)
         if ((chunks + k - 1) / k * k < (chunks + nw - 1) / nw * nw) nw = k;

@@ -60,3 +60,11 @@ def test_narrow_rows_of_binary16(monkeypatch):
     own = _us(**kw)
     monkeypatch.setenv("STG_LBM_INTERIOR", "scalar")
     assert own < 1.1 * _us(**kw)
+
+
+# FP32 BGK, a last chunk of 8 of 64 cells: short runs in blocks of four warps that wait for
+# each other took 1.06 times as long as runs of 9, runs of 4 in blocks of one 0.98 (the tile
+# sets the run, not the block)
+def test_fp32_bgk_on_ragged_rows():
+    kw = dict(nx=200, ny=200, nz=200, collision="bgk")
+    assert _us(**kw) < 1.02 * _us(tile=(1, 9, 24), **kw)
