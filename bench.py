@@ -105,8 +105,8 @@ def _launches(c, t0, steps):
 def _launches_enqueued(c, t0, steps, batch=False):
     """Kernels the steps t0 .. t0+steps-1 really enqueue, as the library cuts them:
     blocks (from a step index divisible by the sampling period; in a batch from any)
-    carry one inlet launch for the first 4 steps and one per 16 more, single steps
-    one each; a pass is one launch on lattices that do not fill the GPU, else two."""
+    carry one inlet launch for the first 4 steps and one per 16 more (in a batch one
+    per 16), single steps one each; a pass is one launch on lattices that do not fill the GPU, else two."""
     k = max(c.stats_every, 1)
     period = k * -(-16 // k) if c.stats_every > 0 else 16
     if batch:
@@ -127,7 +127,7 @@ def _launches_enqueued(c, t0, steps, batch=False):
     while left > 0:
         whole = period <= 256 and left >= period and (batch or t % k == 0)
         b = period if whole else 1
-        n += b * passes + (inlet and 1 + max(0, -(-(b - 4) // 16)))
+        n += b * passes + (inlet and (-(-b // 16) if batch and whole else 1 + max(0, -(-(b - 4) // 16))))
         t += b
         left -= b
     if c.stats_every > 0 and not scalar:

@@ -494,19 +494,29 @@ cudaError_t enqueue_probes(stg_lbm *h, int64_t t, float *out, cudaStream_t s)
 // for the next steps first (they are due when the first pass ends) and the rest of
 // the block, INLET_MAX_PLANES at a time, beside the passes that read those.  One
 // launch per step instead took 10 to 19 us each on lattices whose pass takes 4 to
-// 60, ahead of the pass or of its wall rows.
+// 60, ahead of the pass or of its wall rows.  Among the members of a batch the
+// launches stand in line with the member's own passes, which the other members'
+// overlap: a branch per member is one of too many there (80 channels of 144x24x36 in
+// binary16 327 us per step with the branches, 250 in line; two of 768x128x192 in FP32
+// 823 and 822).
 cudaError_t enqueue_steps(stg_lbm *h, int64_t t, int n, bool probed)
 {
-    constexpr int FIRST = 4;
+    const bool branch = h->in_flight == 0;
+    const int first = branch ? 4 : stg::INLET_MAX_PLANES;
     cudaError_t e = cudaSuccess;
     int asked = 0;  // planes launched: those of the steps t + 1 .. t + asked
-    int due = 0;    // the first step whose plane has not been waited for
+    int due = 0;    // the first step whose plane has not been waited for (in line: launched)
     auto ask = [&](int k) {
         k = std::min(k, n - asked);
         stg::InletArgs in = inlet_args(h, (int)(t & 1));
         in.from_block = asked > 0;
         in.ahead = 1 + asked;
         in.planes = k;
+        if (!branch) {
+            asked += k;
+            e = stg::launch_inlet(in, h->stream);
+            return;
+        }
         e = cudaEventRecord(h->ev_ifork, h->stream);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(h->inlet_side, h->ev_ifork, 0);
         if (e == cudaSuccess) e = stg::launch_inlet(in, h->inlet_side);
@@ -515,10 +525,11 @@ cudaError_t enqueue_steps(stg_lbm *h, int64_t t, int n, bool probed)
     };
     for (int s = 0; s < n && e == cudaSuccess; ++s) {
         if (h->inout && s == due) {
-            if (s > 0) e = cudaStreamWaitEvent(h->stream, h->ev_ijoin, 0);
+            if (s > 0 && branch) e = cudaStreamWaitEvent(h->stream, h->ev_ijoin, 0);
             due = asked + 1;
             // the ring holds the planes that the coming passes read and as many again
-            if (e == cudaSuccess && asked < n) ask(s == 0 ? FIRST : stg::INLET_MAX_PLANES);
+            if (e == cudaSuccess && asked < n) ask(s == 0 ? first : stg::INLET_MAX_PLANES);
+            if (!branch) due = asked;
         }
         // two lattices: the samples of a step are taken beside the next one, which
         // reads the same lattice, and before the one after, which writes it
@@ -538,7 +549,7 @@ cudaError_t enqueue_steps(stg_lbm *h, int64_t t, int n, bool probed)
     }
     for (int s = std::max(0, n - 2); s < n && probed && !h->aa && e == cudaSuccess; ++s)
         e = cudaStreamWaitEvent(h->stream, h->ev_pjoin[s & 1], 0);
-    if (e == cudaSuccess && h->inout && n > 0) e = cudaStreamWaitEvent(h->stream, h->ev_ijoin, 0);
+    if (e == cudaSuccess && h->inout && n > 0 && branch) e = cudaStreamWaitEvent(h->stream, h->ev_ijoin, 0);
     return e;
 }
 
