@@ -82,10 +82,11 @@ def _traffic(workload, storage, streaming="pull"):
 
 
 def _launches_per_step(c):
-    """Kernels one step enqueues: the STG inlet kernel (inlet/outlet channel),
-    then either the vector kernel on rows 1..ny-2 and the vector kernel on the
-    two wall rows (even nx; inlet and outlet nodes included), or the scalar
-    interior and edge kernels (odd nx)."""
+    """Kernels of one step that is launched by itself, on a lattice large enough
+    for two launches per pass: the STG inlet kernel (inlet/outlet channel), then
+    the vector kernel on rows 1..ny-2 and on the two wall rows, or the interior
+    and edge kernels of one cell per thread.  (_launches_enqueued counts what a
+    call really enqueues.)"""
     inlet = 1 if c.bc_x == "stg" else 0
     if c.nx % 2 == 0 and c.nx >= 4:
         return inlet + (1 if c.ny > 2 else 0) + 1
@@ -93,9 +94,9 @@ def _launches_per_step(c):
 
 
 def _launches(c, t0, steps):
-    """Kernels the steps t0 .. t0+steps-1 enqueue: _launches_per_step each, plus
-    the statistics reduction after every sampling step ((t + 1) % stats_every
-    == 0) of the vector path."""
+    """Kernels of the steps t0 .. t0+steps-1 launched one by one: _launches_per_step
+    each, plus the statistics reduction after every sampling step ((t + 1) %
+    stats_every == 0) of aligned rows."""
     n = _launches_per_step(c) * steps
     if c.stats_every > 0 and c.nx % 2 == 0 and c.nx >= 4:
         n += sum(1 for t in range(t0, t0 + steps) if (t + 1) % c.stats_every == 0)

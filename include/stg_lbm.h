@@ -301,7 +301,7 @@ int stg_lbm_step_probed(stg_lbm *h, int64_t n, float *u_host);
 /* Autotuner: time every candidate tile on this lattice (`trial_passes` >= 1
  * plain step passes each, CUDA events on the handle's stream, after one
  * warm-up pass; tiles that stand for the same launches once), keep the fastest,
- * or the default tile unless another is faster by more than 1 %, and store it in
+ * or the default tile unless another is faster by more than 0.5 %, and store it in
  * *chosen (may be NULL).
  * The trial passes recompute the next state from the current one without
  * advancing the step counter, the inlet filter or the statistics, so tuning

@@ -1537,7 +1537,7 @@ int tile_inner_run(stg_lbm *h, const stg_tile &tile)
 
 bool better_tile(int c, float ms, float best_ms, float own_ms)
 {
-    return c == 0 || (ms < best_ms && ms < 0.99f * own_ms);
+    return c == 0 || (ms < best_ms && ms < 0.995f * own_ms);
 }
 
 }  // namespace host

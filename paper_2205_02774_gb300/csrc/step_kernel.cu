@@ -64,10 +64,12 @@ static bool ragged_fp32(const StepArgs &a)
     return a.storage == 0 && !lean(a) && !row_lanes(a) && a.nx % 64 != 0 && a.nx % 64 <= 48;
 }
 
-// FP32 lattices with fewer than 4 cells per resident lane (32 warps per SM): one
-// cell per lane halves the serial work of a warp (64x32x32 5.3 against 6.2 us per
-// step, 144x24x36 7.0 against 8.1, 240x40x60 15.4 against 18.2, 241x41x61 16.9
-// against 19.3; 325x55x81, just above, 44.1 against 42.3).
+// FP32 lattices with fewer than 4 cells per resident lane (32 warps per SM, 622592
+// cells): one cell per lane halves the serial work of a warp (us per step, one cell
+// per lane and pairs, each with the better number of launches: 96x16x24 3.7 and 5.2,
+// 144x24x36 6.0 and 7.4, 240x40x60 15.0 and 17.8).  The line is on the safe side: one
+// cell per lane in two launches stays ahead to about 2 million cells (252x42x63 17.4
+// and 22.0, 324x54x81 38.9 and 42.8, 360x60x90 49.6 and 51.3).
 static bool small_row(const StepArgs &a)
 {
     return std::max<long long>(a.P, a.in_flight) < 4LL * 152 * 32 * 32;
@@ -118,10 +120,15 @@ int lane_cells(const StepArgs &a)
 // that advance together.  While the GPU's warps (16 per SM with the registers of
 // the kernel for any row) have only a few each, a pass is bound by launches and by
 // the latency of one plane, and one launch of all rows saves the branch of the wall
-// rows: 64x32x32 5.6 against 8.2 us per step, 240x40x60 FP32 (3.9 items per warp)
-// 18.0 against 21.0.  Above that the inner rows' own kernel, with more warps per SM,
-// is the faster one: 384x64x96 FP32 (15) 57 against 73 us, 324x54x81 FP16 (5.4) 30.6
-// against 35.0, 240x40x60 FP16 (2.0) 13.2 against 14.4.
+// rows; above that the inner rows' own kernel, with more warps per SM, is the faster
+// one.  us per step, one launch and two, by items per warp:
+//   FP32, one cell per lane: 0.5 3.7 and 5.7, 1.8 6.0 and 6.9, 2.9 8.0 and 7.7, 3.8
+//     9.6 and 8.7, 5.6 12.7 and 11.5, 7.9 18.7 and 15.0 (the line at 4 gives away up to
+//     a tenth between 2.5 and 4)
+//   binary16 quads (the line at 1.5): 240x40x60 (2.0) 14.4 and 13.2; 324x54x81 (5.4)
+//     35.0 and 30.6
+//   FP32 pairs (from 622592 cells, 4 items per warp, on: always two): 300x50x75 39.4
+//     and 38.2, 324x54x81 51.6 and 42.8, 384x64x96 73 and 57
 static long long items_of(const StepArgs &a, int cpl)
 {
     const long long own = (long long)((a.nx + BX * cpl - 1) / (BX * cpl)) * a.ny * a.nz;

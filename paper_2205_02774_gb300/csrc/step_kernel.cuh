@@ -1,7 +1,7 @@
 // Fused LES-LBM time step for one channel lattice (Algorithm 1, step 12, with
 // steps 9-11 for the inlet nodes and the outlet rebuild folded in): the device
-// templates, instantiated per storage and collision by step_f32_reg.cu,
-// step_f32_bgk.cu, step_f16_reg.cu and step_f16_bgk.cu.
+// templates, instantiated per storage, collision and lane layout by the units
+// step_<f32|f16|f16sr>_<reg|bgk>[_quad|_row].cu.
 //
 // One pass per cell: pull the 19 post-collision populations of the previous
 // step along -c_i (eq. lbe, left side) with half-way bounce-back at the y
@@ -17,8 +17,10 @@
 // lane two or four consecutive x cells and a warp an x chunk of one row over a
 // run of z planes: on plain steps as long as the lattice's size makes best
 // (run_planes), on sampling steps a function of the lattice alone, whose
-// per-(x, y) sums are added in order.  The odd-nx path (one cell per thread)
-// keeps a block per (x chunk, row) column.
+// per-(x, y) sums are added in order.  Odd rows and small FP32 lattices take the same
+// launches with lanes that own cells 32 apart (lbm_row.cuh); one cell per thread,
+// with a block per (x chunk, row) column, is left for lattices beyond 32-bit element
+// offsets and for large ones with odd binary16 rows of fewer than 32 cells.
 //
 // Streaming schemes (vector kernels, MODE):
 //  PULL      two lattices: read src[i] at x - c_i, write dst[i] at x;
@@ -300,7 +302,7 @@ __device__ __forceinline__ void step_column(const StepArgs &a, int bx, int y)
     if (do_check) mass_finish<BX * BZ>(a, sdr);
 }
 
-// Scalar interior columns: x chunks [il, ir), y = 1..ny-2 (odd nx or narrow lattices).
+// One cell per thread, interior columns: x chunks [il, ir), y = 1..ny-2.
 template <typename S, bool REG, bool FORCE, bool SP, bool SR>
 __global__ void __launch_bounds__(BX *BZ, 4) lbm_step_kernel(const StepArgs a)
 {
