@@ -100,3 +100,10 @@ def test_inlet_planes_in_a_batch_of_many():
         for ch in chs:
             ch.close()
     assert us["stg"] < 1.35 * us["periodic"]
+
+
+# rows that fill an eighth of a chunk count as what they hold: runs of 8 planes took 1.046
+# times as long as runs of 2
+def test_runs_of_narrow_binary16_rows():
+    kw = dict(nx=16, ny=256, nz=256, storage="fp16sr", streaming="aa")
+    assert _us(**kw) < 1.025 * _us(tile=(0, 16, 24), **kw)
