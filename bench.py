@@ -103,17 +103,20 @@ def _launches(c, t0, steps):
     return n
 
 
-def _launches_enqueued(c, t0, steps, batch=False):
+def _launches_enqueued(c, t0, steps, batch=False, probed=False):
     """Kernels the steps t0 .. t0+steps-1 really enqueue, as the library cuts them:
     blocks (from a step index divisible by the sampling period; in a batch from any)
     carry one inlet launch for the first 4 steps and one per 16 more (in a batch one
-    per 16), single steps one each; a pass is one launch on lattices that do not fill the GPU, else two."""
+    per 16), single steps one each; a pass is one launch on lattices that do not fill the GPU, else two.
+    probed: one more per step, and one for the place of the series if there are blocks
+    (the second call of a series of this length at the latest has them)."""
     k = max(c.stats_every, 1)
     period = k * -(-16 // k) if c.stats_every > 0 else 16
     if batch:
         period = k * (1 if k % 2 == 0 else 2) * -(-16 // (k * (1 if k % 2 == 0 else 2)))
     narrow = c.storage != "fp32" and c.nx < 32 and c.ny * c.nz >= 152 * 20 * (19 if c.storage == "fp16sr" else 24)
-    row = c.streaming == "pull" and (c.nx % 2 != 0 or c.nx < 4) and not narrow
+    big = c.streaming == "pull" and 19 * c.cells >= 2 ** 32
+    row = c.streaming == "pull" and (c.nx % 2 != 0 or c.nx < 4) and not narrow and not big
     small = c.streaming == "pull" and c.storage == "fp32" and c.cells < 4 * 152 * 32 * 32 and not batch
     bgk_pairs = c.collision == "bgk" and not row and (
         c.streaming == "aa" or (c.nx <= (720 if c.storage == "fp16sr" else 580) if c.bc_x == "stg" else
@@ -121,19 +124,23 @@ def _launches_enqueued(c, t0, steps, batch=False):
     quads = row or (c.nx % 4 == 0 and c.nx >= 8 and not bgk_pairs)
     cpl = (4 if quads else 2) if c.storage != "fp32" else (1 if small else 2)
     items = -(-c.nx // (32 * cpl)) * c.ny * c.nz
-    scalar = c.streaming == "pull" and (c.nx % 2 != 0 or c.nx < 4) and not row  # a pass of its own kernels, no reduction
-    passes = 1 if not scalar and (c.ny < 3 or (not batch and 2 * items < 152 * 16 * (3 if cpl == 4 else 8))) else 2
+    # one cell per thread: the edge kernel and, in rows of more than 64 cells, the interior one; no reduction
+    scalar = big or (c.streaming == "pull" and (c.nx % 2 != 0 or c.nx < 4) and not row)
+    passes = 1 if c.ny < 3 or (c.nx <= 64 if scalar else
+                               not batch and 2 * items < 152 * 16 * (3 if cpl == 4 else 8)) else 2
     inlet = c.bc_x == "stg"
     n, t, left = 0, t0, steps
+    blocks = False
     while left > 0:
         whole = period <= 256 and left >= period and (batch or t % k == 0)
+        blocks |= whole
         b = period if whole else 1
         n += b * passes + (inlet and (-(-b // 16) if batch and whole else 1 + max(0, -(-(b - 4) // 16))))
         t += b
         left -= b
     if c.stats_every > 0 and not scalar:
         n += (t0 + steps) // c.stats_every - t0 // c.stats_every
-    return n
+    return n + (steps + blocks if probed else 0)
 
 
 class ClockSampler:
@@ -459,7 +466,9 @@ def run_ours(args):
                    "parallelism": f"replicas x{ws}"},
         "roofline": roofline(BYTES_PER_CELL[c.storage], c.cells, m["ms_step"], m["ms_inlet"], traffic, STEP_KERNEL),
         "hbm_frac_of_step": m["hbm_frac_of_step"],
-        "gpu_launches": _launches_enqueued(c, args.warmup, args.steps) + (args.steps if args.probes > 0 else 0),
+        # (with probes an untimed series comes between)
+        "gpu_launches": _launches_enqueued(c, args.warmup + (args.steps if args.probes > 0 else 0), args.steps,
+                                           probed=args.probes > 0),
         "clocks": m["clocks"],
     }
     line["e2e"] = end_to_end(c, args.steps)
