@@ -5,15 +5,17 @@
 // x neighbours are the same runs one element to the side (no shuffle, no halo
 // case).  What keeps the bytes in flight that an aligned vector keeps is CPL
 // independent loads per population (FP32 2, binary16 4, whose pairs of cells go
-// through the packed collision).  One cell per thread in whole-column blocks, kept
-// for lattices beyond 32-bit element offsets only, and this loop, us per step:
+// through the packed collision).  One cell per thread in whole-column blocks, the
+// form before, and this loop, us per step:
 //                        385x65x97     767x127x191
 //   FP32                 93 -> 66      733 -> 452    (55 and 423 at the copy rate)
-//   binary16             70 -> 54      464 -> 323    (28 and 211)
-//   stochastic rounding  73 -> 69      484 -> 385
-//   the same, BGK        74 -> 72      483 -> 400
+//   binary16             70 -> 54      464 -> 301    (28 and 211)
+//   stochastic rounding  73 -> 69      484 -> 379
+//   the same, BGK        74 -> 71      483 -> 405
 // What is left is the odd alignment (a run of 32 lanes touches one sector more than
-// it fills) and, for binary16, issue: 2-byte accesses and a random word per cell.
+// it fills: FP32 4.5 for 4, binary16 2.7 for 2) and, for binary16, instructions: 2-byte
+// accesses and a random word per cell, 15.3 per cell and warp against 7.9 with quads.
+// (Rows of fewer than 32 cells, large binary16 lattices: one cell per thread, narrow_rows().)
 #pragma once
 
 #include <cuda_fp16.h>
