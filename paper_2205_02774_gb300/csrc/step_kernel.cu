@@ -140,6 +140,13 @@ bool one_launch(const StepArgs &a, int cpl)
     return a.ny < 3 || items_of(a, cpl) * 2 < 152LL * 16 * (cpl == 4 ? 3 : 8);
 }
 
+// Runs of 4 planes in the wall rows, else 1: where the inner rows take long enough to
+// hide the latency of a walk of 4 planes, which FP32 pairs do from 7 items per resident
+// warp on (us per step with 1, 2, 4: 264x44x66 20.3, 20.8, 28.4; 300x50x75 30.5, 30.6,
+// 36.7; 360x60x90 48.7, 48.9, 49.3; 384x64x96 57.3, 57.1, 56.4; 768x128x192 417, 416,
+// 415).  FP32 lanes 32 cells apart are the same either way (240x40x60 13.6, 13.6, 13.6;
+// 385x64x96 64.1, 63.9, 64.2).  Binary16 1 (768x128x192 226, 228, 230, 236 with 24), but
+// 4 among the members of a batch.
 // A run of several planes costs one block start instead of several, but a pass
 // ends with its last runs, and a short pass needs every warp from the start: so
 // runs grow with the number of items per resident warp, up to what the form takes:
@@ -154,16 +161,21 @@ bool one_launch(const StepArgs &a, int cpl)
 //  binary16 lanes 32 cells apart 2 (767x127x191: 302, 308, 321 us with 2, 4, 8, 63x300x300
 //    174, 179, 184).
 // The wall rows, beside the inner launch, are spread over as many warps as their
-// latency needs: binary16 1, FP32 4 (768x128x192: FP16 226, 228, 230 us with
-// 1, 2, 4, and 236 with 24; FP32 420, 420, 418), and 4 among the members of a batch.
+// latency needs (long_walls).
 // A tile that was set sets the runs instead.
+static bool long_walls(const StepArgs &a, int cpl)
+{
+    if (a.storage != 0) return a.in_flight > a.P;
+    return cpl == 1 || row_lanes(a) || items_of(a, cpl) >= 7 * 152 * 32;
+}
+
 int run_planes(const StepArgs &a, int cpl, bool walls)
 {
     const int least = (a.nz + 65534) / 65535;  // a launch holds 65535 runs
     const int tile = walls ? a.tile_wall_zc : a.tile_zc;
     if (tile > 0) return std::max(least, std::min(tile, a.nz));
     const bool fp32 = a.storage == 0;
-    if (walls) return std::max(least, std::min(a.nz, fp32 || a.in_flight > a.P ? 4 : 1));
+    if (walls) return std::max(least, std::min(a.nz, long_walls(a, cpl) ? 4 : 1));
     int most = ragged_fp32(a) ? 4 : 2;
     if (!fp32 && !row_lanes(a)) most = cpl == 4 ? 8 : (lean(a) ? 2 : 4);
     // (binary16: by the cells that the items hold, for rows that fill a fraction of one)

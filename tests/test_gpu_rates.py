@@ -107,3 +107,10 @@ def test_inlet_planes_in_a_batch_of_many():
 def test_runs_of_narrow_binary16_rows():
     kw = dict(nx=16, ny=256, nz=256, storage="fp16sr", streaming="aa")
     assert _us(**kw) < 1.025 * _us(tile=(0, 16, 24), **kw)
+
+
+# FP32 pairs on a few hundred thousand to two million cells: wall rows in runs of 4 planes
+# outlasted the inner rows (1.20 times the time of runs of 1 or 2)
+def test_wall_rows_of_small_fp32_lattices():
+    kw = dict(nx=300, ny=50, nz=75)
+    assert _us(**kw) < 0.93 * _us(tile=(1, 8, 32), **kw)
