@@ -127,7 +127,7 @@ def _launches_enqueued(c, t0, steps, batch=False, probed=False):
     # one cell per thread: the edge kernel and, in rows of more than 64 cells, the interior one; no reduction
     scalar = big or (c.streaming == "pull" and (c.nx % 2 != 0 or c.nx < 4) and not row)
     passes = 1 if c.ny < 3 or (c.nx <= 64 if scalar else
-                               not batch and 2 * items < 152 * 16 * (3 if cpl == 4 else 8)) else 2
+                               not batch and 2 * items < 152 * 16 * (3 if c.storage != "fp32" else 8)) else 2
     inlet = c.bc_x == "stg"
     n, t, left = 0, t0, steps
     blocks = False

@@ -127,6 +127,10 @@ int lane_cells(const StepArgs &a)
 //     a tenth between 2.5 and 4)
 //   binary16 quads (the line at 1.5): 240x40x60 (2.0) 14.4 and 13.2; 324x54x81 (5.4)
 //     35.0 and 30.6
+//   binary16 pairs (the line at 1.5): 142x24x36 (1.1) 6.8 and 5.2, one step alone 10.7
+//     and 11.0; 182x30x45 (1.7) 7.5 and 6.0; 230x38x57 (3.6) 11.6 and 9.2; BGK with
+//     stochastic rounding 240x40x60 (4.0) 14.3 and 12.1; in place 206x34x51 (2.9) 10.7
+//     and 10.3
 //   FP32 pairs (from 622592 cells, 4 items per warp, on: always two): 300x50x75 39.4
 //     and 38.2, 324x54x81 51.6 and 42.8, 384x64x96 73 and 57
 static long long items_of(const StepArgs &a, int cpl)
@@ -137,7 +141,7 @@ static long long items_of(const StepArgs &a, int cpl)
 
 bool one_launch(const StepArgs &a, int cpl)
 {
-    return a.ny < 3 || items_of(a, cpl) * 2 < 152LL * 16 * (cpl == 4 ? 3 : 8);
+    return a.ny < 3 || items_of(a, cpl) * 2 < 152LL * 16 * (a.storage != 0 ? 3 : 8);
 }
 
 // Runs of 4 planes in the wall rows, else 1: where the inner rows take long enough to

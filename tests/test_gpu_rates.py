@@ -114,3 +114,10 @@ def test_runs_of_narrow_binary16_rows():
 def test_wall_rows_of_small_fp32_lattices():
     kw = dict(nx=300, ny=50, nz=75)
     assert _us(**kw) < 0.93 * _us(tile=(1, 8, 32), **kw)
+
+
+# binary16 pairs had FP32's line for one launch of all rows: 206x34x51 took longer than the
+# same channel with 72 planes, which had two launches (1.05 times, 0.86 with two of its own)
+def test_two_launches_of_binary16_pairs():
+    kw = dict(nx=206, ny=34, storage="fp16s")
+    assert _us(nz=51, **kw) < 0.97 * _us(nz=72, **kw)
