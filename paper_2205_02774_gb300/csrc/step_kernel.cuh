@@ -752,8 +752,11 @@ __device__ __forceinline__ float vec_loop(const StepArgs &a, float (*sacc)[9][BX
                 }
             }
         }
-        // (in place, even steps: the quads go through shuffles of the whole warp)
-        constexpr bool SHIFT4 = MODE == AA_SHIFT && CPL == 4;
+        // (in place, even steps, inlet and outlet in x: the quads go through shuffles of
+        // the whole warp, 768x128x192 round to nearest 253 us per step against 259 cell by
+        // cell.  In a periodic box the loads take the shuffles already and the stores by
+        // pieces are faster: stochastic rounding 261 against 271, 1536x128x192 503 and 531)
+        constexpr bool SHIFT4 = MODE == AA_SHIFT && CPL == 4 && H16;
         if (SHIFT4 || active) {
 #pragma unroll
             for (int i = 0; i < Q; ++i) {
@@ -788,8 +791,8 @@ __device__ __forceinline__ float vec_loop(const StepArgs &a, float (*sacc)[9][BX
                     // the target quad x .. x + 3 from the lane's own cells and one of the
                     // lane beside it; where that lane is in another warp (or the row ends)
                     // the own cells alone, cells 1 and 2 as one aligned pair, and the cell
-                    // that leaves the warp's quads by itself: outside at the open ends (the
-                    // own slot), wrapped when x is periodic
+                    // that leaves the warp's quads by itself (outside at the open ends: the
+                    // own slot)
                     const unsigned beside = cx < 0 ? __shfl_down_sync(0xffffffffu, v[i].x, 1)
                                                    : __shfl_up_sync(0xffffffffu, v[i].y, 1);
                     if (!active) continue;
@@ -800,25 +803,31 @@ __device__ __forceinline__ float vec_loop(const StepArgs &a, float (*sacc)[9][BX
                             V::st_mid(tx, v[i]);
                             V::st1(tx - 1, v[i], 3);
                         }
-                        if (lane == 0) V::st1(x > 0 ? tx - 1 : (inout ? own_slot(i) : tx + (nx - 1)), v[i], 0);
+                        if (lane == 0) V::st1(x > 0 ? tx - 1 : own_slot(i), v[i], 0);
                     } else {
                         if (lane > 0) V::st(tx, make_uint2(__byte_perm(beside, v[i].x, 0x5432), mid));
                         else {
                             V::st1(tx + 1, v[i], 0);
                             V::st_mid(tx + 2, v[i]);
                         }
-                        if (side_r) V::st1(x + CPL < nx ? tx + 1 : (inout ? own_slot(i) : tx - (x + CPL - 1)), v[i], CPL - 1);
+                        if (side_r) V::st1(x + CPL < nx ? tx + 1 : own_slot(i), v[i], CPL - 1);
                     }
                 } else if (cx < 0) {
-                    // cell x + 1 -> x, cell x -> x - 1; the row's first cell (lanes with
-                    // x = 0 only): outside at the inlet (the own slot), wraps to
-                    // x = nx - 1 when x is periodic
-                    V::st1(tx - 1, v[i], 1);
+                    // cells x + 1 .. -> x .. (quads: cells 1, 2 as one aligned pair), cell
+                    // x -> x - 1; the row's first cell (lanes with x = 0 only): outside at
+                    // the inlet (the own slot), wraps to x = nx - 1 when x is periodic
+                    if constexpr (CPL == 4) {
+                        V::st_mid(tx, v[i]);
+                        V::st1(tx - 1, v[i], 3);
+                    } else {
+                        V::st1(tx - 1, v[i], 1);
+                    }
                     V::st1(x > 0 ? tx - 1 : (inout ? own_slot(i) : tx + (nx - 1)), v[i], 0);
                 } else {
-                    // cell x -> x + 1, cell x + 1 -> x + 2; the row's last cell (lanes with
-                    // x = nx - 2 only): outside at the outlet, wraps to 0
+                    // cells x .. -> x + 1 .., the last one to x + CPL; the row's last cell (lanes
+                    // with x = nx - CPL only): outside at the outlet, wraps to 0
                     V::st1(tx + 1, v[i], 0);
+                    if constexpr (CPL == 4) V::st_mid(tx + 2, v[i]);
                     V::st1(x + CPL < nx ? tx + 1 : (inout ? own_slot(i) : tx - (x + CPL - 1)), v[i], CPL - 1);
                 }
             }

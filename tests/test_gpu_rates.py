@@ -121,3 +121,10 @@ def test_wall_rows_of_small_fp32_lattices():
 def test_two_launches_of_binary16_pairs():
     kw = dict(nx=206, ny=34, storage="fp16s")
     assert _us(nz=51, **kw) < 0.97 * _us(nz=72, **kw)
+
+
+# in place, periodic x: stores through shuffles beside the loads' own took 1.06 times as long
+# (1.10 times the time of the channel, 1.03 without)
+def test_in_place_stores_of_periodic_rows():
+    kw = dict(nx=1536, ny=128, nz=192, storage="fp16sr", streaming="aa")
+    assert _us(bc_x="periodic", **kw) < 1.065 * _us(**kw)
