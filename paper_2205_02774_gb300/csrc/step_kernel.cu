@@ -159,7 +159,9 @@ bool one_launch(const StepArgs &a, int cpl)
 //    a ragged last chunk 4 (200^3 228, 218, 216 us with 2, 4, 8; full rows stay at 2:
 //    320x160x160 193, 193, 197, 256x128x128 97.6, 98.4, 106.7);
 //  binary16 quads 8 (1536x256x384: 1.82, 1.76, 1.72, 1.72 ms with 1, 2, 4, 8;
-//    384x64x96: 2; in place 16x256x256, an eighth of a chunk per row, 132, 132, 132, 138 us);
+//    384x64x96: 2), in place 4 (us with 2, 4, 8: round to nearest 320x128x200 140.9, 140.7,
+//    146.1, 512x128x128 121.7, 122.8, 128.5, 768x128x192 246, 248, 253, stochastic rounding
+//    276, 273, 276, 1536x128x192 496, 489, 490);
 //  binary16 pairs (128 B) 2, with BGK or a force 4 (250x125x125 61.8, 64.9, 69.1 us with
 //    2, 4, 8, 770x128x192 282, 293, 305; BGK 200^3 142, 136, 142);
 //  binary16 lanes 32 cells apart 2 (767x127x191: 302, 308, 321 us with 2, 4, 8, 63x300x300
@@ -181,7 +183,7 @@ int run_planes(const StepArgs &a, int cpl, bool walls)
     const bool fp32 = a.storage == 0;
     if (walls) return std::max(least, std::min(a.nz, long_walls(a, cpl) ? 4 : 1));
     int most = ragged_fp32(a) ? 4 : 2;
-    if (!fp32 && !row_lanes(a)) most = cpl == 4 ? 8 : (lean(a) ? 2 : 4);
+    if (!fp32 && !row_lanes(a)) most = cpl == 4 ? (a.aa ? 4 : 8) : (lean(a) ? 2 : 4);
     // (binary16: by the cells that the items hold, for rows that fill a fraction of one)
     const long long items = fp32 ? items_of(a, cpl) : std::max<long long>(a.P, a.in_flight) / (BX * cpl);
     const long long per_warp = items / (152 * (fp32 ? 32 : 20));

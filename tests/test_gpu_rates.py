@@ -128,3 +128,9 @@ def test_two_launches_of_binary16_pairs():
 def test_in_place_stores_of_periodic_rows():
     kw = dict(nx=1536, ny=128, nz=192, storage="fp16sr", streaming="aa")
     assert _us(bc_x="periodic", **kw) < 1.065 * _us(**kw)
+
+
+# in place, runs of 8 planes (1.05 times the time of runs of 4, runs of 9 no better than 8)
+def test_runs_in_place():
+    kw = dict(nx=512, ny=128, nz=128, storage="fp16s", streaming="aa")
+    assert _us(**kw) < 0.985 * _us(tile=(1, 9, 24), **kw)
